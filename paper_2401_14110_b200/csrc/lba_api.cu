@@ -75,7 +75,7 @@ struct Plan {
   float pk_a, pk_b, nrm_scale, inv_top;
   float clamp_lim, slab_factor, fold_factor;
   int pq, rne_packed;
-  float rne_k_acc, rne_k_prod;
+  float acc_k1, acc_k2, prod_k1, prod_k2;
   QConst qp, qa;
   int chunk_slabs, chunk;
   int kp, ka, sx;   // product carrier = value * 2^kp, accumulator carrier = value * 2^ka, A operand = x * 2^sx
@@ -275,8 +275,8 @@ int make_plan(const lba_fmt* pf, const lba_fmt* af, int order, int chunk, int64_
     pl->fold_factor = 1.0f;
   }
 
-  // ---- packed kernel: what Q_prod does beyond the flush.  Nearest-even rounds on the FP32 pipe by adding and
-  // subtracting 1.5 * 2^(23-M) * 2^e, which needs that much exponent headroom above the largest carried magnitude.
+  // ---- packed kernel: what Q_prod does beyond the flush.  Nearest-even rounds on the FP32 pipe through
+  // the value times 2^(23-M), which needs that much exponent headroom above the largest carried magnitude.
   // Its sum is one FMA rounded to nearest, which equals one rounding of the exact sum only under these conditions:
   //   * the quantised product has no more significant bits than the accumulator (else a product that is the larger
   //     operand can sit exactly on a tie of the accumulator's grid, which a far smaller sum must break);
@@ -287,8 +287,19 @@ int make_plan(const lba_fmt* pf, const lba_fmt* af, int order, int chunk, int64_
   //     away next to -R_UF_acc and leave R_UF_acc itself standing).
   // Everything else in nearest-even mode runs in the generic kernel (round-to-odd, then the cut).
   pl->pq = p_sat ? PQ_MASK_SAT : (p_round ? PQ_MASK : PQ_NONE);
-  pl->rne_k_acc = (float)std::ldexp(1.0, 23 - af->man_bits);
-  pl->rne_k_prod = (float)std::ldexp(1.0, 23 - pf->man_bits);
+  const auto pow2 = [](int e) { return (float)std::ldexp(1.0, e); };
+  pl->acc_k1 = 1.0f - pow2(23 - af->man_bits);
+  pl->acc_k2 = pow2(23 - af->man_bits);
+  if (nearest) {
+    pl->prod_k1 = 1.0f - pow2(23 - pf->man_bits);
+    pl->prod_k2 = pow2(23 - pf->man_bits);
+  } else if (p_round) {
+    pl->prod_k1 = 1.0f + pow2(23 - pf->man_bits);
+    pl->prod_k2 = -pow2(23 - pf->man_bits);
+  } else {  // nothing to cut: the identity
+    pl->prod_k1 = 1.0f;
+    pl->prod_k2 = 0.0f;
+  }
   pl->rne_packed = 0;
   if (pl->qm == QM_RNE_FULL) {
     const int top_acc = (a_sat ? a_emax + 1 : (int)std::ceil(std::log2(max_sum)) + 1) + ka;
@@ -296,8 +307,11 @@ int make_plan(const lba_fmt* pf, const lba_fmt* af, int order, int chunk, int64_
     // significant bits of a quantised product: the exact product's, cut to M_prod + 1; a saturated product is R_OF_prod,
     // which has all M_prod + 1
     const int prod_bits = (p_sat || pf->man_bits + 1 < in.product_bits) ? pf->man_bits + 1 : in.product_bits;
-    pl->rne_packed = (top_acc + 25 - af->man_bits <= 127) && (top_prod + 25 - pf->man_bits <= 127) && af->man_bits <= 10 &&
+    const bool ok = (top_acc + 25 - af->man_bits <= 127) && (top_prod + 25 - pf->man_bits <= 127) && af->man_bits <= 10 &&
                      prod_bits <= af->man_bits + 1 && ka - kp >= -12 && ka - kp <= 60;
+    // M = 7 in chunks of 16: round through bfloat16 (8.6 against 7.7 TMAC/s on 4096 x 4096 x 2048).  Sequentially the
+    // conversion sits in every link of the chain and the FP32-pipe cut is faster (7.9 against 7.4).
+    pl->rne_packed = !ok ? 0 : (af->man_bits == 7 && order == LBA_ORDER_CHUNKED && chunk == BK && K > BK) ? 2 : 1;
   }
 
   // ---- fused product and sum: Q_prod must be the identity on every reachable product (no cut, no saturation, no
@@ -417,8 +431,8 @@ void apply_plan(Problem* p, const Plan& pl) {
   p->pq = pl.pq;
   p->rne_packed = pl.rne_packed;
   p->in_m4e3 = pl.in_m4e3;
-  p->rne_k_acc = pl.rne_k_acc;
-  p->rne_k_prod = pl.rne_k_prod;
+  p->acc_k1 = pl.acc_k1; p->acc_k2 = pl.acc_k2;
+  p->prod_k1 = pl.prod_k1; p->prod_k2 = pl.prod_k2;
   p->fx_shift0 = pl.fx_shift0;
   p->fx_lo_p = pl.fx_lo_p; p->fx_hi_p = pl.fx_hi_p; p->fx_sh_p = pl.fx_sh_p; p->fx_hold_p = pl.fx_hold_p;
   p->fx_lo_a = pl.fx_lo_a; p->fx_hi_a = pl.fx_hi_a; p->fx_sh_a = pl.fx_sh_a; p->fx_wrap_a = pl.fx_wrap_a;

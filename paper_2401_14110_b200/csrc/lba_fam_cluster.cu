@@ -9,7 +9,7 @@ constexpr int BM = 64, BN = 64, TM = 4, TN = 8, CL = 2;
 
 template <int PQ, int LD, bool H16>
 cudaError_t launch(const Problem& p, cudaStream_t stream) {
-  auto kernel = lba_contract_packed_kernel<BM, BN, TM, TN, PQ, false, ORD_CHUNK16, LD, 0, CL, H16>;
+  auto kernel = lba_contract_packed_kernel<BM, BN, TM, TN, PQ, 0, ORD_CHUNK16, LD, 0, CL, H16>;
   constexpr size_t smem = packed_cluster_smem_bytes<BM, BN, TM, TN>();
   static_assert(smem <= 48 * 1024, "no opt-in needed");
   cudaLaunchConfig_t cfg = {};

@@ -10,7 +10,7 @@ constexpr int BM = 64, BN = 64, TM = 4, TN = 8;
 template <int PQ, int ORD, int LD>
 cudaError_t launch(const Problem& p, cudaStream_t stream) {
   const dim3 grid((unsigned)((p.M + BM - 1) / BM), (unsigned)((p.N + BN - 1) / BN), 1);
-  auto kernel = lba_contract_packed_kernel<BM, BN, TM, TN, PQ, false, ORD, LD, 1>;
+  auto kernel = lba_contract_packed_kernel<BM, BN, TM, TN, PQ, 0, ORD, LD, 1>;
   constexpr size_t smem = packed_ste_smem_bytes<BM, BN, TM, TN>();
   static_assert(smem > 48 * 1024, "opt-in below assumes the large shared-memory carve-out is needed");
   static bool done[64] = {};  // opt in to large dynamic shared memory, once per device and kernel

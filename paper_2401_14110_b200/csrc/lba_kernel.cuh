@@ -73,9 +73,10 @@ struct Problem {
   float nrm_scale;     // 2^-(e_max_acc + 1), or 0 when the accumulator cannot saturate
   float inv_top;       // accumulator carrier -> fraction of 2^(e_max_acc + 1)
   int pq;              // PackedProd: what Q_prod does beyond the flush
-  int rne_packed;      // nearest-even: 1 if the packed kernel's conditions hold (see the host plan)
+  int rne_packed;      // nearest-even: not 0 if the packed kernel's conditions hold (see the host plan), the kernel's RNE argument
   int in_m4e3;         // operands are bytes of the paper's M4E3 W/A format (Sec. 3.1) instead of OCP E4M3
-  float rne_k_acc, rne_k_prod;  // 2^(23 - M) for the accumulator and the product format
+  float acc_k1, acc_k2;    // nearest-even cut of a sum: v k2 + rn(v k1) (see rne2_fp)
+  float prod_k1, prod_k2;  // the same for a product; under floor rounding v k2 + rz(v k1) (see floor2_fp)
   // clamp elision: a slab or fold runs without the magnitude clamp while (bound + growth) * factor < clamp_lim.
   // Floor never raises a magnitude: factors 1, limit just under 1 (of 2^(e_max+1)).  Nearest-even can raise one by
   // half a grid step per rounding: slab_factor bounds sixteen such steps (and the product's own rounding),
@@ -236,21 +237,29 @@ __device__ __forceinline__ u64 fma2_rn_ftz(u64 a, u64 b, u64 c) {
   asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
   return d;
 }
-// Nearest-even cut of a pair of binary32 values to M mantissa bits on the FP32 pipe.  With e the value's own
-// exponent, K = 1.5 * 2^(23-M) * 2^e (same sign) moves the value into a binade whose unit in the last place is the
-// target grid step, so the addition v + K itself rounds to nearest-even on that grid (K/ulp is even, so ties carry
-// over); subtracting K again is exact.  k0 = +-1.5 * 2^e is one logic operation per value (sign and exponent
-// kept, mantissa set to 1.5), and both steps are one packed FMA each: r = k0 * ks + v, result = k0 * (-ks) + r
-// with ks = 2^(23-M).  A zero stays zero (k0 is then a subnormal; r = k0 * ks is cancelled exactly).  Needs M <= 21
-// and exponent headroom for K, which the host checks.  `v` must be exact (or the correctly rounded binary32 image
-// of a sum whose rounding cannot decide an M-bit tie; see the host's conditions for the packed nearest-even path).
-__device__ __forceinline__ u64 rne2_fp(u64 v, u64 ks, u64 nks) {
-  uint32_t lo, hi;
-  asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "l"(v));
-  u64 k0;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(k0) : "r"((lo & 0xFF800000u) | 0x00400000u), "r"((hi & 0xFF800000u) | 0x00400000u));
-  const u64 r = fma2_rn(k0, ks, v);
-  return fma2_rn(k0, nks, r);
+__device__ __forceinline__ u64 mul2_rn(u64 a, u64 b) {  // subnormal operands and results honoured
+  u64 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+// Nearest-even cut of a pair of binary32 values to M <= 10 mantissa bits, two packed FP32 instructions and no logic
+// operation.  With s = 23 - M, k1 = 1 - 2^s, k2 = 2^s: r = rn(v * k1) = -(2^s v - v), whose unit in the last place is the
+// target grid step of v; 2^s v itself lies on that grid (as an even multiple whenever v is a tie), so the
+// multiplication rounds v to nearest-even, and v * k2 + r takes 2^s v off again exactly.  Where v k1 falls into the
+// binade below (v within 2^-s of a power of two, M <= 10) the finer grid rounds to the same power of two; 1 + 2^s in
+// place of 2^s - 1 would cross into the binade above and be wrong there.  Measured in the bare instruction mix: 4.1
+// clocks per warp-MAC against 6.0 for adding and subtracting 1.5 * 2^(s+e) (two LOP3 and two FFMA2).  `v` must be exact
+// (or the correctly rounded binary32 image of a sum whose rounding cannot decide an M-bit tie; see the host's conditions
+// for the packed nearest-even path).
+__device__ __forceinline__ u64 rne2_fp(u64 v, u64 k1, u64 k2) { return fma2_rn(v, k2, mul2_rn(v, k1)); }
+// The same for M = 7: a bfloat16 has exactly those bits, so the conversion rounds both values in one instruction and
+// two logic instructions widen them again (3.6 clocks per warp-MAC in the bare mix).
+__device__ __forceinline__ u64 rne2_bf16(float lo, float hi) {
+  uint32_t h;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(h) : "f"(hi), "f"(lo));
+  u64 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(h << 16), "r"(h & 0xFFFF0000u));
+  return d;
 }
 __device__ __forceinline__ u64 mul2_rn_ftz(u64 a, u64 b) {
   u64 d;
@@ -267,14 +276,12 @@ __device__ __forceinline__ u64 mul2_rz_ftz(u64 a, u64 b) {
   asm("mul.rz.ftz.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
+// Floor cut of a pair of products to M bits on the FP32 pipe: k1 = 1 + 2^s, k2 = -2^s, r = rz(v * k1) = 2^s v + v cut to v's
+// grid, minus 2^s v exactly.  Only for values of at most 10 significant bits (s > 10): v k1 must not reach the next binade.
+__device__ __forceinline__ u64 floor2_fp(u64 v, u64 k1, u64 k2) { return fma2_rn(v, k2, mul2_rz_ftz(v, k1)); }
 __device__ __forceinline__ u64 add2_rz_ftz(u64 a, u64 b) {
   u64 d;
   asm("add.rz.ftz.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ u64 mul2_rn(u64 a, u64 b) {  // subnormal operands and results honoured
-  u64 d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
 
@@ -801,6 +808,10 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), TRACK == TRACK_MASK_DIF
 // B-row norms of the slab give one bound per CTA, and each thread carries an upper bound `u` of
 // its own |S| (as a fraction of 2^(e_max+1)), refreshed from the registers when it gets too loose.
 // A warp whose bound fails runs the same slab with the clamp.  Results are identical either way.
+// Under floor rounding with a product cut the logic pipe binds (four masks per pair and step).  Every second register pair of
+// a micro-tile row (j % 2 == FP_CUT) therefore cuts its product on the FP32 pipe: 7.8 against 7.1 TMAC/s on 4096^3 in chunk-16
+// order (every fourth pair 7.3), 8.1 against 7.8 sequentially.
+constexpr int FP_CUT = 1;
 constexpr int KUNROLL = 16;  // k-steps unrolled in the packed slab body (the whole slab: measured fastest)
 
 // two E4M3 bytes (low 16 bits of `pair`) -> their exact values, by the hardware converter
@@ -834,7 +845,7 @@ __device__ __forceinline__ u64 pack2u(uint32_t lo, uint32_t hi) {
 }
 
 // columns of tensor memory a CTA of the packed kernel allocates (0: second-level sums stay in registers)
-template <int BM, int BN, int TM, int TN, bool RNE, int ORD>
+template <int BM, int BN, int TM, int TN, int RNE, int ORD>
 __host__ __device__ constexpr int packed_tmem_cols() {
   constexpr int warps = (BM / TM) * (BN / TN) / 32;
   constexpr int cols = ((warps + 3) / 4) * TM * TN;
@@ -851,7 +862,7 @@ __host__ __device__ constexpr int packed_tmem_cols() {
 // exact product and the sum; the B operand then carries the accumulator's scaling.
 enum PackedProd { PQ_NONE = 0, PQ_MASK = 1, PQ_MASK_SAT = 2, PQ_FUSED = 3 };
 
-// RNE: nearest-even instead of floor (then PQ_MASK means "round the product to M_prod bits").  Nearest-even
+// RNE: nearest-even instead of floor, 1 = any M <= 10, 2 = M_acc = 7 (then PQ_MASK means "round the product to M_prod bits").  Nearest-even
 // can raise a magnitude by half a grid step per rounding, so the slab-level proof that the clamp is idle carries a
 // growth factor for the roundings of a slab and a limit that keeps every sum at or below R_OF.
 //
@@ -870,7 +881,7 @@ enum PackedProd { PQ_NONE = 0, PQ_MASK = 1, PQ_MASK_SAT = 2, PQ_FUSED = 3 };
 // one cluster barrier per pair of chunks.  H16: the chunk sums travel as bfloat16 pairs, which a value with at most 7
 // mantissa bits is exactly (half the traffic, 2 % faster); otherwise as binary32 words.
 // This doubles the CTAs of a small problem without splitting any sequential chain, and both CTAs do the same work.
-template <int BM, int BN, int TM, int TN, int PQ, bool RNE, int ORD, int LD, int STE = 0, int CL = 1, bool H16 = false>
+template <int BM, int BN, int TM, int TN, int PQ, int RNE, int ORD, int LD, int STE = 0, int CL = 1, bool H16 = false>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN),
                                   ((TM * TN == 64 && ORD != ORD_CHUNK_SLAB && !RNE) ||
                                    ((LD == LD_ANY || STE != 0) && !RNE && ORD != ORD_CHUNK_SLAB))
@@ -975,8 +986,16 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
   const float sat = p.qa.sat;
   const uint32_t pmask = p.qp.mask;
   const float psat = p.qp.sat;
-  const u64 ks_acc = pack2(p.rne_k_acc, p.rne_k_acc), nks_acc = pack2(-p.rne_k_acc, -p.rne_k_acc);
-  const u64 ks_prod = pack2(p.rne_k_prod, p.rne_k_prod), nks_prod = pack2(-p.rne_k_prod, -p.rne_k_prod);
+  const u64 acc_k1 = pack2(p.acc_k1, p.acc_k1), acc_k2 = pack2(p.acc_k2, p.acc_k2);
+  const u64 prod_k1 = pack2(p.prod_k1, p.prod_k1), prod_k2 = pack2(p.prod_k2, p.prod_k2);
+  auto rne_acc = [&](u64 v) -> u64 {
+    if (RNE == 2) {
+      float lo, hi;
+      unpack2(v, lo, hi);
+      return rne2_bf16(lo, hi);
+    }
+    return rne2_fp(v, acc_k1, acc_k2);
+  };
 
   // one slab of 16 k-steps; CLAMP selects whether the magnitude clamp of Eq. 2 is applied.  The clamped
   // variant is the rare one and stays a rolled loop.  In chunk-16 order the slab starts a chunk: its first
@@ -985,7 +1004,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
   auto slab_body = [&](int buf, auto clamp_tag) {
     constexpr bool CLAMP = decltype(clamp_tag)::value;
     constexpr bool REC = CLAMP && STE != 0;
-    constexpr int UNR = CLAMP ? 1 : (RNE ? 4 : KUNROLL);  // nearest-even: a four-step body keeps the loop in the instruction cache
+    constexpr int UNR = CLAMP ? 1 : (RNE ? 8 : KUNROLL);  // nearest-even: an eight-step body (2 % over four)
     if constexpr (REC) {
 #pragma unroll
       for (int i = 0; i < TM; ++i)
@@ -1009,13 +1028,16 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
       if constexpr (!RNE) {
         // floor: the products of micro-tile row i + 1 are formed while row i is added and masked, so that
         // multiplies (FP32 pipe) and masks (logic pipe) of independent outputs sit side by side in the stream
-        auto product = [&](u64 av, u64 bv) -> u64 {
+        auto product = [&](u64 av, u64 bv, int j) -> u64 {
           u64 pr = mul2_ftz(bv, av);
           if (PQ == PQ_MASK || PQ == PQ_MASK_SAT) {  // floor of Eq. 2 on the exact product, then its saturation
             float plo, phi;
+            if (j % 2 == FP_CUT) pr = floor2_fp(pr, prod_k1, prod_k2);
             unpack2(pr, plo, phi);
-            plo = and_bits(plo, pmask);
-            phi = and_bits(phi, pmask);
+            if (j % 2 != FP_CUT) {
+              plo = and_bits(plo, pmask);
+              phi = and_bits(phi, pmask);
+            }
             if (PQ == PQ_MASK_SAT) {
               plo = clamp_mag(plo, psat);
               phi = clamp_mag(phi, psat);
@@ -1048,12 +1070,12 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
         }
         u64 pr[PN], nx[PN];
 #pragma unroll
-        for (int j = 0; j < PN; ++j) pr[j] = product(a2[0], b2[j]);
+        for (int j = 0; j < PN; ++j) pr[j] = product(a2[0], b2[j], j);
 #pragma unroll
         for (int i = 0; i < TM; ++i) {
           if (i + 1 < TM) {
 #pragma unroll
-            for (int j = 0; j < PN; ++j) nx[j] = product(a2[i + 1], b2[j]);
+            for (int j = 0; j < PN; ++j) nx[j] = product(a2[i + 1], b2[j], j);
           }
 #pragma unroll
           for (int j = 0; j < PN; ++j) {
@@ -1095,7 +1117,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
           } else {
             u64 pr = mul2_ftz(b2[j], a2[i]);
             if (PQ == PQ_MASK || PQ == PQ_MASK_SAT) {  // nearest-even on the exact product, then its saturation
-              pr = rne2_fp(pr, ks_prod, nks_prod);
+              pr = rne2_fp(pr, prod_k1, prod_k2);
               if (PQ == PQ_MASK_SAT) {
                 float plo, phi;
                 unpack2(pr, plo, phi);
@@ -1105,7 +1127,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
             v = (CH16 && kk == 0) ? mul2_rn_ftz(cc2, pr) : fma2_rn_ftz(cc2, pr, acc1[i][j]);
           }
           float lo, hi;
-          const u64 q = rne2_fp(v, ks_acc, nks_acc);
+          const u64 q = rne_acc(v);
           if (CLAMP) {
             unpack2(q, lo, hi);
             acc1[i][j] = pack2(clamp_mag(lo, sat), clamp_mag(hi, sat));
@@ -1130,7 +1152,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
         u64& t2 = acc2[T_IN_REGS ? i : 0][T_IN_REGS ? j : 0];
         float lo, hi;
         if (RNE) {  // both operands lie on the accumulator's grid: see the note at the first hierarchy
-          unpack2(rne2_fp(add2_rn_ftz(acc1[i][j], t2), ks_acc, nks_acc), lo, hi);
+          unpack2(rne_acc(add2_rn_ftz(acc1[i][j], t2)), lo, hi);
         } else {
           unpack2(add2_rz_ftz(acc1[i][j], t2), lo, hi);
           lo = and_bits(lo, mask);

@@ -1,0 +1,32 @@
+"""Kernel variants at the sizes where they can go wrong, against the CPU oracle, bit for bit.  Needs a B200."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import lba_oracle as orc
+from paper_2401_14110_b200 import binding as lba
+from paper_2401_14110_b200 import synth
+from paper_2401_14110_b200 import code_domain_formats, m4e3_input_formats, ORDER_SEQUENTIAL as SEQ, ORDER_CHUNKED as CHK
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def check_gemm(A, B, prod, acc, order, chunk=16, what=""):
+    one = torch.ones(1)
+    got = lba.lba_gemm(A.to(DEV), B.to(DEV), one.to(DEV), one.to(DEV), None, prod, acc, order, chunk)
+    want = orc.gemm(A.numpy(), B.numpy(), one.numpy(), one.numpy(), None, prod.as_tuple(), acc.as_tuple(), order, chunk)
+    assert (got.cpu().numpy().view(np.uint32) == want.view(np.uint32)).all(), what
+
+
+@pytest.mark.parametrize("rounding", [0, 1])
+@pytest.mark.parametrize("man", [1, 3, 4, 5, 6, 7, 8, 10])
+def test_rounding_cuts_of_every_width(man, rounding):
+    # product and sum cut to `man` bits, in both orders, E4M3 and M4E3 bytes; dense codes and Gaussian data
+    for exp in (4, 5, 6):
+        for make, dense in ((code_domain_formats, synth.random_codes((70, 112), 3)),
+                            (m4e3_input_formats, torch.arange(70 * 112).mul(37).to(torch.uint8).reshape(70, 112))):
+            prod, acc = make(man, exp, rounding)
+            B = dense.flip(0).roll(5, 1)[:67].contiguous()
+            for order in (SEQ, CHK):
+                check_gemm(dense, B, prod, acc, order, what=f"{make.__name__} M{man}E{exp} r{rounding} order {order}")
