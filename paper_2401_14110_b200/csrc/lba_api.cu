@@ -52,7 +52,7 @@ const LaunchFn kLaunch[QM_COUNT][ORD_COUNT] = {
 
 const char* const kQmName[QM_COUNT] = {"floor_fast", "floor_full", "rne_full", "rne_wide"};
 const char* const kOrdName[ORD_COUNT] = {"seq", "chunk_slab", "chunk_any", "chunk16"};
-const char* const kLdName[LD_COUNT] = {"gemm_vec", "conv_vec", "any"};
+const char* const kLdName[LD_COUNT] = {"gemm_vec", "conv_vec", "any", "gemm_rows"};
 
 // What the host needs to know about the operand bytes: the largest |x*w|, the grid every product (hence every sum)
 // lies on, the smallest non-zero |x*w| as a power of two at or below it, and the widest product significand.
@@ -368,11 +368,11 @@ int choose_tile(int64_t M, int64_t N, int64_t batch, int qm, int ord, int load, 
   // nearest-even: three more packed instructions per pair and step; the 8x8 micro-tile loses its lead
   const double eff_rne_seq[TILE_COUNT] = {1.00, 0.97, 0.99, 0.95};
   const double eff_rne_chunk[TILE_COUNT] = {0.88, 0.95, 1.00, 0.91};
-  // byte-wise loader (ResNet stem, 401408 x 64 x 147): the fetch is costly, so the tile with the fewest
+  // byte-wise convolution loader (ResNet stem, 401408 x 64 x 147): the fetch is costly, so the tile with the fewest
   // fetched rows per output wins as long as it keeps its registers
   const double eff_any[TILE_COUNT] = {0.55, 1.00, 0.87, 0.73};
   const bool rne = qm == QM_RNE_FULL;
-  const double* eff = load == LD_ANY ? eff_any
+  const double* eff = load == LD_CONV_ANY ? eff_any
                                      : (ord == ORD_SEQ ? (rne ? eff_rne_seq : eff_seq) : (rne ? eff_rne_chunk : eff_chunk));
   int best = 0;
   double best_cost = 1e300;
@@ -450,7 +450,7 @@ int run(const Problem& p, const Plan& pl, int load, cudaStream_t stream) {
     const cudaError_t e = launch_fixed(pl.ord, load, p, stream);
     return e == cudaSuccess ? LBA_OK : cuda_fail(e);
   }
-  const bool pair_ok = pl.ord == ORD_CHUNK16 && (pl.qm == QM_FLOOR_FAST || pl.qm == QM_FLOOR_FULL) && load != LD_ANY &&
+  const bool pair_ok = pl.ord == ORD_CHUNK16 && (pl.qm == QM_FLOOR_FAST || pl.qm == QM_FLOOR_FULL) && (load == LD_GEMM_VEC || load == LD_CONV_VEC) &&
                        2 * ((p.M + 63) / 64) <= 2147483647LL;
   const int tile = choose_tile(p.M, p.N, p.batch, pl.qm, pl.ord, load, pair_ok);
   if (tile == TILE_PAIR) {
@@ -559,7 +559,7 @@ int lba_gemm(const uint8_t* A, const uint8_t* B, const float* scale_a, int scale
   p.out = out;
   apply_plan(&p, pl);
   const bool vec = K % BK == 0 && aligned16(A) && aligned16(B);
-  return run(p, pl, vec ? LD_GEMM_VEC : LD_ANY, (cudaStream_t)stream);
+  return run(p, pl, vec ? LD_GEMM_VEC : LD_GEMM_ROWS, (cudaStream_t)stream);
 }
 
 int lba_gemm_batched(const uint8_t* A, const uint8_t* B, const float* scale_a, int scale_a_len, const float* scale_b,
@@ -597,7 +597,7 @@ int lba_gemm_batched(const uint8_t* A, const uint8_t* B, const float* scale_a, i
     q.A = A + b0 * stride_a;
     q.B = B + b0 * stride_b;
     q.out = out + b0 * stride_out;
-    if ((st = run(q, pl, vec ? LD_GEMM_VEC : LD_ANY, (cudaStream_t)stream)) != LBA_OK) return st;
+    if ((st = run(q, pl, vec ? LD_GEMM_VEC : LD_GEMM_ROWS, (cudaStream_t)stream)) != LBA_OK) return st;
   }
   return LBA_OK;
 }
@@ -623,7 +623,7 @@ int lba_gemm_last_overflow(const uint8_t* A, const uint8_t* B, int64_t M, int64_
   p.out = reinterpret_cast<float*>(last);
   apply_plan(&p, pl);
   const bool vec = K % BK == 0 && aligned16(A) && aligned16(B);
-  const cudaError_t e = launch_last_overflow(pl.qm, vec ? LD_GEMM_VEC : LD_ANY, p, (cudaStream_t)stream);
+  const cudaError_t e = launch_last_overflow(pl.qm, vec ? LD_GEMM_VEC : LD_GEMM_ROWS, p, (cudaStream_t)stream);
   return e == cudaSuccess ? LBA_OK : cuda_fail(e);
 }
 
@@ -689,7 +689,7 @@ int lba_gemm_ste_mask(const uint8_t* A, const uint8_t* B, int64_t M, int64_t N, 
     p.chunk_slabs = chunk / BK;
   }
   const bool vec = K % BK == 0 && aligned16(A) && aligned16(B);
-  const int load = vec ? LD_GEMM_VEC : LD_ANY;
+  const int load = vec ? LD_GEMM_VEC : LD_GEMM_ROWS;
   // the overflow masks in sequential and chunk-16 order come from the packed kernel (tile override 3 keeps the
   // scalar tracking kernel, for tests and comparisons); everything else from the scalar one
   const bool packed = ste == LBA_STE_OF && (!chunked || chunk == BK) && g_tile_override.load(std::memory_order_relaxed) != 3;
@@ -724,7 +724,7 @@ int lba_conv2d(const uint8_t* x, const uint8_t* w, const float* scale_x, int sca
   p.Hout = g.Hout; p.Wout = g.Wout;
   apply_plan(&p, pl);
   const bool vec = C_in % BK == 0 && aligned16(x) && aligned16(w);
-  return run(p, pl, vec ? LD_CONV_VEC : LD_ANY, (cudaStream_t)stream);
+  return run(p, pl, vec ? LD_CONV_VEC : LD_CONV_ANY, (cudaStream_t)stream);
 }
 
 size_t lba_gemm_host_workspace_bytes(int64_t M, int64_t N, int64_t K, int scale_a_len, int scale_b_len,
@@ -849,14 +849,14 @@ int lba_describe_plan_batched(int64_t batch, int64_t M, int64_t N, int64_t K, co
   Plan pl;
   const int st = make_plan(prod_fmt, acc_fmt, order, chunk, K, &pl);
   if (st != LBA_OK) return st;
-  const int load = vec_ok ? (is_conv ? LD_CONV_VEC : LD_GEMM_VEC) : LD_ANY;
+  const int load = vec_ok ? (is_conv ? LD_CONV_VEC : LD_GEMM_VEC) : (is_conv ? LD_CONV_ANY : LD_GEMM_ROWS);
   if (pl.fixed) {
     if (buf && buf_len)
       std::snprintf(buf, buf_len, "tile=64x64x%d micro=4x4 q=fixed order=%s load=%s grid=%lldx%lld", BK, kOrdName[pl.ord],
                     kLdName[load], (long long)((M + 63) / 64), (long long)((N + 63) / 64));
     return LBA_OK;
   }
-  const bool pair_ok = pl.ord == ORD_CHUNK16 && (pl.qm == QM_FLOOR_FAST || pl.qm == QM_FLOOR_FULL) && load != LD_ANY;
+  const bool pair_ok = pl.ord == ORD_CHUNK16 && (pl.qm == QM_FLOOR_FAST || pl.qm == QM_FLOOR_FULL) && (load == LD_GEMM_VEC || load == LD_CONV_VEC);
   const int tile = choose_tile(M > 0 ? M : 1, N > 0 ? N : 1, batch, pl.qm, pl.ord, load, pair_ok);
   // which kernel runs and what Q_prod costs there beyond the flush
   const bool packed = pl.ord != ORD_CHUNK_ANY &&

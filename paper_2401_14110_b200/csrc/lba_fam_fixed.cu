@@ -26,7 +26,8 @@ cudaError_t by_loader(int load, const Problem& p, cudaStream_t stream) {
   switch (load) {
     case LD_GEMM_VEC: return by_wrap<ORD, LD_GEMM_VEC>(p, stream);
     case LD_CONV_VEC: return by_wrap<ORD, LD_CONV_VEC>(p, stream);
-    default: return by_wrap<ORD, LD_ANY>(p, stream);
+    case LD_CONV_ANY: return by_wrap<ORD, LD_CONV_ANY>(p, stream);
+    default: return by_wrap<ORD, LD_GEMM_ROWS>(p, stream);
   }
 }
 

@@ -29,7 +29,7 @@ cudaError_t launch(const Problem& p, cudaStream_t stream) {
 
 template <int PQ, int ORD>
 cudaError_t by_loader(int load, const Problem& p, cudaStream_t stream) {
-  return load == LD_GEMM_VEC ? launch<PQ, ORD, LD_GEMM_VEC>(p, stream) : launch<PQ, ORD, LD_ANY>(p, stream);
+  return load == LD_GEMM_VEC ? launch<PQ, ORD, LD_GEMM_VEC>(p, stream) : launch<PQ, ORD, LD_GEMM_ROWS>(p, stream);
 }
 
 template <int ORD>

@@ -37,7 +37,9 @@ namespace lba {
 enum QMode { QM_FLOOR_FAST = 0, QM_FLOOR_FULL = 1, QM_RNE_FULL = 2, QM_RNE_WIDE = 3, QM_COUNT = 4 };
 // ORD_CHUNK16: chunk == BK, the paper's chunk size; only the packed floor kernel specialises it
 enum OrdMode { ORD_SEQ = 0, ORD_CHUNK_SLAB = 1, ORD_CHUNK_ANY = 2, ORD_CHUNK16 = 3, ORD_COUNT = 4 };
-enum LoadMode { LD_GEMM_VEC = 0, LD_CONV_VEC = 1, LD_ANY = 2, LD_COUNT = 3 };
+// GEMM rows at 16-byte boundaries; NHWC taps with C_in a multiple of 16; any convolution, byte by byte; GEMM rows at any
+// byte address with any K
+enum LoadMode { LD_GEMM_VEC = 0, LD_CONV_VEC = 1, LD_CONV_ANY = 2, LD_GEMM_ROWS = 3, LD_COUNT = 4 };
 
 constexpr int BK = 16;  // bytes of K per row per slab = one 128-bit load = one paper-sized chunk
 
@@ -297,6 +299,11 @@ struct RowLoader {
   bool row_ok[LPT];
   int ih0[LPT], iw0[LPT];               // conv: top-left input coordinate of the receptive field
   int ld_kh = 0, ld_kw = 0, ld_c0 = 0;  // conv vector path: position of the next slab inside (kh, kw, c_in)
+  // LD_GEMM_ROWS: the row starts `shift` bytes past the 16-byte boundary row_ptr; `carry` is the aligned block that
+  // the next slab starts in, and blocks [blk_lo, blk_hi) lie wholly inside the operand
+  static constexpr int LPS = LD == LD_GEMM_ROWS ? LPT : 1;
+  int shift[LPS], blk_lo[LPS], blk_hi[LPS];
+  uint4 carry[LPS];
   // conv byte-wise path: for one output position and one kh, the taps (kw, c_in) are KW*C_in contiguous
   // bytes of the input row ih0 + kh; the cursor is (kh, offset inside that run) of the next slab's first k
   int any_kh = 0, any_off = 0;
@@ -311,12 +318,18 @@ struct RowLoader {
       row_ok[l] = false;
       ih0[l] = 0;
       iw0[l] = 0;
+      if constexpr (LD == LD_GEMM_ROWS) {
+        shift[l] = blk_lo[l] = blk_hi[l] = 0;
+        carry[l] = make_uint4(0u, 0u, 0u, 0u);
+      }
       if (r < BM) {
         const int64_t m = m0 + r;
         if (m < p.M) {
           row_ok[l] = true;
-          if (LD == LD_GEMM_VEC || (LD == LD_ANY && !p.is_conv)) {
+          if (LD == LD_GEMM_VEC) {
             row_ptr[l] = baseA + m * p.K;
+          } else if constexpr (LD == LD_GEMM_ROWS) {
+            init_row(p, l, baseA, m, p.M);
           } else {
             const int ow = (int)(m % p.Wout);
             const int64_t t = m / p.Wout;
@@ -331,9 +344,65 @@ struct RowLoader {
         const int64_t n = n0 + (r - BM);
         if (n < p.N) {
           row_ok[l] = true;
-          row_ptr[l] = baseB + n * p.K;
+          if constexpr (LD == LD_GEMM_ROWS) init_row(p, l, baseB, n, p.N);
+          else row_ptr[l] = baseB + n * p.K;
         }
       }
+    }
+  }
+
+  // ---- LD_GEMM_ROWS.  A slab of a row that starts at any byte address spans two 16-byte blocks; the second one is the
+  // next slab's first, so each slab costs one aligned 128-bit load and a byte shift of the pair (take).  Sixteen
+  // single-byte loads per slab took 240 us where this takes 146 (1111 x 777 x 1203), 1208 against 945 (4096 x 3072 x 767).  A block that reaches past either end of
+  // the operand (first and last row only) is put together from its valid bytes.
+  __device__ __forceinline__ void init_row(const Problem& p, int l, const uint8_t* base, int64_t row, int64_t rows) {
+    const uint8_t* const start = base + row * p.K;
+    shift[l] = (int)(reinterpret_cast<uintptr_t>(start) & 15);
+    row_ptr[l] = start - shift[l];
+    blk_lo[l] = row_ptr[l] < base ? 1 : 0;
+    const int64_t whole = (base + rows * p.K - row_ptr[l]) / 16;  // blocks that end inside the operand
+    blk_hi[l] = (int)(whole < 0x7FFFFFFF ? whole : 0x7FFFFFFF);
+    carry[l] = load_block(p, l, 0);
+  }
+  __device__ __forceinline__ uint4 load_block(const Problem& p, int l, int i) const {
+    const int64_t lo = (int64_t)i * 16, row_end = shift[l] + p.K;  // byte offsets from row_ptr
+    if (lo >= row_end) return make_uint4(0u, 0u, 0u, 0u);
+    if (i >= blk_lo[l] && i < blk_hi[l]) return __ldg(reinterpret_cast<const uint4*>(row_ptr[l]) + i);
+    uint32_t w4[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll 1
+      for (int j = 0; j < 4; ++j) {
+        const int64_t off = lo + q * 4 + j;
+        if (off >= shift[l] && off < row_end) w4[q] |= (uint32_t)__ldg(row_ptr[l] + off) << (8 * j);
+      }
+    return make_uint4(w4[0], w4[1], w4[2], w4[3]);
+  }
+  // the sixteen bytes of slab `slab` from what fetch returned for it (the other loaders return them as they are).
+  // Slabs in increasing order, each once.
+  __device__ __forceinline__ uint4 take(const Problem& p, int l, int slab, const uint4& raw) {
+    if constexpr (LD != LD_GEMM_ROWS) {
+      return raw;
+    } else {
+      uint32_t w[8] = {carry[l].x, carry[l].y, carry[l].z, carry[l].w, raw.x, raw.y, raw.z, raw.w};
+      carry[l] = raw;
+      const bool by2 = shift[l] & 8, by1 = shift[l] & 4;
+      const int bits = (shift[l] & 3) * 8;
+#pragma unroll
+      for (int i = 0; i < 6; ++i) w[i] = by2 ? w[i + 2] : w[i];
+#pragma unroll
+      for (int i = 0; i < 5; ++i) w[i] = by1 ? w[i + 1] : w[i];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) w[i] = __funnelshift_r(w[i], w[i + 1], bits);
+      const int64_t left = p.K - (int64_t)slab * BK;
+      if (left < BK) {  // the bytes past K belong to the next row
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int n = (int)left - 4 * i;
+          w[i] = n >= 4 ? w[i] : n <= 0 ? 0u : (w[i] & ((1u << (8 * n)) - 1u));
+        }
+      }
+      return make_uint4(w[0], w[1], w[2], w[3]);
     }
   }
 
@@ -353,9 +422,11 @@ struct RowLoader {
           const int ih = ih0[l] + ld_kh, iw = iw0[l] + ld_kw;
           if (ih >= 0 && ih < p.H && iw >= 0 && iw < p.W)
             v = __ldg(reinterpret_cast<const uint4*>(row_ptr[l] + ((int64_t)ih * p.W + iw) * p.Cin + ld_c0));
-        } else {  // LD_ANY: byte-wise, any K, any alignment, GEMM or conv
+        } else if constexpr (LD == LD_GEMM_ROWS) {
+          v = load_block(p, l, slab + 1);
+        } else {  // LD_CONV_ANY: byte-wise, any C_in, any alignment
           uint32_t w4[4] = {0u, 0u, 0u, 0u};
-          if (!is_a || !p.is_conv) {
+          if (!is_a) {
 #pragma unroll
             for (int j = 0; j < BK; ++j) {
               const int64_t k = k0 + j;
@@ -400,7 +471,7 @@ struct RowLoader {
   // move the convolution cursors past one slab without fetching it (fetch does this itself; a CTA that
   // handles every second slab calls it once more)
   __device__ __forceinline__ void skip_slab(const Problem& p) {
-    if (LD == LD_ANY && p.is_conv) {  // advance the run cursor by one slab
+    if (LD == LD_CONV_ANY) {  // advance the run cursor by one slab
       const int run = p.KW * p.Cin;
       any_off += BK;
       while (any_off >= run) {
@@ -462,7 +533,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), TRACK == TRACK_MASK_DIF
   loader.init(p, tid, m0, n0);
   auto fetch = [&](int slab, uint4 (&raw)[LPT]) { loader.fetch(p, tid, slab, raw); };
 
-  auto decode_store = [&](const uint4 (&raw)[LPT], int buf) {
+  auto decode_store = [&](const uint4 (&raw)[LPT], int buf, int slab) {
 #pragma unroll
     for (int l = 0; l < LPT; ++l) {
       const int r = tid + l * NT;
@@ -471,7 +542,8 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), TRACK == TRACK_MASK_DIF
         const float mul = is_a ? p.dec_a : p.dec_b;
         float* dst = is_a ? &As[buf][0][r] : &Bs[buf][0][r - BM];
         const int stride = is_a ? BM : BN;
-        const uint32_t w4[4] = {raw[l].x, raw[l].y, raw[l].z, raw[l].w};
+        const uint4 row = loader.take(p, l, slab, raw[l]);
+        const uint32_t w4[4] = {row.x, row.y, row.z, row.w};
 #pragma unroll
         for (int j = 0; j < BK; ++j) {
           const uint32_t top = byte_to_top(w4[j >> 2], j & 3);
@@ -680,7 +752,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), TRACK == TRACK_MASK_DIF
   int k_in_chunk = 0;      // ORD_CHUNK_ANY
   if (nslab > 0) {
     fetch(0, raw);
-    decode_store(raw, 0);
+    decode_store(raw, 0, 0);
   }
   __syncthreads();
   for (int s = 0; s < nslab; ++s) {
@@ -723,7 +795,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), TRACK == TRACK_MASK_DIF
         }
       if ((s & 1) || s + 1 == nslab) flush_words(mask1z, W1, (int64_t)(s >> 1), bits1);
     }
-    if (s + 1 < nslab) decode_store(raw, buf ^ 1);
+    if (s + 1 < nslab) decode_store(raw, buf ^ 1, s + 1);
     __syncthreads();
     kbase += BK;
   }
@@ -884,10 +956,11 @@ enum PackedProd { PQ_NONE = 0, PQ_MASK = 1, PQ_MASK_SAT = 2, PQ_FUSED = 3 };
 template <int BM, int BN, int TM, int TN, int PQ, int RNE, int ORD, int LD, int STE = 0, int CL = 1, bool H16 = false>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN),
                                   ((TM * TN == 64 && ORD != ORD_CHUNK_SLAB && !RNE) ||
-                                   ((LD == LD_ANY || STE != 0) && !RNE && ORD != ORD_CHUNK_SLAB))
+                                   ((LD == LD_CONV_ANY || LD == LD_GEMM_ROWS || STE != 0) && !RNE && ORD != ORD_CHUNK_SLAB))
                                       ? 512 / ((BM / TM) * (BN / TN)) : 1)
     lba_contract_packed_kernel(const Problem p) {
   static_assert(STE == 0 || (!RNE && TM == 4 && TN == 8 && (ORD == ORD_SEQ || ORD == ORD_CHUNK16)), "mask variant");
+  static_assert(CL == 1 || LD == LD_GEMM_VEC || LD == LD_CONV_VEC, "a CTA of the pair skips slabs");
   static_assert(CL == 1 || (CL == 2 && !RNE && STE == 0 && ORD == ORD_CHUNK16 && TM == 4), "cluster variant");
   constexpr int NT = (BM / TM) * (BN / TN);
   constexpr int TX = BN / TN;
@@ -933,14 +1006,15 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
   RowLoader<BM, BN, NT, LD> loader;
   loader.init(p, tid, m0, n0);
 
-  auto decode_store = [&](const uint4 (&raw)[LPT], int buf, int cell) {
+  auto decode_store = [&](const uint4 (&raw)[LPT], int buf, int cell, int slab) {
 #pragma unroll
     for (int l = 0; l < LPT; ++l) {
       const int r = tid + l * NT;
       if (r < ROWS) {  // uniform per warp: BM, BN and NT are multiples of 32
         const bool is_a = r < BM;
         const float mul = is_a ? p.pk_a : p.pk_b;
-        const uint32_t w4[4] = {raw[l].x, raw[l].y, raw[l].z, raw[l].w};
+        const uint4 row = loader.take(p, l, slab, raw[l]);
+        const uint32_t w4[4] = {row.x, row.y, row.z, row.w};
         float n2 = 0.0f;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -1250,7 +1324,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
   if (CL > 1 && crank != 0) loader.skip_slab(p);
   if (s_first < nslab) {
     loader.fetch(p, tid, s_first, raw);
-    decode_store(raw, 0, 0);
+    decode_store(raw, 0, 0, s_first);
   }
   __syncthreads();
 
@@ -1491,7 +1565,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
         fold_received(std::integral_constant<int, 1>(), q);
         if (have) fold_own(std::integral_constant<int, 1>(), grow);
       }
-      if (more) decode_store(raw, buf ^ 1, cell_next);
+      if (more) decode_store(raw, buf ^ 1, cell_next, s + CL);
       __syncthreads();
       cell = cell_next;
     }
@@ -1588,7 +1662,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
         }
       }
     }
-    if (s + 1 < nslab) decode_store(raw, buf ^ 1, cell_next);
+    if (s + 1 < nslab) decode_store(raw, buf ^ 1, cell_next, s + 1);
     __syncthreads();
     cell = cell_next;
   }

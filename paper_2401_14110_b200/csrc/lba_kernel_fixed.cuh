@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(256) lba_fixed_kernel(const Problem p) {
   RowLoader<BM, BN, NT, LD> loader;
   loader.init(p, tid, m0, n0);
 
-  auto decode_store = [&](const uint4 (&raw)[LPT], int buf) {
+  auto decode_store = [&](const uint4 (&raw)[LPT], int buf, int slab) {
 #pragma unroll
     for (int l = 0; l < LPT; ++l) {
       const int r = tid + l * NT;
@@ -67,7 +67,8 @@ __global__ void __launch_bounds__(256) lba_fixed_kernel(const Problem p) {
         int* dm = is_a ? &Am[buf][0][r] : &Bm[buf][0][r - BM];
         int* dq = is_a ? &Aq[buf][0][r] : &Bq[buf][0][r - BM];
         const int stride = is_a ? BM : BN;
-        const uint32_t w4[4] = {raw[l].x, raw[l].y, raw[l].z, raw[l].w};
+        const uint4 row = loader.take(p, l, slab, raw[l]);
+        const uint32_t w4[4] = {row.x, row.y, row.z, row.w};
 #pragma unroll
         for (int j = 0; j < BK; ++j) {
           const uint32_t c = (w4[j >> 2] >> (8 * (j & 3))) & 0xFFu;
@@ -142,7 +143,7 @@ __global__ void __launch_bounds__(256) lba_fixed_kernel(const Problem p) {
   int k_in_chunk = 0;
   if (nslab > 0) {
     loader.fetch(p, tid, 0, raw);
-    decode_store(raw, 0);
+    decode_store(raw, 0, 0);
   }
   __syncthreads();
   for (int s = 0; s < nslab; ++s) {
@@ -175,7 +176,7 @@ __global__ void __launch_bounds__(256) lba_fixed_kernel(const Problem p) {
         }
       }
     }
-    if (s + 1 < nslab) decode_store(raw, buf ^ 1);
+    if (s + 1 < nslab) decode_store(raw, buf ^ 1, s + 1);
     __syncthreads();
   }
   if (ORD == ORD_CHUNK_SLAB && slabs_in_chunk > 0) close_chunk();

@@ -18,7 +18,7 @@ cudaError_t launch(const Problem& p, cudaStream_t stream) {
 
 template <int QM, int ORD, int TRACK>
 cudaError_t by_loader(int load, const Problem& p, cudaStream_t stream) {
-  return load == LD_GEMM_VEC ? launch<QM, ORD, LD_GEMM_VEC, TRACK>(p, stream) : launch<QM, ORD, LD_ANY, TRACK>(p, stream);
+  return load == LD_GEMM_VEC ? launch<QM, ORD, LD_GEMM_VEC, TRACK>(p, stream) : launch<QM, ORD, LD_GEMM_ROWS, TRACK>(p, stream);
 }
 
 template <int QM, int TRACK>

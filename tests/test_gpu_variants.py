@@ -30,3 +30,20 @@ def test_rounding_cuts_of_every_width(man, rounding):
             B = dense.flip(0).roll(5, 1)[:67].contiguous()
             for order in (SEQ, CHK):
                 check_gemm(dense, B, prod, acc, order, what=f"{make.__name__} M{man}E{exp} r{rounding} order {order}")
+
+
+@pytest.mark.parametrize("K", [1, 15, 16, 17, 31, 33, 130])
+def test_rows_at_every_byte_address(K):
+    # operands that start at every offset from a 16-byte boundary, at the very end of their storage, K around whole blocks
+    prod, acc = code_domain_formats(7, 4)
+    M, N = 5, 35
+    one = torch.ones(1, device=DEV)
+    for off in range(16):
+        A, B = synth.random_codes((M, K), 100 + off), synth.random_codes((N, K), 200 + off)
+        store = [torch.full((off + t.numel(),), 0x7F, dtype=torch.uint8, device=DEV) for t in (A, B)]
+        a, b = [s[off:].view(t.shape).copy_(t) for s, t in zip(store, (A, B))]
+        for order in (SEQ, CHK):
+            got = lba.lba_gemm(a, b, one, one, None, prod, acc, order, 16).cpu().numpy()
+            want = orc.gemm(A.numpy(), B.numpy(), np.ones(1, np.float32), np.ones(1, np.float32), None, prod.as_tuple(),
+                            acc.as_tuple(), order, 16)
+            assert (got.view(np.uint32) == want.view(np.uint32)).all(), (off, order)
