@@ -8,7 +8,7 @@
 #include <mutex>
 
 #include "../../include/lba.h"
-#include "lba_kernel.cuh"
+#include "lba_kernel_small.cuh"
 
 namespace lba {
 
@@ -20,6 +20,9 @@ LBA_DECL(QM_FLOOR_FULL, ORD_SEQ) LBA_DECL(QM_FLOOR_FULL, ORD_CHUNK_SLAB) LBA_DEC
 LBA_DECL(QM_RNE_FULL, ORD_SEQ) LBA_DECL(QM_RNE_FULL, ORD_CHUNK_SLAB) LBA_DECL(QM_RNE_FULL, ORD_CHUNK_ANY)
 LBA_DECL(QM_RNE_WIDE, ORD_SEQ) LBA_DECL(QM_RNE_WIDE, ORD_CHUNK_SLAB) LBA_DECL(QM_RNE_WIDE, ORD_CHUNK_ANY)
 #undef LBA_DECL
+template <> cudaError_t launch_small<0>(int, int, const Problem&, cudaStream_t);
+template <> cudaError_t launch_small<1>(int, int, const Problem&, cudaStream_t);
+template <> cudaError_t launch_small<2>(int, int, const Problem&, cudaStream_t);
 
 cudaError_t launch_last_overflow(int qm, int load, const Problem& p, cudaStream_t stream);
 cudaError_t launch_ste_mask(int qm, int ord, int diff, int load, const Problem& p, cudaStream_t stream);
@@ -356,11 +359,22 @@ int sm_count() {
 // neighbours runs each of them faster, so the last, partial round costs less than a full one: measured on
 // 4096-row GEMMs of 768 to 3072 columns, counting half of the rounding-up reproduces the order of the tiles.
 // Pick the cheapest by that model.
-// pair_ok: the call qualifies for the 64x64 tile shared by a cluster of two CTAs (TILE_PAIR)
-int choose_tile(int64_t M, int64_t N, int64_t batch, int qm, int ord, int load, bool pair_ok = false) {
+TileInfo small_tile(int t) {
+  return t == TILE_SPLIT ? TileInfo{16, 16, 2, 4} : t == TILE_SPLIT + 1 ? TileInfo{32, 32, 4, 8}
+         : TileInfo{16, 16, 1, 2};
+}
+
+int choose_tile(int64_t M, int64_t N, int64_t K, int64_t batch, const Plan& pl, int load) {
+  const int qm = pl.qm, ord = pl.ord;
+  const bool vec = load == LD_GEMM_VEC || load == LD_CONV_VEC, floor = qm == QM_FLOOR_FAST || qm == QM_FLOOR_FULL;
+  const bool pair_ok = ord == ORD_CHUNK16 && floor && vec && 2 * ((M + 63) / 64) <= 2147483647LL;
+  const bool small_ok = load != LD_CONV_ANY && (floor || (qm == QM_RNE_FULL && pl.rne_packed)) && N <= 16 * 65535LL &&
+                        M <= 16 * 2147483647LL;
   const int forced = g_tile_override.load(std::memory_order_relaxed);
   if (forced >= 0 && forced < TILE_COUNT) return forced;
   if (forced == TILE_PAIR && pair_ok) return TILE_PAIR;
+  if ((forced == TILE_SPLIT || forced == TILE_SPLIT + 1) && small_ok && ord == ORD_CHUNK16) return forced;
+  if (forced == TILE_CHAIN && small_ok && ord == ORD_SEQ) return forced;
   const int sms = sm_count();
   // relative MAC rate of each tile with every SM loaded (8192^2 x 1024 and 4096 x 3072 x 768 GEMMs)
   const double eff_seq[TILE_COUNT] = {1.00, 0.92, 0.96, 0.82};
@@ -450,9 +464,13 @@ int run(const Problem& p, const Plan& pl, int load, cudaStream_t stream) {
     const cudaError_t e = launch_fixed(pl.ord, load, p, stream);
     return e == cudaSuccess ? LBA_OK : cuda_fail(e);
   }
-  const bool pair_ok = pl.ord == ORD_CHUNK16 && (pl.qm == QM_FLOOR_FAST || pl.qm == QM_FLOOR_FULL) && (load == LD_GEMM_VEC || load == LD_CONV_VEC) &&
-                       2 * ((p.M + 63) / 64) <= 2147483647LL;
-  const int tile = choose_tile(p.M, p.N, p.batch, pl.qm, pl.ord, load, pair_ok);
+  const int tile = choose_tile(p.M, p.N, p.K, p.batch, pl, load);
+  if (tile >= TILE_SPLIT) {  // choose_tile keeps the grid within its limits
+    const int rne = pl.qm == QM_RNE_FULL ? pl.rne_packed : 0;
+    const cudaError_t e = rne == 0 ? launch_small<0>(tile, load, p, stream)
+                                   : rne == 1 ? launch_small<1>(tile, load, p, stream) : launch_small<2>(tile, load, p, stream);
+    return e == cudaSuccess ? LBA_OK : cuda_fail(e);
+  }
   if (tile == TILE_PAIR) {
     if ((p.N + 63) / 64 > 65535) return LBA_ERR_SHAPE;
     const cudaError_t e = launch_cluster_pair(pl.qm == QM_FLOOR_FAST ? PQ_NONE : pl.pq, load, p, stream);
@@ -518,7 +536,7 @@ int lba_version(void) { return 1; }
 int lba_last_cuda_error(void) { return g_last_cuda_error; }
 
 int lba_set_tile_override(int tile) {
-  if (tile < -1 || tile > TILE_PAIR || tile == TILE_COUNT) return LBA_ERR_SHAPE;
+  if (tile < -1 || tile > TILE_CHAIN || tile == TILE_COUNT || tile == 8 || tile == 9) return LBA_ERR_SHAPE;
   g_tile_override.store(tile, std::memory_order_relaxed);
   return LBA_OK;
 }
@@ -856,13 +874,12 @@ int lba_describe_plan_batched(int64_t batch, int64_t M, int64_t N, int64_t K, co
                     kLdName[load], (long long)((M + 63) / 64), (long long)((N + 63) / 64));
     return LBA_OK;
   }
-  const bool pair_ok = pl.ord == ORD_CHUNK16 && (pl.qm == QM_FLOOR_FAST || pl.qm == QM_FLOOR_FULL) && (load == LD_GEMM_VEC || load == LD_CONV_VEC);
-  const int tile = choose_tile(M > 0 ? M : 1, N > 0 ? N : 1, batch, pl.qm, pl.ord, load, pair_ok);
+  const int tile = choose_tile(M > 0 ? M : 1, N > 0 ? N : 1, K, batch, pl, load);
   // which kernel runs and what Q_prod costs there beyond the flush
   const bool packed = pl.ord != ORD_CHUNK_ANY &&
                       (pl.qm == QM_FLOOR_FAST || pl.qm == QM_FLOOR_FULL || (pl.qm == QM_RNE_FULL && pl.rne_packed));
   const char* const kern = packed ? "packed" : "generic";
-  const char* const pq = (pl.fused && packed && tile != TILE_PAIR) ? "fused"
+  const char* const pq = (pl.fused && packed && tile < TILE_PAIR) ? "fused"
                          : (pl.qm == QM_FLOOR_FAST || pl.qm == QM_RNE_WIDE ? "none"
                             : (pl.pq == PQ_MASK_SAT ? "cut_sat" : (pl.pq == PQ_MASK ? "cut" : "none")));
   if (tile == TILE_PAIR) {
@@ -870,6 +887,14 @@ int lba_describe_plan_batched(int64_t batch, int64_t M, int64_t N, int64_t K, co
       std::snprintf(buf, buf_len, "tile=64x64x%d pair micro=4x8 q=%s pq=%s kernel=%s order=%s load=%s grid=%lldx%lld", BK,
                     kQmName[pl.qm], pq, kern, kOrdName[pl.ord], kLdName[load], (long long)(2 * ((M + 63) / 64)),
                     (long long)((N + 63) / 64));
+    return LBA_OK;
+  }
+  if (tile >= TILE_SPLIT) {
+    const TileInfo t = small_tile(tile);
+    if (buf && buf_len)
+      std::snprintf(buf, buf_len, "tile=%dx%dx%d %s micro=%dx%d q=%s pq=%s kernel=%s order=%s load=%s grid=%lldx%lld", t.bm, t.bn, BK,
+                    tile >= TILE_CHAIN ? "chain" : "split", t.tm, t.tn, kQmName[pl.qm], pq, kern, kOrdName[pl.ord], kLdName[load],
+                    (long long)((M + t.bm - 1) / t.bm), (long long)((N + t.bn - 1) / t.bn));
     return LBA_OK;
   }
   const TileInfo ti = tile_info(tile);

@@ -468,6 +468,15 @@ struct RowLoader {
     skip_slab(p);
   }
 
+  // the same for a caller that skips slabs: the first block of a row's slab is then not the one it carries
+  __device__ __forceinline__ void fetch_apart(const Problem& p, int tid, int slab, uint4 (&raw)[LPT]) {
+    if constexpr (LD == LD_GEMM_ROWS) {
+#pragma unroll
+      for (int l = 0; l < LPT; ++l) carry[l] = row_ok[l] ? load_block(p, l, slab) : make_uint4(0u, 0u, 0u, 0u);
+    }
+    fetch(p, tid, slab, raw);
+  }
+
   // move the convolution cursors past one slab without fetching it (fetch does this itself; a CTA that
   // handles every second slab calls it once more)
   __device__ __forceinline__ void skip_slab(const Problem& p) {
@@ -1748,6 +1757,8 @@ constexpr size_t packed_ste_smem_bytes() {
 struct TileInfo { int bm, bn, tm, tn; };
 constexpr int TILE_COUNT = 4;
 constexpr int TILE_PAIR = 5;  // 64x64 tile shared by a cluster of two CTAs (chunk-16 order, floor rounding)
+constexpr int TILE_SPLIT = 6;   // 6, 7: 16x16 and 32x32 with the chunk sums spread over the warps (lba_split_kernel)
+constexpr int TILE_CHAIN = 10;  // 16x16, one pair of chains per thread (lba_chain_kernel)
 __host__ inline TileInfo tile_info(int t) {
   const TileInfo tab[TILE_COUNT] = {{128, 128, 8, 8}, {128, 64, 4, 8}, {64, 64, 4, 8}, {32, 32, 4, 4}};
   return tab[t];

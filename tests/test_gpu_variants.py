@@ -6,7 +6,7 @@ import torch
 from oracle import lba_oracle as orc
 from paper_2401_14110_b200 import binding as lba
 from paper_2401_14110_b200 import synth
-from paper_2401_14110_b200 import code_domain_formats, m4e3_input_formats, ORDER_SEQUENTIAL as SEQ, ORDER_CHUNKED as CHK
+from paper_2401_14110_b200 import LbaFormat, code_domain_formats, m4e3_input_formats, ORDER_SEQUENTIAL as SEQ, ORDER_CHUNKED as CHK
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -47,3 +47,43 @@ def test_rows_at_every_byte_address(K):
             want = orc.gemm(A.numpy(), B.numpy(), np.ones(1, np.float32), np.ones(1, np.float32), None, prod.as_tuple(),
                             acc.as_tuple(), order, 16)
             assert (got.view(np.uint32) == want.view(np.uint32)).all(), (off, order)
+
+
+SMALL_FORMATS = {
+    "m7e4": code_domain_formats(7, 4), "m4e4": code_domain_formats(4, 4), "m10e6": code_domain_formats(10, 6),
+    "m7e4_rne": code_domain_formats(7, 4, 1), "m10e5_rne": code_domain_formats(10, 5, 1), "m4e4_rne": code_domain_formats(4, 4, 1),
+    "m7e4_m4e3": m4e3_input_formats(7, 4), "m7e4_low_top": (LbaFormat(7, 4, 4), LbaFormat(7, 4, 6)),
+}
+
+
+@pytest.mark.parametrize("tile", [6, 7, 10])
+@pytest.mark.parametrize("name", list(SMALL_FORMATS))
+def test_small_problem_kernels(tile, name):
+    # edges of the tiles, one to many rounds of chunks, short last chunk and round, saturating data; all loaders
+    prod, acc = SMALL_FORMATS[name]
+    order = CHK if tile < 10 else SEQ
+    one = torch.ones(1)
+    lba.set_tile_override(tile)
+    try:
+        for (M, N, K) in ((1, 1, 17), (16, 32, 32), (33, 47, 127), (5, 100, 128), (40, 17, 144), (31, 33, 1040), (2, 64, 1039)):
+            A, B = synth.random_codes((M, K), 7 * M + K), synth.random_codes((N, K), 11 * N + K)
+            if K == 1040:
+                A, B = A & 0x7F, B & 0x7F
+                A[:, 600:] |= 0x80
+            if name == "m7e4":
+                assert ("split" if tile < 10 else "chain") in lba.describe_plan(M, N, K, prod, acc, order, 16, vec_ok=K % 16 == 0)
+            sa, sb, bias = torch.linspace(0.5, 1.5, M), torch.linspace(0.01, 0.02, N), torch.linspace(-1, 1, N)
+            got = lba.lba_gemm(A.to(DEV), B.to(DEV), sa.to(DEV), sb.to(DEV), bias.to(DEV), prod, acc, order, 16).cpu().numpy()
+            want = orc.gemm(A.numpy(), B.numpy(), sa.numpy(), sb.numpy(), bias.numpy(), prod.as_tuple(), acc.as_tuple(), order, 16)
+            assert (got.view(np.uint32) == want.view(np.uint32)).all(), (M, N, K)
+        x, w = synth.random_codes((2, 5, 7, 32), 1), synth.random_codes((19, 3, 3, 32), 2)
+        got = lba.lba_conv2d(x.to(DEV), w.to(DEV), one.to(DEV), one.to(DEV), None, (2, 1), (1, 1), prod, acc, order, 16).cpu().numpy()
+        want = orc.conv2d(x.numpy(), w.numpy(), one.numpy(), one.numpy(), None, (2, 1), (1, 1), prod.as_tuple(), acc.as_tuple(), order, 16)
+        assert (got.view(np.uint32) == want.view(np.uint32)).all()
+        A, B = synth.random_codes((3, 20, 48), 5), synth.random_codes((3, 35, 48), 6)
+        got = lba.lba_gemm_batched(A.to(DEV), B.to(DEV), one.to(DEV), one.to(DEV), None, prod, acc, order, 16).cpu().numpy()
+        for z in range(3):
+            want = orc.gemm(A[z].numpy(), B[z].numpy(), one.numpy(), one.numpy(), None, prod.as_tuple(), acc.as_tuple(), order, 16)
+            assert (got[z].view(np.uint32) == want.view(np.uint32)).all()
+    finally:
+        lba.set_tile_override(-1)
