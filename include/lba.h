@@ -239,7 +239,10 @@ int lba_count_nan_codes(const uint8_t* codes, int64_t n, unsigned long long* cou
  * "tile=64x64x16 micro=4x8 q=floor_fast pq=none kernel=packed order=chunk16 load=gemm_vec grid=128x128"
  * (pq: what Q_prod does beyond its flush -- none, cut = mantissa cut, cut_sat = cut and saturation, fused = Q_prod is
  * the identity on every reachable product, so product and sum are one instruction; kernel: the
- * packed two-outputs-per-instruction kernel or the generic scalar one).
+ * packed two-outputs-per-instruction kernel or the generic scalar one).  A problem too small to fill the GPU with these tiles
+ * runs in one of the small-problem kernels instead; the text then ends in " by=split16x16" or " by=split32x32" (chunks of
+ * 16: the chunk sums of a tile spread over the warps of a CTA) or " by=chain16x16" (sequential), and tile, micro and grid
+ * are those of the packed kernel it replaces.
  * is_conv selects the loader family; for a convolution pass M = B*H_out*W_out, N = C_out,
  * K = KH*KW*C_in and vec_ok = (C_in % 16 == 0 and pointers aligned).  Returns LBA_OK or the
  * error the real call would return; buf may be NULL. */
@@ -253,7 +256,8 @@ int lba_describe_plan_batched(int64_t batch, int64_t M, int64_t N, int64_t K, co
 
 /* Testing and tuning hook: force the CTA tile (0 = 128x128, 1 = 128x64, 2 = 64x64, 3 = 32x32 outputs; 5 = the 64x64
  * tile shared by a cluster of two CTAs, each taking every second chunk, used only in chunk-16 order with floor
- * rounding and 16-byte loads, ignored otherwise; -1 = automatic choice, the default).  For lba_gemm_ste_mask, 3
+ * rounding and 16-byte loads, ignored otherwise; 6, 7 = the small-problem kernels of chunk-16 order on 16x16 and 32x32
+ * tiles, 10 = that of sequential order, ignored where they do not apply; -1 = automatic choice, the default).  For lba_gemm_ste_mask, 3
  * selects the scalar tracking kernel where the packed one would run.  Results never depend on the tile, only speed
  * does.  The setting is one process-wide word (an atomic store): it is meant for tests and tuning runs, it applies
  * to every thread's later calls, and a caller that changes it while other threads are inside the library gets an

@@ -69,8 +69,6 @@ struct InputInfo {
 };
 constexpr InputInfo kE4M3 = {448.0 * 448.0, 18, -18, -18, 8, 120};
 constexpr InputInfo kM4E3 = {248.0 * 248.0, 16, -8, 0, 10, 0};
-constexpr double kPartialRound = 0.5;          // share of the rounding-up of CTAs / SMs that a partial last round costs (measured)
-constexpr double kPairEff = 0.91;              // MAC rate of the cluster-pair tile relative to the plain 64x64 tile (measured)
 
 struct Plan {
   int qm, ord;
@@ -353,63 +351,84 @@ int sm_count() {
   return v;
 }
 
-// Tile choice.  All CTAs of a launch have the same work and K is never split, so the launch ends when the
-// busiest SM has run its ceil(CTAs / SMs) tiles; larger tiles spend fewer instructions per MAC (eff, measured
-// on B200 with every SM loaded), smaller ones fill the SMs more evenly.  An SM that holds fewer CTAs than its
-// neighbours runs each of them faster, so the last, partial round costs less than a full one: measured on
-// 4096-row GEMMs of 768 to 3072 columns, counting half of the rounding-up reproduces the order of the tiles.
-// Pick the cheapest by that model.
-TileInfo small_tile(int t) {
-  return t == TILE_SPLIT ? TileInfo{16, 16, 2, 4} : t == TILE_SPLIT + 1 ? TileInfo{32, 32, 4, 8}
-         : TileInfo{16, 16, 1, 2};
-}
+// Tile choice.  All CTAs of a launch have the same work and K is split only between the warps of a CTA (lba_split_kernel) or
+// the CTAs of a pair, so the launch ends when the busiest SM has run its CTAs.  Its time is modelled per tile as
+//   base + cbrt((rounds * L)^3 + (slabs / g * b * q)^3)   microseconds,
+// L: time of one round of a CTA that has the SM to itself (the latency of its chain of steps), b: time a round adds where the SM is
+// full, g: slabs of 16 k that a round takes, q: CTAs on the busiest SM, of whose rounding-up a share w counts (CTAs that are few on
+// their SM run faster).  The constants are fitted to 75 shapes per table (16 to 8192 rows and columns, K 64 to 4608, the layers of
+// ResNet-18, ResNet-50 and BERT among them), every tile timed on each: on average 0.1 to 1.3 % slower than the best tile of
+// each shape, where one table of relative rates lost 17 to 45 % because it knew no latency and no small tiles.
+struct TileCost { double L, b, base, w; };
+enum { COST_PAIR = 4, COST_SMALL = 5, COST_TILES = 7 };
+const TileCost kCost[7][COST_TILES] = {
+    // 128x128, 128x64, 64x64, 32x32, pair, 16x16 chain (sequential) or split, 32x32 split
+    {{0.02, 3.314, 5.3, 0.87}, {0.98, 1.785, 3.8, 0.92}, {0.88, 0.867, 4.3, 1}, {0.71, 0.261, 3.1, 1}, {0, 0, 0, 0}, {0.02, 0.138, 3.4, 1}, {0, 0, 0, 0}},  // floor, sequential
+    {{0.86, 3.66, 5.8, 0.84}, {1.14, 1.878, 3.5, 0.96}, {0.94, 0.931, 4, 1}, {0.73, 0.28, 3.1, 1}, {1.8, 1.079, 3.4, 1}, {0, 1.863, 2.4, 0.57}, {1.49, 2.437, 2.4, 0.85}},  // floor, chunks of 16
+    {{3.81, 6.691, 3, 1}, {3.08, 3.613, 1.9, 1}, {2.15, 1.822, 3.7, 1}, {1.65, 0.538, 2.2, 0.69}, {0, 0, 0, 0}, {0, 0.206, 3.9, 0.85}, {0, 0, 0, 0}},  // floor with product cut, sequential
+    {{2.87, 5.191, 6, 1}, {1.78, 2.756, 3.7, 0.97}, {1.76, 1.4, 4.4, 0.97}, {1.03, 0.394, 3.4, 0.97}, {2.86, 1.551, 3.2, 0.62}, {0, 2.736, 2.6, 0.82}, {2.42, 4.412, 2.9, 0.92}},  // floor with product cut, chunks of 16
+    {{1.9, 4.724, 4.7, 0.98}, {1.49, 2.478, 3.2, 1}, {1.2, 1.277, 2.9, 1}, {0.95, 0.354, 2.1, 1}, {0, 0, 0, 0}, {0.24, 0.145, 2.5, 0.99}, {0, 0, 0, 0}},  // nearest-even, sequential
+    {{0.08, 5.151, 4.6, 1}, {0.01, 2.783, 3.2, 1}, {1.25, 1.317, 3.5, 1}, {0.97, 0.365, 3.5, 1}, {0, 0, 0, 0}, {0.01, 1.993, 2.6, 0.68}, {1.8, 2.967, 2.7, 0.9}},  // nearest-even, chunks of 16
+    {{0, 4.75, 4.2, 1}, {0.05, 2.575, 3.3, 1}, {1.29, 1.14, 3.9, 1}, {0.95, 0.323, 3, 1}, {0, 0, 0, 0}, {0, 1.972, 2.6, 0.5}, {1.98, 2.766, 2.5, 0.92}},  // nearest-even through bfloat16, chunks of 16
+};
+// byte-wise convolution loader (ResNet stem, 401408 x 64 x 147): the fetch is costly, so the tile with the fewest fetched rows
+// per output wins as long as it keeps its registers
+const TileCost kCostConvAny[TILE_COUNT] = {{6, 10.4, 4, 0.5}, {2, 2.85, 4, 0.5}, {1.2, 1.64, 4, 0.5}, {0.8, 0.49, 4, 0.5}};
 
-int choose_tile(int64_t M, int64_t N, int64_t K, int64_t batch, const Plan& pl, int load) {
+struct TileChoice {
+  int packed;  // the fastest of the tiles of the packed and generic kernels (TILE_PAIR among them)
+  int run;     // the tile that runs: `packed`, or one of the small-problem kernels where that is faster
+};
+
+TileChoice choose_tile(int64_t M, int64_t N, int64_t K, int64_t batch, const Plan& pl, int load) {
   const int qm = pl.qm, ord = pl.ord;
   const bool vec = load == LD_GEMM_VEC || load == LD_CONV_VEC, floor = qm == QM_FLOOR_FAST || qm == QM_FLOOR_FULL;
   const bool pair_ok = ord == ORD_CHUNK16 && floor && vec && 2 * ((M + 63) / 64) <= 2147483647LL;
   const bool small_ok = load != LD_CONV_ANY && (floor || (qm == QM_RNE_FULL && pl.rne_packed)) && N <= 16 * 65535LL &&
                         M <= 16 * 2147483647LL;
+  const bool split_ok = small_ok && ord == ORD_CHUNK16, chain_ok = small_ok && ord == ORD_SEQ;
   const int forced = g_tile_override.load(std::memory_order_relaxed);
-  if (forced >= 0 && forced < TILE_COUNT) return forced;
-  if (forced == TILE_PAIR && pair_ok) return TILE_PAIR;
-  if ((forced == TILE_SPLIT || forced == TILE_SPLIT + 1) && small_ok && ord == ORD_CHUNK16) return forced;
-  if (forced == TILE_CHAIN && small_ok && ord == ORD_SEQ) return forced;
+  if (forced >= 0 && forced < TILE_COUNT) return {forced, forced};
+  if (forced == TILE_PAIR && pair_ok) return {TILE_PAIR, TILE_PAIR};
+
+  const bool chunked = ord != ORD_SEQ;
+  const int row = qm == QM_RNE_FULL ? (pl.rne_packed == 2 ? 6 : chunked ? 5 : 4) : qm == QM_FLOOR_FULL ? (chunked ? 3 : 2) : chunked;
+  const double slabs = std::fmax(1.0, (double)((K + BK - 1) / BK));
   const int sms = sm_count();
-  // relative MAC rate of each tile with every SM loaded (8192^2 x 1024 and 4096 x 3072 x 768 GEMMs)
-  const double eff_seq[TILE_COUNT] = {1.00, 0.92, 0.96, 0.82};
-  const double eff_chunk[TILE_COUNT] = {1.00, 0.96, 0.99, 0.87};
-  // nearest-even: three more packed instructions per pair and step; the 8x8 micro-tile loses its lead
-  const double eff_rne_seq[TILE_COUNT] = {1.00, 0.97, 0.99, 0.95};
-  const double eff_rne_chunk[TILE_COUNT] = {0.88, 0.95, 1.00, 0.91};
-  // byte-wise convolution loader (ResNet stem, 401408 x 64 x 147): the fetch is costly, so the tile with the fewest
-  // fetched rows per output wins as long as it keeps its registers
-  const double eff_any[TILE_COUNT] = {0.55, 1.00, 0.87, 0.73};
-  const bool rne = qm == QM_RNE_FULL;
-  const double* eff = load == LD_CONV_ANY ? eff_any
-                                     : (ord == ORD_SEQ ? (rne ? eff_rne_seq : eff_seq) : (rne ? eff_rne_chunk : eff_chunk));
-  int best = 0;
-  double best_cost = 1e300;
+  const auto time = [&](const TileCost& c, int bm, int bn, double per_tile, double g) {
+    const double x = per_tile * (double)((M + bm - 1) / bm) * (double)((N + bn - 1) / bn) * (double)batch / sms;
+    const double q = std::fmax(1.0, x + c.w * (std::ceil(x) - x));
+    const double chain = std::ceil(slabs / g) * c.L, work = slabs / g * c.b * q;
+    return c.base + std::cbrt(chain * chain * chain + work * work * work);
+  };
+  TileChoice best = {0, 0};
+  double least = 1e300;
   for (int t = 0; t < TILE_COUNT; ++t) {
     const TileInfo ti = tile_info(t);
-    const double ctas = (double)((M + ti.bm - 1) / ti.bm) * (double)((N + ti.bn - 1) / ti.bn) * (double)batch;
-    const double rounds = std::ceil(ctas / sms);
-    const double per_sm = std::fmax(1.0, ctas / sms + kPartialRound * (rounds - ctas / sms));
-    double cost = per_sm * ti.bm * ti.bn / eff[t];
-    if (t == 0 && rounds < 2) cost /= 0.85;  // one 8-warp CTA alone does not keep an SM's pipes busy
-    if (cost < best_cost) {
-      best_cost = cost;
-      best = t;
+    const double c = time(load == LD_CONV_ANY ? kCostConvAny[t] : kCost[row][t], ti.bm, ti.bn, 1.0, 1.0);
+    if (c < least) {
+      least = c;
+      best.packed = t;
     }
   }
   if (pair_ok) {
-    // two CTAs per 64x64 tile, each with half the chunks: twice the CTAs at half the work, a few per cent for the
-    // hand-over of the chunk sums and the cluster barrier
-    const double ctas = 2.0 * (double)((M + 63) / 64) * (double)((N + 63) / 64) * (double)batch;
-    const double per_sm = std::fmax(1.0, ctas / sms + kPartialRound * (std::ceil(ctas / sms) - ctas / sms));
-    const double cost = per_sm * (64.0 * 64.0 / 2.0) / (eff[2] * kPairEff);
-    if (cost < best_cost) best = TILE_PAIR;
+    const double c = time(kCost[row][COST_PAIR], 64, 64, 2.0, 2.0);
+    if (c < least) {
+      least = c;
+      best.packed = TILE_PAIR;
+    }
   }
+  best.run = best.packed;
+  if (forced == TILE_CHAIN ? chain_ok : (forced == TILE_SPLIT || forced == TILE_SPLIT + 1) && split_ok) best.run = forced;
+  if (forced >= 0) return best;
+  if (chain_ok || split_ok) {
+    const double c = time(kCost[row][COST_SMALL], 16, 16, 1.0, split_ok ? 16.0 : 1.0);
+    if (c < least) {
+      least = c;
+      best.run = split_ok ? TILE_SPLIT : TILE_CHAIN;
+    }
+  }
+  if (split_ok && time(kCost[row][COST_SMALL + 1], 32, 32, 1.0, 8.0) < least) best.run = TILE_SPLIT + 1;
   return best;
 }
 
@@ -464,7 +483,7 @@ int run(const Problem& p, const Plan& pl, int load, cudaStream_t stream) {
     const cudaError_t e = launch_fixed(pl.ord, load, p, stream);
     return e == cudaSuccess ? LBA_OK : cuda_fail(e);
   }
-  const int tile = choose_tile(p.M, p.N, p.K, p.batch, pl, load);
+  const int tile = choose_tile(p.M, p.N, p.K, p.batch, pl, load).run;
   if (tile >= TILE_SPLIT) {  // choose_tile keeps the grid within its limits
     const int rne = pl.qm == QM_RNE_FULL ? pl.rne_packed : 0;
     const cudaError_t e = rne == 0 ? launch_small<0>(tile, load, p, stream)
@@ -874,7 +893,9 @@ int lba_describe_plan_batched(int64_t batch, int64_t M, int64_t N, int64_t K, co
                     kLdName[load], (long long)((M + 63) / 64), (long long)((N + 63) / 64));
     return LBA_OK;
   }
-  const int tile = choose_tile(M > 0 ? M : 1, N > 0 ? N : 1, K, batch, pl, load);
+  const TileChoice choice = choose_tile(M > 0 ? M : 1, N > 0 ? N : 1, K, batch, pl, load);
+  const int tile = choice.packed;
+  const char* const by = choice.run == choice.packed ? "" : choice.run == TILE_SPLIT ? " by=split16x16" : choice.run == TILE_CHAIN ? " by=chain16x16" : " by=split32x32";
   // which kernel runs and what Q_prod costs there beyond the flush
   const bool packed = pl.ord != ORD_CHUNK_ANY &&
                       (pl.qm == QM_FLOOR_FAST || pl.qm == QM_FLOOR_FULL || (pl.qm == QM_RNE_FULL && pl.rne_packed));
@@ -884,24 +905,16 @@ int lba_describe_plan_batched(int64_t batch, int64_t M, int64_t N, int64_t K, co
                             : (pl.pq == PQ_MASK_SAT ? "cut_sat" : (pl.pq == PQ_MASK ? "cut" : "none")));
   if (tile == TILE_PAIR) {
     if (buf && buf_len)
-      std::snprintf(buf, buf_len, "tile=64x64x%d pair micro=4x8 q=%s pq=%s kernel=%s order=%s load=%s grid=%lldx%lld", BK,
+      std::snprintf(buf, buf_len, "tile=64x64x%d pair micro=4x8 q=%s pq=%s kernel=%s order=%s load=%s grid=%lldx%lld%s", BK,
                     kQmName[pl.qm], pq, kern, kOrdName[pl.ord], kLdName[load], (long long)(2 * ((M + 63) / 64)),
-                    (long long)((N + 63) / 64));
-    return LBA_OK;
-  }
-  if (tile >= TILE_SPLIT) {
-    const TileInfo t = small_tile(tile);
-    if (buf && buf_len)
-      std::snprintf(buf, buf_len, "tile=%dx%dx%d %s micro=%dx%d q=%s pq=%s kernel=%s order=%s load=%s grid=%lldx%lld", t.bm, t.bn, BK,
-                    tile >= TILE_CHAIN ? "chain" : "split", t.tm, t.tn, kQmName[pl.qm], pq, kern, kOrdName[pl.ord], kLdName[load],
-                    (long long)((M + t.bm - 1) / t.bm), (long long)((N + t.bn - 1) / t.bn));
+                    (long long)((N + 63) / 64), by);
     return LBA_OK;
   }
   const TileInfo ti = tile_info(tile);
   if (buf && buf_len)
-    std::snprintf(buf, buf_len, "tile=%dx%dx%d micro=%dx%d q=%s pq=%s kernel=%s order=%s load=%s grid=%lldx%lld", ti.bm, ti.bn,
+    std::snprintf(buf, buf_len, "tile=%dx%dx%d micro=%dx%d q=%s pq=%s kernel=%s order=%s load=%s grid=%lldx%lld%s", ti.bm, ti.bn,
                   BK, ti.tm, ti.tn, kQmName[pl.qm], pq, kern, kOrdName[pl.ord], kLdName[load],
-                  (long long)((M + ti.bm - 1) / ti.bm), (long long)((N + ti.bn - 1) / ti.bn));
+                  (long long)((M + ti.bm - 1) / ti.bm), (long long)((N + ti.bn - 1) / ti.bn), by);
   return LBA_OK;
 }
 
