@@ -73,7 +73,8 @@ constexpr InputInfo kM4E3 = {248.0 * 248.0, 16, -8, 0, 10, 0};
 struct Plan {
   int qm, ord;
   float dec_a, dec_b, c, un1, un2;
-  float pk_a, pk_b, nrm_scale, inv_top;
+  float pk_a, pk_b, pk_a0, nrm_scale, inv_top;
+  int first_plain;
   float clamp_lim, slab_factor, fold_factor;
   int pq, rne_packed;
   float acc_k1, acc_k2, prod_k1, prod_k2;
@@ -315,6 +316,16 @@ int make_plan(const lba_fmt* pf, const lba_fmt* af, int order, int chunk, int64_
     pl->rne_packed = !ok ? 0 : (af->man_bits == 7 && order == LBA_ORDER_CHUNKED && chunk == BK && K > BK) ? 2 : 1;
   }
 
+  // ---- first step of a chunk (see Problem::first_plain).  A nearest-even cut of the product must see the flush of Q_prod
+  // first, and a saturation of Q_prod its scaling: those keep the general form.
+  {
+    const int prod_bits = pf->man_bits + 1 < in.product_bits ? pf->man_bits + 1 : in.product_bits;
+    const int s0 = sx + (ka - kp);
+    pl->first_plain = !p_sat && !(nearest && p_round) && prod_bits <= af->man_bits + 1 &&
+                      (!p_flush || (a_flush && af->bias <= pf->bias)) && s0 - 9 >= -126 && s0 + 9 <= 126;
+    pl->pk_a0 = pl->first_plain ? (float)std::ldexp(1.0, s0) : pl->pk_a;
+  }
+
   // ---- fused product and sum: Q_prod must be the identity on every reachable product (no cut, no saturation, no
   // product under R_UF_prod), and the rescaled B operand must stay a normal binary32 number
   {
@@ -366,7 +377,7 @@ const TileCost kCost[7][COST_TILES] = {
     {{0.02, 3.314, 5.3, 0.87}, {0.98, 1.785, 3.8, 0.92}, {0.88, 0.867, 4.3, 1}, {0.71, 0.261, 3.1, 1}, {0, 0, 0, 0}, {0.02, 0.138, 3.4, 1}, {0, 0, 0, 0}},  // floor, sequential
     {{0.86, 3.66, 5.8, 0.84}, {1.14, 1.878, 3.5, 0.96}, {0.94, 0.931, 4, 1}, {0.73, 0.28, 3.1, 1}, {1.8, 1.079, 3.4, 1}, {0, 1.863, 2.4, 0.57}, {1.49, 2.437, 2.4, 0.85}},  // floor, chunks of 16
     {{3.81, 6.691, 3, 1}, {3.08, 3.613, 1.9, 1}, {2.15, 1.822, 3.7, 1}, {1.65, 0.538, 2.2, 0.69}, {0, 0, 0, 0}, {0, 0.206, 3.9, 0.85}, {0, 0, 0, 0}},  // floor with product cut, sequential
-    {{2.87, 5.191, 6, 1}, {1.78, 2.756, 3.7, 0.97}, {1.76, 1.4, 4.4, 0.97}, {1.03, 0.394, 3.4, 0.97}, {2.86, 1.551, 3.2, 0.62}, {0, 2.736, 2.6, 0.82}, {2.42, 4.412, 2.9, 0.92}},  // floor with product cut, chunks of 16
+    {{2.87, 5.191, 6, 1}, {1.78, 2.756, 3.7, 0.97}, {1.76, 1.37, 4.4, 0.97}, {1.03, 0.394, 3.4, 0.97}, {2.86, 1.551, 3.2, 0.62}, {0, 2.736, 2.6, 0.82}, {2.42, 4.412, 2.9, 0.92}},  // floor with product cut, chunks of 16
     {{1.9, 4.724, 4.7, 0.98}, {1.49, 2.478, 3.2, 1}, {1.2, 1.277, 2.9, 1}, {0.95, 0.354, 2.1, 1}, {0, 0, 0, 0}, {0.24, 0.145, 2.5, 0.99}, {0, 0, 0, 0}},  // nearest-even, sequential
     {{0.08, 5.151, 4.6, 1}, {0.01, 2.783, 3.2, 1}, {1.25, 1.317, 3.5, 1}, {0.97, 0.365, 3.5, 1}, {0, 0, 0, 0}, {0.01, 1.993, 2.6, 0.68}, {1.8, 2.967, 2.7, 0.9}},  // nearest-even, chunks of 16
     {{0, 4.75, 4.2, 1}, {0.05, 2.575, 3.3, 1}, {1.29, 1.14, 3.9, 1}, {0.95, 0.323, 3, 1}, {0, 0, 0, 0}, {0, 1.972, 2.6, 0.5}, {1.98, 2.766, 2.5, 0.92}},  // nearest-even through bfloat16, chunks of 16
@@ -456,6 +467,8 @@ void apply_plan(Problem* p, const Plan& pl) {
   p->chunk = pl.chunk;
   p->pk_a = pl.pk_a;
   p->pk_b = pl.pk_b;
+  p->pk_a0 = pl.pk_a0;
+  p->first_plain = pl.first_plain;
   p->nrm_scale = pl.nrm_scale;
   p->inv_top = pl.inv_top;
   p->clamp_lim = pl.clamp_lim;
@@ -500,7 +513,8 @@ int run(const Problem& p, const Plan& pl, int load, cudaStream_t stream) {
   if (pl.fused && pl.ord != ORD_CHUNK_ANY) {  // the plain packed tiles have the fused variant
     Problem q = p;
     q.pq = PQ_FUSED;
-    q.pk_b = pl.pk_b_fused;
+    q.pk_b = pl.pk_b_fused;  // carries the accumulator's scaling in every step
+    q.pk_a0 = pl.pk_a;
     const cudaError_t e = kLaunch[pl.qm][pl.ord](tile, load, q, stream);
     return e == cudaSuccess ? LBA_OK : cuda_fail(e);
   }

@@ -72,6 +72,11 @@ struct Problem {
   int chunk;           // ORD_CHUNK_ANY
   // packed floor kernel only
   float pk_a, pk_b;    // 2^sx, 2^sw: decoded value -> product-carrier operand
+  // chunk-16 order: 1 if the first step of a chunk, Q_acc(Q_prod(x w) + 0), is the (cut) product alone: it has no more
+  // significant bits than the accumulator and is flushed by Q_acc wherever Q_prod flushes it.  A's first operand of
+  // every chunk then carries the accumulator's scaling (pk_a0), and the step is one multiplication without a mask.
+  int first_plain;
+  float pk_a0;
   float nrm_scale;     // 2^-(e_max_acc + 1), or 0 when the accumulator cannot saturate
   float inv_top;       // accumulator carrier -> fraction of 2^(e_max_acc + 1)
   int pq;              // PackedProd: what Q_prod does beyond the flush
@@ -934,7 +939,8 @@ __host__ __device__ constexpr int packed_tmem_cols() {
 }
 
 // the 8x8 micro-tile is held to 128 registers (two CTAs of 256 threads per SM) wherever the second-level
-// sums are not in registers; so is the byte-wise loader, whose sixteen loads in flight would otherwise
+// sums are not in registers; so is the 4x8 one in chunk-16 order (two registers more had cost it a quarter of its CTAs),
+// and the byte-wise loader, whose sixteen loads in flight would otherwise
 // cost fifty registers and half the resident CTAs
 // PQ: what Q_prod has to do beyond the flush (the host proves which cases are reachable): nothing, cut the
 // mantissa (M_prod < 7), or cut and saturate (448^2 >= R_OF_prod)
@@ -964,7 +970,7 @@ enum PackedProd { PQ_NONE = 0, PQ_MASK = 1, PQ_MASK_SAT = 2, PQ_FUSED = 3 };
 // This doubles the CTAs of a small problem without splitting any sequential chain, and both CTAs do the same work.
 template <int BM, int BN, int TM, int TN, int PQ, int RNE, int ORD, int LD, int STE = 0, int CL = 1, bool H16 = false>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN),
-                                  ((TM * TN == 64 && ORD != ORD_CHUNK_SLAB && !RNE) ||
+                                  ((TM * TN == 64 && ORD != ORD_CHUNK_SLAB && !RNE) || (TM * TN == 32 && ORD == ORD_CHUNK16 && !RNE) ||
                                    ((LD == LD_CONV_ANY || LD == LD_GEMM_ROWS || STE != 0) && !RNE && ORD != ORD_CHUNK_SLAB))
                                       ? 512 / ((BM / TM) * (BN / TN)) : 1)
     lba_contract_packed_kernel(const Problem p) {
@@ -1021,7 +1027,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
       const int r = tid + l * NT;
       if (r < ROWS) {  // uniform per warp: BM, BN and NT are multiples of 32
         const bool is_a = r < BM;
-        const float mul = is_a ? p.pk_a : p.pk_b;
+        const float mul = is_a ? p.pk_a : p.pk_b, mul_first = CH16 && is_a ? p.pk_a0 : mul;
         const uint4 row = loader.take(p, l, slab, raw[l]);
         const uint32_t w4[4] = {row.x, row.y, row.z, row.w};
         float n2 = 0.0f;
@@ -1038,7 +1044,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             n2 = fma_rn(v[j], v[j], n2);
-            const float s = mul_ieee(v[j], mul);
+            const float s = mul_ieee(v[j], q + j == 0 ? mul_first : mul);
             if (is_a) As[buf][q * 4 + j][r] = make_float2(s, s);
             else Bs[buf][q * 4 + j][r - BM] = s;
           }
@@ -1069,6 +1075,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
   const float sat = p.qa.sat;
   const uint32_t pmask = p.qp.mask;
   const float psat = p.qp.sat;
+  const bool first_plain = p.first_plain;
   const u64 acc_k1 = pack2(p.acc_k1, p.acc_k1), acc_k2 = pack2(p.acc_k2, p.acc_k2);
   const u64 prod_k1 = pack2(p.prod_k1, p.prod_k1), prod_k2 = pack2(p.prod_k2, p.prod_k2);
   auto rne_acc = [&](u64 v) -> u64 {
@@ -1129,6 +1136,25 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
           }
           return pr;
         };
+        if (CH16 && kk == 0 && first_plain) {  // see Problem::first_plain
+#pragma unroll
+          for (int i = 0; i < TM; ++i)
+#pragma unroll
+            for (int j = 0; j < PN; ++j) {
+              const u64 t = product(a2[i], b2[j], j);
+              acc1[i][j] = t;
+              if constexpr (CLAMP) {
+                float lo, hi;
+                unpack2(t, lo, hi);
+                if constexpr (REC) {
+                  if (fabsf(lo) < sat) hb[i][j] |= 1u;
+                  if (fabsf(hi) < sat) hb[i][j] |= 0x10000u;
+                }
+                acc1[i][j] = pack2(clamp_mag(lo, sat), clamp_mag(hi, sat));
+              }
+            }
+          continue;
+        }
         if constexpr (PQ == PQ_FUSED) {
 #pragma unroll
           for (int i = 0; i < TM; ++i)
@@ -1185,10 +1211,21 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
         continue;
       }
       if constexpr (RNE) {
+      const bool plain = CH16 && kk == 0 && first_plain;  // see Problem::first_plain
 #pragma unroll
       for (int i = 0; i < TM; ++i)
 #pragma unroll
         for (int j = 0; j < PN; ++j) {
+          if ((PQ == PQ_NONE || PQ == PQ_FUSED) && plain) {
+            u64 t = mul2_ftz(b2[j], a2[i]);
+            if (CLAMP) {
+              float lo, hi;
+              unpack2(t, lo, hi);
+              t = pack2(clamp_mag(lo, sat), clamp_mag(hi, sat));
+            }
+            acc1[i][j] = t;
+            continue;
+          }
           // nearest-even (the floor path has left the loop body above).  The sum is formed by one packed FMA rounded to
           // nearest: whenever that rounding is inexact the smaller operand lies so far below the larger one (which is
           // on the accumulator's grid) that neither the exact sum nor its binary32 image can reach a tie of the M-bit

@@ -87,3 +87,22 @@ def test_small_problem_kernels(tile, name):
             assert (got[z].view(np.uint32) == want.view(np.uint32)).all()
     finally:
         lba.set_tile_override(-1)
+
+
+@pytest.mark.parametrize("name,fmts", [
+    ("plain", code_domain_formats(7, 4)), ("fused", code_domain_formats(10, 6)), ("cut", code_domain_formats(4, 4)),
+    ("product_wider", (LbaFormat(7, 4, -2), LbaFormat(5, 4, -4))), ("flush_not_shared", (LbaFormat(7, 4, -2), LbaFormat(7, 4, 0))),
+    ("no_acc_flush", (LbaFormat(7, 4, -2), LbaFormat(7, 4, -4, 0, 0))), ("saturating", (LbaFormat(7, 4, 12), LbaFormat(7, 4, 10))),
+    ("rne", code_domain_formats(7, 4, 1)), ("rne_cut", code_domain_formats(4, 4, 1))], ids=lambda v: v if isinstance(v, str) else "")
+@pytest.mark.parametrize("tile", [0, 2, 5])
+def test_first_step_of_a_chunk(tile, name, fmts):
+    # chunks whose first product is tiny, short or large: the step that may leave out the mask and one multiplication
+    A, B = synth.random_codes((65, 80), 5), synth.random_codes((70, 80), 6)
+    A[:40, ::16] = torch.arange(40, dtype=torch.uint8)[:, None]      # subnormal and small codes
+    B[:30, ::16] = torch.arange(1, 31, dtype=torch.uint8)[:, None]
+    lba.set_tile_override(tile)
+    try:
+        check_gemm(A, B, *fmts, CHK, what=name)
+        check_gemm(A[:, :77].contiguous(), B[:, :77].contiguous(), *fmts, CHK, what=name)
+    finally:
+        lba.set_tile_override(-1)
