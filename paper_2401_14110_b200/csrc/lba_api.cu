@@ -24,9 +24,9 @@ template <> cudaError_t launch_small<0>(int, int, const Problem&, cudaStream_t);
 template <> cudaError_t launch_small<1>(int, int, const Problem&, cudaStream_t);
 template <> cudaError_t launch_small<2>(int, int, const Problem&, cudaStream_t);
 
-cudaError_t launch_last_overflow(int qm, int load, const Problem& p, cudaStream_t stream);
-cudaError_t launch_ste_mask(int qm, int ord, int diff, int load, const Problem& p, cudaStream_t stream);
-cudaError_t launch_ste_packed(int pq, int chunk16, int load, const Problem& p, cudaStream_t stream);
+cudaError_t launch_last_overflow(bool small, int qm, int load, const Problem& p, cudaStream_t stream);
+cudaError_t launch_ste_mask(bool small, int qm, int ord, int diff, int load, const Problem& p, cudaStream_t stream);
+cudaError_t launch_ste_packed(bool small, int pq, int chunk16, int load, const Problem& p, cudaStream_t stream);
 cudaError_t launch_fixed(int ord, int load, const Problem& p, cudaStream_t stream);
 cudaError_t launch_cluster_pair(int pq, int load, const Problem& p, cudaStream_t stream);
 
@@ -443,6 +443,28 @@ TileChoice choose_tile(int64_t M, int64_t N, int64_t K, int64_t batch, const Pla
   return best;
 }
 
+// Tile of the mask and last-overflow passes: 64x64, or 32x32 where that is faster by the same model (override 2 and 7
+// force one of them).  Measured on fourteen shapes from 64 x 64 x 96 to 4096 x 3072 x 768; 512^3, 64x64 against 32x32: overflow
+// masks 48 / 34 us sequential, 73 / 43 us chunked, difference masks 119 / 104 and 128 / 141, last overflow 90 / 57 us;
+// 4096 x 3072 x 768: 965 / 1124, 1073 / 1311, 2955 / 3310, 3245 / 3888, 2343 / 2429.
+enum SteKernel { STE_OF_SEQ = 0, STE_OF_CHUNK = 1, STE_DIFF_SEQ = 2, STE_DIFF_CHUNK = 3, STE_TRACK_OF = 4 };
+bool small_ste_tile(int64_t M, int64_t N, int64_t K, SteKernel kernel) {
+  const int forced = g_tile_override.load(std::memory_order_relaxed);
+  if (forced == 2 || forced == 7) return forced == 7;
+  static const TileCost kSte[5][2] = {{{1.38, 0.965, 4, 1}, {0.93, 0.297, 3, 1}}, {{2.15, 1.08, 4, 1}, {1.22, 0.345, 3, 1}},
+                                      {{2.7, 2.95, 4, 1}, {2.65, 0.95, 3, 1}},    {{2.9, 3.2, 4, 1}, {3.5, 1.5, 3, 1}},
+                                      {{2.0, 2.33, 4, 1}, {1.6, 0.65, 3, 1}}};
+  const double slabs = std::fmax(1.0, (double)((K + BK - 1) / BK));
+  double t[2];
+  for (int i = 0; i < 2; ++i) {
+    const TileCost& c = kSte[kernel][i];
+    const int64_t e = i == 0 ? 64 : 32;
+    const double x = (double)((M + e - 1) / e) * (double)((N + e - 1) / e) / sm_count(), q = std::fmax(1.0, std::ceil(x));
+    t[i] = c.base + slabs * std::cbrt(c.L * c.L * c.L + c.b * q * c.b * q * c.b * q);
+  }
+  return t[1] < t[0] && (N + 31) / 32 <= 65535;
+}
+
 int fill_scales(Problem* p, const float* sa, int sa_len, const float* sb, int sb_len, const float* bias) {
   if (!sa || !sb) return LBA_ERR_NULL;
   if (!(sa_len == 1 || (int64_t)sa_len == p->M) || !(sb_len == 1 || (int64_t)sb_len == p->N))
@@ -674,7 +696,7 @@ int lba_gemm_last_overflow(const uint8_t* A, const uint8_t* B, int64_t M, int64_
   p.out = reinterpret_cast<float*>(last);
   apply_plan(&p, pl);
   const bool vec = K % BK == 0 && aligned16(A) && aligned16(B);
-  const cudaError_t e = launch_last_overflow(pl.qm, vec ? LD_GEMM_VEC : LD_GEMM_ROWS, p, (cudaStream_t)stream);
+  const cudaError_t e = launch_last_overflow(small_ste_tile(M, N, K, STE_TRACK_OF), pl.qm, vec ? LD_GEMM_VEC : LD_GEMM_ROWS, p, (cudaStream_t)stream);
   return e == cudaSuccess ? LBA_OK : cuda_fail(e);
 }
 
@@ -744,8 +766,8 @@ int lba_gemm_ste_mask(const uint8_t* A, const uint8_t* B, int64_t M, int64_t N, 
   // the overflow masks in sequential and chunk-16 order come from the packed kernel (tile override 3 keeps the
   // scalar tracking kernel, for tests and comparisons); everything else from the scalar one
   const bool packed = ste == LBA_STE_OF && (!chunked || chunk == BK) && g_tile_override.load(std::memory_order_relaxed) != 3;
-  const cudaError_t e = packed ? launch_ste_packed(pl.qm == QM_FLOOR_FAST ? PQ_NONE : pl.pq, chunked ? 1 : 0, load, p, (cudaStream_t)stream)
-                               : launch_ste_mask(pl.qm, ord, ste == LBA_STE_DIFF, load, p, (cudaStream_t)stream);
+  const cudaError_t e = packed ? launch_ste_packed(small_ste_tile(M, N, K, chunked ? STE_OF_CHUNK : STE_OF_SEQ), pl.qm == QM_FLOOR_FAST ? PQ_NONE : pl.pq, chunked ? 1 : 0, load, p, (cudaStream_t)stream)
+                               : launch_ste_mask(small_ste_tile(M, N, K, ste != LBA_STE_DIFF ? STE_TRACK_OF : chunked ? STE_DIFF_CHUNK : STE_DIFF_SEQ), pl.qm, ord, ste == LBA_STE_DIFF, load, p, (cudaStream_t)stream);
   return e == cudaSuccess ? LBA_OK : cuda_fail(e);
 }
 

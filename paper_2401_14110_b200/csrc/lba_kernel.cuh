@@ -974,7 +974,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
                                    ((LD == LD_CONV_ANY || LD == LD_GEMM_ROWS || STE != 0) && !RNE && ORD != ORD_CHUNK_SLAB))
                                       ? 512 / ((BM / TM) * (BN / TN)) : 1)
     lba_contract_packed_kernel(const Problem p) {
-  static_assert(STE == 0 || (!RNE && TM == 4 && TN == 8 && (ORD == ORD_SEQ || ORD == ORD_CHUNK16)), "mask variant");
+  static_assert(STE == 0 || (!RNE && TM == 4 && (ORD == ORD_SEQ || ORD == ORD_CHUNK16)), "mask variant");
   static_assert(CL == 1 || LD == LD_GEMM_VEC || LD == LD_CONV_VEC, "a CTA of the pair skips slabs");
   static_assert(CL == 1 || (CL == 2 && !RNE && STE == 0 && ORD == ORD_CHUNK16 && TM == 4), "cluster variant");
   constexpr int NT = (BM / TM) * (BN / TN);

@@ -106,3 +106,27 @@ def test_first_step_of_a_chunk(tile, name, fmts):
         check_gemm(A[:, :77].contiguous(), B[:, :77].contiguous(), *fmts, CHK, what=name)
     finally:
         lba.set_tile_override(-1)
+
+
+@pytest.mark.parametrize("tile", [2, 7])
+@pytest.mark.parametrize("name", ["m7e4", "m4e4", "m10e6"])
+def test_mask_passes_on_both_tiles(tile, name):
+    # edges of the tiles, words of the masks cut short, saturating data
+    prod, acc = SMALL_FORMATS[name]
+    t, a = prod.as_tuple(), acc.as_tuple()
+    lba.set_tile_override(tile)
+    try:
+        for (M, N, K) in ((1, 1, 1), (33, 31, 40), (65, 70, 545), (30, 100, 528)):
+            A, B = synth.random_codes((M, K), 3 * M + K), synth.random_codes((N, K), 5 * N + K)
+            if K == 545:
+                A, B = A & 0x7F, B & 0x7F
+            g = lambda x: x.cpu().numpy().view(np.uint32)
+            for order in (SEQ, CHK):
+                for kind, e1, e2 in ((lba.STE_OF, 0.0, 0.0), (lba.STE_DIFF, 4.0, 2.0 ** -7)):
+                    m1, m2 = lba.lba_gemm_ste_mask(A.to(DEV), B.to(DEV), prod, acc, order, 16, kind, e1, e2)
+                    w1, w2 = orc.gemm_ste_mask(A.numpy(), B.numpy(), t, a, order, 16, kind, e1, e2)
+                    assert (g(m1) == w1).all() and (m2 is None or (g(m2) == w2).all()), (M, N, K, order, kind)
+            last = lba.lba_gemm_last_overflow(A.to(DEV), B.to(DEV), prod, acc).cpu().numpy()
+            assert (last == orc.gemm_last_overflow(A.numpy(), B.numpy(), t, a)).all(), (M, N, K)
+    finally:
+        lba.set_tile_override(-1)
