@@ -451,6 +451,7 @@ enum SteKernel { STE_OF_SEQ = 0, STE_OF_CHUNK = 1, STE_DIFF_SEQ = 2, STE_DIFF_CH
 bool small_ste_tile(int64_t M, int64_t N, int64_t K, SteKernel kernel) {
   const int forced = g_tile_override.load(std::memory_order_relaxed);
   if (forced == 2 || forced == 7) return forced == 7;
+  if (kernel == STE_DIFF_CHUNK) return false;  // 118 against 127 us at best (128 x 256 x 512), 41 against 39 (418 x 160 x 144)
   static const TileCost kSte[5][2] = {{{1.38, 0.965, 4, 1}, {0.93, 0.297, 3, 1}}, {{2.15, 1.08, 4, 1}, {1.22, 0.345, 3, 1}},
                                       {{2.7, 2.95, 4, 1}, {2.65, 0.95, 3, 1}},    {{2.9, 3.2, 4, 1}, {3.5, 1.5, 3, 1}},
                                       {{2.0, 2.33, 4, 1}, {1.6, 0.65, 3, 1}}};
