@@ -386,6 +386,13 @@ const TileCost kCost[7][COST_TILES] = {
 // per output wins as long as it keeps its registers
 const TileCost kCostConvAny[TILE_COUNT] = {{6, 10.4, 4, 0.5}, {2, 2.85, 4, 0.5}, {1.2, 1.64, 4, 0.5}, {0.8, 0.49, 4, 0.5}};
 
+// a launch has at most 2^31 - 1 rows and 65535 columns of CTAs of bm x bn outputs
+bool grid_fits(int64_t M, int64_t N, int bm, int bn, int ctas_per_tile = 1) {
+  return (N + bn - 1) / bn <= 65535 && ctas_per_tile * ((M + bm - 1) / bm) <= 2147483647LL;
+}
+
+// A tile whose grid cannot be launched is not a candidate; where none can, `run` is one of them all the same and the
+// caller, which checks it with grid_fits, refuses the shape.
 struct TileChoice {
   int packed;  // the fastest of the tiles of the packed and generic kernels (TILE_PAIR among them)
   int run;     // the tile that runs: `packed`, or one of the small-problem kernels where that is faster
@@ -394,9 +401,8 @@ struct TileChoice {
 TileChoice choose_tile(int64_t M, int64_t N, int64_t K, int64_t batch, const Plan& pl, int load) {
   const int qm = pl.qm, ord = pl.ord;
   const bool vec = load == LD_GEMM_VEC || load == LD_CONV_VEC, floor = qm == QM_FLOOR_FAST || qm == QM_FLOOR_FULL;
-  const bool pair_ok = ord == ORD_CHUNK16 && floor && vec && 2 * ((M + 63) / 64) <= 2147483647LL;
-  const bool small_ok = load != LD_CONV_ANY && (floor || (qm == QM_RNE_FULL && pl.rne_packed)) && N <= 16 * 65535LL &&
-                        M <= 16 * 2147483647LL;
+  const bool pair_ok = ord == ORD_CHUNK16 && floor && vec && grid_fits(M, N, 64, 64, 2);
+  const bool small_ok = load != LD_CONV_ANY && (floor || (qm == QM_RNE_FULL && pl.rne_packed)) && grid_fits(M, N, 16, 16);
   const bool split_ok = small_ok && ord == ORD_CHUNK16, chain_ok = small_ok && ord == ORD_SEQ;
   const int forced = g_tile_override.load(std::memory_order_relaxed);
   if (forced >= 0 && forced < TILE_COUNT) return {forced, forced};
@@ -416,6 +422,7 @@ TileChoice choose_tile(int64_t M, int64_t N, int64_t K, int64_t batch, const Pla
   double least = 1e300;
   for (int t = 0; t < TILE_COUNT; ++t) {
     const TileInfo ti = tile_info(t);
+    if (!grid_fits(M, N, ti.bm, ti.bn)) continue;
     const double c = time(load == LD_CONV_ANY ? kCostConvAny[t] : kCost[row][t], ti.bm, ti.bn, 1.0, 1.0);
     if (c < least) {
       least = c;
@@ -515,24 +522,23 @@ int run(const Problem& p, const Plan& pl, int load, cudaStream_t stream) {
   if (p.M == 0 || p.N == 0 || p.batch == 0) return LBA_OK;
   if (p.batch > 65535) return LBA_ERR_SHAPE;
   if (pl.fixed) {  // Eq. 1: the integer kernel, one tile shape
-    if ((p.N + 63) / 64 > 65535) return LBA_ERR_SHAPE;
+    if (!grid_fits(p.M, p.N, 64, 64)) return LBA_ERR_SHAPE;
     const cudaError_t e = launch_fixed(pl.ord, load, p, stream);
     return e == cudaSuccess ? LBA_OK : cuda_fail(e);
   }
   const int tile = choose_tile(p.M, p.N, p.K, p.batch, pl, load).run;
-  if (tile >= TILE_SPLIT) {  // choose_tile keeps the grid within its limits
+  if (tile >= TILE_SPLIT) {  // choose_tile keeps the grid of these and of the pair within its limits
     const int rne = pl.qm == QM_RNE_FULL ? pl.rne_packed : 0;
     const cudaError_t e = rne == 0 ? launch_small<0>(tile, load, p, stream)
                                    : rne == 1 ? launch_small<1>(tile, load, p, stream) : launch_small<2>(tile, load, p, stream);
     return e == cudaSuccess ? LBA_OK : cuda_fail(e);
   }
   if (tile == TILE_PAIR) {
-    if ((p.N + 63) / 64 > 65535) return LBA_ERR_SHAPE;
     const cudaError_t e = launch_cluster_pair(pl.qm == QM_FLOOR_FAST ? PQ_NONE : pl.pq, load, p, stream);
     return e == cudaSuccess ? LBA_OK : cuda_fail(e);
   }
   const TileInfo ti = tile_info(tile);
-  if ((p.N + ti.bn - 1) / ti.bn > 65535 || (p.M + ti.bm - 1) / ti.bm > 2147483647LL) return LBA_ERR_SHAPE;
+  if (!grid_fits(p.M, p.N, ti.bm, ti.bn)) return LBA_ERR_SHAPE;
   if (pl.fused && pl.ord != ORD_CHUNK_ANY) {  // the plain packed tiles have the fused variant
     Problem q = p;
     q.pq = PQ_FUSED;
@@ -925,12 +931,13 @@ int lba_describe_plan_batched(int64_t batch, int64_t M, int64_t N, int64_t K, co
   if (st != LBA_OK) return st;
   const int load = vec_ok ? (is_conv ? LD_CONV_VEC : LD_GEMM_VEC) : (is_conv ? LD_CONV_ANY : LD_GEMM_ROWS);
   if (pl.fixed) {
+    if (!grid_fits(M, N, 64, 64)) return LBA_ERR_SHAPE;
     if (buf && buf_len)
       std::snprintf(buf, buf_len, "tile=64x64x%d micro=4x4 q=fixed order=%s load=%s grid=%lldx%lld", BK, kOrdName[pl.ord],
                     kLdName[load], (long long)((M + 63) / 64), (long long)((N + 63) / 64));
     return LBA_OK;
   }
-  const TileChoice choice = choose_tile(M > 0 ? M : 1, N > 0 ? N : 1, K, batch, pl, load);
+  const TileChoice choice = choose_tile(M > 0 ? M : 1, N > 0 ? N : 1, K, batch < 65535 ? batch : 65535, pl, load);  // a launch takes 65535 problems
   const int tile = choice.packed;
   const char* const by = choice.run == choice.packed ? "" : choice.run == TILE_SPLIT ? " by=split16x16" : choice.run == TILE_CHAIN ? " by=chain16x16" : " by=split32x32";
   // which kernel runs and what Q_prod costs there beyond the flush
@@ -948,6 +955,7 @@ int lba_describe_plan_batched(int64_t batch, int64_t M, int64_t N, int64_t K, co
     return LBA_OK;
   }
   const TileInfo ti = tile_info(tile);
+  if (choice.run == tile && !grid_fits(M, N, ti.bm, ti.bn)) return LBA_ERR_SHAPE;
   if (buf && buf_len)
     std::snprintf(buf, buf_len, "tile=%dx%dx%d micro=%dx%d q=%s pq=%s kernel=%s order=%s load=%s grid=%lldx%lld%s", ti.bm, ti.bn,
                   BK, ti.tm, ti.tn, kQmName[pl.qm], pq, kern, kOrdName[pl.ord], kLdName[load],

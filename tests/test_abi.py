@@ -123,3 +123,26 @@ def test_describe_plan_for_batched_calls():
     assert lba.describe_plan(128, 128, 64, *f, CHK, 16, batch=384).startswith("tile=64x64x16 micro=4x8")
     with pytest.raises(lba.LbaError):
         lba.describe_plan(128, 128, 64, *f, CHK, 16, batch=0)
+
+
+@pytest.mark.parametrize("fmts", [code_domain_formats(7, 4), code_domain_formats(4, 4), code_domain_formats(7, 4, rounding=1),
+                                  code_domain_formats(12, 5, rounding=1)], ids=["floor", "cut", "nearest", "nearest_generic"])
+@pytest.mark.parametrize("order,chunk", [(SEQ, 16), (CHK, 16), (CHK, 24), (CHK, 32)])
+def test_wide_outputs_get_a_tile_that_can_be_launched(fmts, order, chunk):
+    # a grid has at most 65535 columns of CTAs: up to 65535 * 128 columns there is a tile that fits, beyond there is none
+    for N in (16 * 65535 + 1, 32 * 65535, 32 * 65535 + 1, 64 * 65535, 64 * 65535 + 1, 128 * 65535):
+        for M in (1, 17, 80, 96, 280):
+            for K in (64, 17):
+                plan = lba.describe_plan(M, N, K, *fmts, order, chunk, vec_ok=K % 16 == 0)
+                assert int(plan.split("grid=")[1].split()[0].split("x")[1]) <= 65535 or "by=" in plan, (M, N, K, plan)
+    with pytest.raises(lba.LbaError) as e:
+        lba.describe_plan(4, 128 * 65535 + 1, 64, *fmts, order, chunk)
+    assert e.value.status == -2
+
+
+def test_wide_outputs_of_the_fixed_point_kernel_are_refused_by_the_plan_too():
+    f = LbaFormat(16, 0, -4, 0, 0)
+    assert "q=fixed" in lba.describe_plan(4, 64 * 65535, 64, f, f)
+    with pytest.raises(lba.LbaError) as e:
+        lba.describe_plan(4, 64 * 65535 + 1, 64, f, f)
+    assert e.value.status == -2
