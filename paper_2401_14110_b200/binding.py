@@ -5,7 +5,6 @@ the computation runs in the CUDA kernels behind the C entry points.  There is no
 library is missing, or a call returns an error, an exception is raised.
 """
 import ctypes as C
-import functools
 import os
 
 import torch
@@ -86,15 +85,25 @@ def _fmt(f):
     return _Fmt(*[int(v) for v in t])
 
 
-@functools.lru_cache(maxsize=256)
-def _fmt_ref_of(values):
-    return C.byref(_Fmt(*[int(v) for v in values]))
+_fmt_refs = {}   # five Python integers -> pointer to their C struct, which the library only reads
 
 
 def _fmt_ref(f):
-    """Pointer to the format's C struct, which the library only reads (one struct per value: building it anew took a fifth of
-    a small call's 17 to 21 us on the host)."""
-    return _fmt_ref_of(f.as_tuple() if isinstance(f, LbaFormat) else tuple(f))
+    """Pointer to the format's C struct (building it anew took a fifth of a small call's 17 to 21 us on the host).  Only tuples
+    of Python integers are kept: the fields may also be arrays or tensors of one element, which do not hash by value."""
+    t = f.as_tuple() if isinstance(f, LbaFormat) else tuple(f)
+    try:
+        ref = _fmt_refs.get(t)
+    except TypeError:
+        ref = None
+    if ref is None:
+        t = tuple(int(v) for v in t)
+        ref = _fmt_refs.get(t)
+        if ref is None:
+            if len(_fmt_refs) >= 256:
+                _fmt_refs.clear()
+            ref = _fmt_refs[t] = C.byref(_Fmt(*t))
+    return ref
 
 
 def _stream(stream):

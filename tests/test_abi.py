@@ -4,7 +4,9 @@ import ctypes as C
 import os
 import re
 
+import numpy as np
 import pytest
+import torch
 
 from paper_2401_14110_b200 import binding as lba
 from paper_2401_14110_b200 import LbaFormat, code_domain_formats, ORDER_CHUNKED as CHK, ORDER_SEQUENTIAL as SEQ
@@ -146,3 +148,16 @@ def test_wide_outputs_of_the_fixed_point_kernel_are_refused_by_the_plan_too():
     with pytest.raises(lba.LbaError) as e:
         lba.describe_plan(4, 64 * 65535 + 1, 64, f, f)
     assert e.value.status == -2
+
+
+@pytest.mark.parametrize("box", [np.array, torch.tensor, np.int32, float], ids=["array", "tensor", "int32", "float"])
+def test_format_fields_are_read_by_value_at_every_call(box):
+    p, a = code_domain_formats(7, 4)
+    plan = lambda f: lba.describe_plan(512, 512, 512, f, a)
+    f = [box(v) for v in p.as_tuple()]
+    assert plan(f) == plan(p) == plan(LbaFormat(*f)) == plan(tuple(f))
+    if hasattr(f[0], "fill_"):
+        f[0].fill_(4)     # the same object, another value
+    else:
+        f[0] = box(4)
+    assert "pq=cut" in plan(f) and "pq=cut" in plan(LbaFormat(*f)) and "pq=none" in plan(p)
