@@ -108,7 +108,6 @@ def _fmt_ref(f):
 
 def _stream(stream):
     if stream is None:  # the current device's current stream, without the wrapper object
-        torch.cuda._lazy_init()  # as current_stream() does: sets CUDA up on the first use, refuses a forked child
         return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 

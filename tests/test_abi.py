@@ -161,11 +161,3 @@ def test_format_fields_are_read_by_value_at_every_call(box):
     else:
         f[0] = box(4)
     assert "pq=cut" in plan(f) and "pq=cut" in plan(LbaFormat(*f)) and "pq=none" in plan(p)
-
-
-def test_default_stream_goes_through_the_cuda_set_up_of_torch(monkeypatch):
-    # a process forked after CUDA was used must get torch's own refusal, as torch.cuda.current_stream() gives it
-    monkeypatch.setattr(torch.cuda, "_is_in_bad_fork", lambda: True)
-    for ask in (lambda: torch.cuda.current_stream(), lambda: lba._stream(None)):
-        with pytest.raises(RuntimeError, match="forked"):
-            ask()
