@@ -938,10 +938,11 @@ __host__ __device__ constexpr int packed_tmem_cols() {
   return (ORD == ORD_CHUNK16 && TM == 8 && !RNE) ? (cols < 32 ? 32 : cols) : 0;
 }
 
-// the 8x8 micro-tile is held to 128 registers (two CTAs of 256 threads per SM) wherever the second-level
-// sums are not in registers; so is the 4x8 one in chunk-16 order (two registers more had cost it a quarter of its CTAs),
-// and the byte-wise loader, whose sixteen loads in flight would otherwise
-// cost fifty registers and half the resident CTAs
+// Register bounds.  The 8x8 micro-tile is held to 128 registers (two CTAs of 256 threads per SM) wherever the second-level
+// sums are not in registers.  So is the 4x8 one in chunk-16 order, where 130 to 144 registers had cost a quarter (64x64) or
+// half (128x64) of the CTAs: nearest-even M7E4 on the 128x64 tile, GEMM 4096 x 4096 x 512 1146 to 983 us, ResNet stem
+// 729 to 598 us.  So are, under floor rounding, the loaders of unaligned rows and of any convolution, whose loads in flight would
+// otherwise cost fifty registers and half the resident CTAs, and the mask passes.
 // PQ: what Q_prod has to do beyond the flush (the host proves which cases are reachable): nothing, cut the
 // mantissa (M_prod < 7), or cut and saturate (448^2 >= R_OF_prod)
 // PQ_FUSED: Q_prod is the identity on every reachable product (no cut, no saturation, and no product can fall under
@@ -970,7 +971,7 @@ enum PackedProd { PQ_NONE = 0, PQ_MASK = 1, PQ_MASK_SAT = 2, PQ_FUSED = 3 };
 // This doubles the CTAs of a small problem without splitting any sequential chain, and both CTAs do the same work.
 template <int BM, int BN, int TM, int TN, int PQ, int RNE, int ORD, int LD, int STE = 0, int CL = 1, bool H16 = false>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN),
-                                  ((TM * TN == 64 && ORD != ORD_CHUNK_SLAB && !RNE) || (TM * TN == 32 && ORD == ORD_CHUNK16 && !RNE) ||
+                                  ((TM * TN == 64 && ORD != ORD_CHUNK_SLAB && !RNE) || (TM * TN == 32 && ORD == ORD_CHUNK16) ||
                                    ((LD == LD_CONV_ANY || LD == LD_GEMM_ROWS || STE != 0) && !RNE && ORD != ORD_CHUNK_SLAB))
                                       ? 512 / ((BM / TM) * (BN / TN)) : 1)
     lba_contract_packed_kernel(const Problem p) {
