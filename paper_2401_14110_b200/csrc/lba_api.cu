@@ -367,21 +367,50 @@ int sm_count() {
 //   base + cbrt((rounds * L)^3 + (slabs / g * b * q)^3)   microseconds,
 // L: time of one round of a CTA that has the SM to itself (the latency of its chain of steps), b: time a round adds where the SM is
 // full, g: slabs of 16 k that a round takes, q: CTAs on the busiest SM, of whose rounding-up a share w counts (CTAs that are few on
-// their SM run faster).  The constants are fitted to 75 shapes per table (16 to 8192 rows and columns, K 64 to 4608, the layers of
-// ResNet-18, ResNet-50 and BERT among them), every tile timed on each: on average 0.1 to 1.3 % slower than the best tile of
-// each shape, where one table of relative rates lost 17 to 45 % because it knew no latency and no small tiles.
+// their SM run faster).  One row per kernel: rows shared between kernels had put the generic nearest-even kernel (M12E5) on the
+// 128x128 tile, 3.72 ms where 32x32 takes 2.08 (2048 x 1024 x 1024, sequential) and 13.5 ms where 128x64 takes 7.4
+// (4096 x 4096 x 512, chunks).  profiles/tile_times.txt holds the times that the constants are fitted to and what the choice
+// loses on them.
 struct TileCost { double L, b, base, w; };
 enum { COST_PAIR = 4, COST_SMALL = 5, COST_TILES = 7 };
-const TileCost kCost[7][COST_TILES] = {
+enum CostRow { ROW_SEQ = 0, ROW_CHUNK16 = 1, ROW_CUT_SEQ = 2, ROW_CUT_CHUNK16 = 3, ROW_RNE_SEQ = 4, ROW_RNE_CHUNK16 = 5, ROW_BF16_CHUNK16 = 6,
+               ROW_LONG = 7, ROW_CUT_LONG = 8, ROW_RNE_LONG = 9, ROW_ANY = 10, ROW_RNE_ANY = 11, ROW_GENERIC_SEQ = 12, ROW_GENERIC_LONG = 13,
+               ROW_WIDE_SEQ = 14, ROW_WIDE_LONG = 15, ROW_WIDE_ANY = 16, ROW_COUNT = 17 };
+const TileCost kCost[ROW_COUNT][COST_TILES] = {
     // 128x128, 128x64, 64x64, 32x32, pair, 16x16 chain (sequential) or split, 32x32 split
-    {{0.02, 3.314, 5.3, 0.87}, {0.98, 1.785, 3.8, 0.92}, {0.88, 0.867, 4.3, 1}, {0.71, 0.261, 3.1, 1}, {0, 0, 0, 0}, {0.02, 0.138, 3.4, 1}, {0, 0, 0, 0}},  // floor, sequential
-    {{0.86, 3.66, 5.8, 0.84}, {1.14, 1.878, 3.5, 0.96}, {0.94, 0.931, 4, 1}, {0.73, 0.28, 3.1, 1}, {1.8, 1.079, 3.4, 1}, {0, 1.863, 2.4, 0.57}, {1.49, 2.437, 2.4, 0.85}},  // floor, chunks of 16
-    {{3.81, 6.691, 3, 1}, {3.08, 3.613, 1.9, 1}, {2.15, 1.822, 3.7, 1}, {1.65, 0.538, 2.2, 0.69}, {0, 0, 0, 0}, {0, 0.206, 3.9, 0.85}, {0, 0, 0, 0}},  // floor with product cut, sequential
-    {{2.87, 5.191, 6, 1}, {1.78, 2.756, 3.7, 0.97}, {1.76, 1.37, 4.4, 0.97}, {1.03, 0.394, 3.4, 0.97}, {2.86, 1.551, 3.2, 0.62}, {0, 2.736, 2.6, 0.82}, {2.42, 4.412, 2.9, 0.92}},  // floor with product cut, chunks of 16
+    {{0.02, 3.314, 5.3, 0.87}, {0.98, 1.785, 3.8, 0.92}, {0.88, 0.867, 4.3, 1}, {0.71, 0.261, 3.9, 1}, {0, 0, 0, 0}, {0.02, 0.138, 3.4, 1}, {0, 0, 0, 0}},  // floor, sequential
+    {{2.4, 3.66, 5.8, 0.84}, {1.14, 1.878, 3.5, 0.96}, {0.94, 0.931, 4, 1}, {0.73, 0.28, 3.1, 1}, {1.8, 1.079, 3.4, 1}, {0, 1.863, 2.4, 0.57}, {1.49, 2.437, 2.4, 0.85}},  // floor, chunks of 16
+    {{3.81, 6.691, 3, 1}, {3.08, 3.613, 1.9, 1}, {1.67, 1.822, 3.7, 0.779}, {0.882, 0.506, 2.2, 0.585}, {0, 0, 0, 0}, {0, 0.206, 3.9, 0.85}, {0, 0, 0, 0}},  // floor with product cut, sequential
+    {{2.87, 5.191, 6, 1}, {1.78, 2.756, 3.7, 0.97}, {1.76, 1.37, 4.4, 0.97}, {0.934, 0.392, 3.4, 0.97}, {2.86, 1.551, 3.2, 0.62}, {0, 2.736, 2.6, 0.82}, {2.42, 4.412, 2.9, 0.96}},  // floor with product cut, chunks of 16
     {{1.9, 4.724, 4.7, 0.98}, {1.49, 2.478, 3.2, 1}, {1.2, 1.277, 2.9, 1}, {0.95, 0.354, 2.1, 1}, {0, 0, 0, 0}, {0.24, 0.145, 2.5, 0.99}, {0, 0, 0, 0}},  // nearest-even, sequential
     {{0.08, 5.151, 4.6, 1}, {0.01, 2.783, 3.2, 1}, {1.25, 1.317, 3.5, 1}, {0.97, 0.365, 3.5, 1}, {0, 0, 0, 0}, {0.01, 1.993, 2.6, 0.68}, {1.8, 2.967, 2.7, 0.9}},  // nearest-even, chunks of 16
     {{0, 4.75, 4.2, 1}, {0.05, 2.575, 3.3, 1}, {1.29, 1.14, 3.9, 1}, {0.95, 0.323, 3, 1}, {0, 0, 0, 0}, {0, 1.972, 2.6, 0.5}, {1.98, 2.766, 2.5, 0.92}},  // nearest-even through bfloat16, chunks of 16
+    {{0, 3.39, 4.56, 1}, {0, 2.08, 4.18, 1}, {1.05, 0.843, 4.45, 1}, {0.703, 0.28, 3.64, 0.973}},  // floor, longer chunks
+    {{0, 5.16, 4.99, 0.967}, {1.71, 2.6, 4.34, 1}, {1.65, 1.28, 4.82, 1}, {0.89, 0.361, 4.97, 0.834}},  // floor with product cut, longer chunks
+    {{0, 5.15, 4.7, 1}, {0, 2.77, 4.11, 1}, {1.17, 1.27, 4.27, 1}, {0.877, 0.36, 3.9, 0.906}},  // nearest-even, longer chunks
+    {{0, 7.52, 4.36, 1}, {2.57, 3.76, 3.39, 1}, {2.22, 1.93, 2.73, 0.838}, {1.65, 0.514, 3.3, 1}},  // generic kernel, floor, any chunk length
+    {{0, 33.6, 4.5, 0.997}, {6.79, 17.8, 3.35, 1}, {5.83, 8.04, 3.67, 0.73}, {4.45, 2.17, 4.09, 0.4}},  // generic kernel, nearest-even, any chunk length
+    {{9.44, 57.9, 1.5, 0.972}, {27.5, 16, 1.5, 1}, {24.3, 10.5, 1.5, 0.981}, {6.74, 2.27, 1.5, 1}},  // generic kernel, nearest-even, sequential
+    {{13.9, 60.3, 1.55, 0.976}, {27.6, 19.1, 1.5, 0.779}, {25.5, 10.8, 1.5, 0.795}, {6.92, 2.44, 1.5, 1}},  // generic kernel, nearest-even, longer chunks
+    {{2.01, 2.87, 4.99, 1}, {1.24, 1.59, 3.57, 0.998}, {1.06, 0.763, 3.81, 1}, {0.782, 0.22, 3.5, 1}},  // 24-bit accumulator, sequential
+    {{0, 3.41, 4.46, 0.761}, {1.32, 1.63, 3.83, 1}, {1.03, 0.793, 4.14, 0.846}, {0.78, 0.244, 3, 1}},  // 24-bit accumulator, longer chunks
+    {{0, 3.28, 4.37, 1}, {1.56, 1.85, 3.54, 0.826}, {1.86, 0.804, 3.29, 1}, {1.13, 0.271, 3.14, 1}},  // 24-bit accumulator, any chunk length
 };
+
+int cost_row(const Plan& pl) {
+  const auto by_order = [&pl](int seq, int chunk16, int longer, int any) {
+    return pl.ord == ORD_SEQ ? seq : pl.ord == ORD_CHUNK16 ? chunk16 : pl.ord == ORD_CHUNK_SLAB ? longer : any;
+  };
+  switch (pl.qm) {
+    case QM_FLOOR_FAST: return by_order(ROW_SEQ, ROW_CHUNK16, ROW_LONG, ROW_ANY);
+    case QM_FLOOR_FULL: return by_order(ROW_CUT_SEQ, ROW_CUT_CHUNK16, ROW_CUT_LONG, ROW_ANY);
+    case QM_RNE_WIDE: return by_order(ROW_WIDE_SEQ, ROW_WIDE_LONG, ROW_WIDE_LONG, ROW_WIDE_ANY);
+    default:
+      if (!pl.rne_packed) return by_order(ROW_GENERIC_SEQ, ROW_GENERIC_LONG, ROW_GENERIC_LONG, ROW_RNE_ANY);
+      return by_order(ROW_RNE_SEQ, pl.rne_packed == 2 ? ROW_BF16_CHUNK16 : ROW_RNE_CHUNK16, ROW_RNE_LONG, ROW_RNE_ANY);
+  }
+}
+
 // byte-wise convolution loader (ResNet stem, 401408 x 64 x 147): the fetch is costly, so the tile with the fewest fetched rows
 // per output wins as long as it keeps its registers
 const TileCost kCostConvAny[TILE_COUNT] = {{6, 10.4, 4, 0.5}, {2, 2.85, 4, 0.5}, {1.2, 1.64, 4, 0.5}, {0.8, 0.49, 4, 0.5}};
@@ -408,8 +437,7 @@ TileChoice choose_tile(int64_t M, int64_t N, int64_t K, int64_t batch, const Pla
   if (forced >= 0 && forced < TILE_COUNT) return {forced, forced};
   if (forced == TILE_PAIR && pair_ok) return {TILE_PAIR, TILE_PAIR};
 
-  const bool chunked = ord != ORD_SEQ;
-  const int row = qm == QM_RNE_FULL ? (pl.rne_packed == 2 ? 6 : chunked ? 5 : 4) : qm == QM_FLOOR_FULL ? (chunked ? 3 : 2) : chunked;
+  const int row = cost_row(pl);
   const double slabs = std::fmax(1.0, (double)((K + BK - 1) / BK));
   const int sms = sm_count();
   const auto time = [&](const TileCost& c, int bm, int bn, double per_tile, double g) {

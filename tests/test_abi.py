@@ -161,3 +161,26 @@ def test_format_fields_are_read_by_value_at_every_call(box):
     else:
         f[0] = box(4)
     assert "pq=cut" in plan(f) and "pq=cut" in plan(LbaFormat(*f)) and "pq=none" in plan(p)
+
+
+WIDE = LbaFormat(23, 8, 127, 1, 0)
+FASTEST = [   # formats, order, chunk, shape, the tile that measured fastest (us against the next one)
+    (code_domain_formats(12, 5, 1), SEQ, 16, (2048, 1024, 1024), "32x32"),    # 2080, 2278
+    (code_domain_formats(12, 5, 1), SEQ, 16, (4096, 4096, 512), "128x64"),    # 7161, 7923
+    (code_domain_formats(12, 5, 1), CHK, 16, (4096, 4096, 512), "128x64"),    # 7416, 8443
+    (code_domain_formats(12, 5, 1), CHK, 24, (512, 512, 512), "32x32"),       # 156, 289
+    ((WIDE, WIDE), CHK, 16, (3000, 1500, 1008), "64x64"),                     # 389, 405
+    ((WIDE, WIDE), CHK, 24, (25088, 128, 256), "64x64"),                      # 92, 94
+    (code_domain_formats(7, 4), CHK, 32, (25088, 128, 256), "64x64"),         # 97, 100
+    (code_domain_formats(7, 4), CHK, 16, (2048, 1024, 1024), "64x64"),        # 242, 244; the 128x128 tile 254
+    (code_domain_formats(7, 4), SEQ, 16, (12288, 128, 64), "64x64"),          # 14.3, 15.5
+    (code_domain_formats(4, 4), SEQ, 16, (512, 512, 512), "32x32"),           # 32.8; the chain kernel 42
+    (code_domain_formats(4, 4), SEQ, 16, (64, 4096, 2048), "32x32"),          # 124; the chain kernel 158
+    (code_domain_formats(4, 4), CHK, 16, (64, 4096, 2048), "32x32"),          # 132; the split kernels 138
+]
+
+
+@pytest.mark.parametrize("fmts,order,chunk,shape,tile", FASTEST, ids=lambda v: str(v) if isinstance(v, (str, int)) else "")
+def test_tile_choice_knows_each_kernel(fmts, order, chunk, shape, tile):
+    plan = lba.describe_plan(*shape, *fmts, order, chunk)
+    assert plan.startswith(f"tile={tile}x16 micro") and "by=" not in plan
