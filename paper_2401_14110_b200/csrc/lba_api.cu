@@ -412,8 +412,9 @@ int cost_row(const Plan& pl) {
 }
 
 // byte-wise convolution loader (ResNet stem, 401408 x 64 x 147): the fetch is costly, so the tile with the fewest fetched rows
-// per output wins as long as it keeps its registers
-const TileCost kCostConvAny[TILE_COUNT] = {{6, 10.4, 4, 0.5}, {2, 2.85, 4, 0.5}, {1.2, 1.64, 4, 0.5}, {0.8, 0.49, 4, 0.5}};
+// per output wins as long as it keeps its registers, also on a few more than a hundred CTAs (16384 x 64 x 216: 128x64 37 to 88 us,
+// 64x64 41 to 93).  One row for every rounding and product mode, fitted to the fourteen shapes in profiles/tile_times.txt
+const TileCost kCostConvAny[TILE_COUNT] = {{6, 10.4, 4, 0.5}, {1.5, 2.85, 4, 0.5}, {1.2, 1.64, 4, 0.5}, {0.8, 0.49, 4, 0.5}};
 
 // a launch has at most 2^31 - 1 rows and 65535 columns of CTAs of bm x bn outputs
 bool grid_fits(int64_t M, int64_t N, int bm, int bn, int ctas_per_tile = 1) {
