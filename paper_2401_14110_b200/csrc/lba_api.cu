@@ -480,26 +480,38 @@ TileChoice choose_tile(int64_t M, int64_t N, int64_t K, int64_t batch, const Pla
 }
 
 // Tile of the mask and last-overflow passes: 64x64, or 32x32 where that is faster by the same model (override 2 and 7
-// force one of them).  Measured on fourteen shapes from 64 x 64 x 96 to 4096 x 3072 x 768; 512^3, 64x64 against 32x32: overflow
-// masks 48 / 34 us sequential, 73 / 43 us chunked, difference masks 119 / 104 and 128 / 141, last overflow 90 / 57 us;
-// 4096 x 3072 x 768: 965 / 1124, 1073 / 1311, 2955 / 3310, 3245 / 3888, 2343 / 2429.
-enum SteKernel { STE_OF_SEQ = 0, STE_OF_CHUNK = 1, STE_DIFF_SEQ = 2, STE_DIFF_CHUNK = 3, STE_TRACK_OF = 4 };
-bool small_ste_tile(int64_t M, int64_t N, int64_t K, SteKernel kernel) {
+// force one of them).  A row per kernel, without and with a product cut, which costs the scalar 32x32 kernels their lead.  512^3
+// on 64x64 / 32x32, us: difference masks sequential 119 / 104 and with the cut 142 / 150, chunks of 24 159 / 96 and 178 / 100; last
+// overflow 89 / 57 and 124 / 112; overflow masks in chunks of 32 86 / 68 and 115 / 132, of 24 136 / 89 and 165 / 104.  Difference
+// masks in chunks of whole slabs stay on 64x64: 128 / 140 there, and what 32x32 gains on a handful of CTAs (64 x 64 x 96, 25 / 22) it
+// lost on another GPU (26 / 27).  Sequential difference masks of unaligned rows without a cut, 174 / 190 (1111 x 777 x 403), carry a factor.
+// profiles/tile_times.txt holds the times behind the constants.
+enum SteKernel { STE_OF_SEQ = 0, STE_OF_CHUNK16 = 1, STE_LAST = 2, STE_OF_LONG = 3, STE_OF_ANY = 4, STE_DIFF_SEQ = 5, STE_DIFF_ANY = 6, STE_DIFF_LONG = 7 };
+bool small_ste_tile(int64_t M, int64_t N, int64_t K, SteKernel kernel, bool cut, int load) {
   const int forced = g_tile_override.load(std::memory_order_relaxed);
   if (forced == 2 || forced == 7) return forced == 7;
-  if (kernel == STE_DIFF_CHUNK) return false;  // 118 against 127 us at best (128 x 256 x 512), 41 against 39 (418 x 160 x 144)
-  static const TileCost kSte[5][2] = {{{1.38, 0.965, 4, 1}, {0.93, 0.297, 3, 1}}, {{2.15, 1.08, 4, 1}, {1.22, 0.345, 3, 1}},
-                                      {{2.7, 2.95, 4, 1}, {2.65, 0.95, 3, 1}},    {{2.9, 3.2, 4, 1}, {3.5, 1.5, 3, 1}},
-                                      {{2.0, 2.33, 4, 1}, {1.6, 0.65, 3, 1}}};
+  if (kernel == STE_DIFF_LONG) return false;
+  struct SteCost { double L, b; };
+  static const SteCost kSte[7][2][2] = {
+      {{{1.13, 1.05}, {0.874, 0.313}}, {{2.16, 1.35}, {1.04, 0.39}}},   // overflow masks, sequential (packed kernel)
+      {{{2.05, 1.14}, {1.17, 0.364}}, {{3.17, 1.19}, {1.4, 0.437}}},    // chunks of 16 (packed kernel)
+      {{{1.53, 2.41}, {1.51, 0.68}}, {{2.05, 3.48}, {3.17, 0.955}}},    // last overflow
+      {{{0, 2.63}, {1.97, 0.637}}, {{0, 3.56}, {4.2, 0.888}}},          // overflow masks, longer chunks
+      {{{0, 4.05}, {2.56, 0.974}}, {{0, 5.0}, {2.97, 1.22}}},           // any chunk length
+      {{{2.6, 3.02}, {2.87, 0.908}}, {{2.99, 3.77}, {4.17, 1.29}}},     // difference masks, sequential
+      {{{3.96, 4.25}, {2.69, 1.19}}, {{3.96, 4.64}, {2.81, 1.17}}},     // any chunk length
+  };
+  constexpr double kBase[2] = {4, 3}, kUnalignedDiff = 1.1;
   const double slabs = std::fmax(1.0, (double)((K + BK - 1) / BK));
   double t[2];
   for (int i = 0; i < 2; ++i) {
-    const TileCost& c = kSte[kernel][i];
+    const SteCost& c = kSte[kernel][cut][i];
     const int64_t e = i == 0 ? 64 : 32;
     const double x = (double)((M + e - 1) / e) * (double)((N + e - 1) / e) / sm_count(), q = std::fmax(1.0, std::ceil(x));
-    t[i] = c.base + slabs * std::cbrt(c.L * c.L * c.L + c.b * q * c.b * q * c.b * q);
+    t[i] = slabs * std::cbrt(c.L * c.L * c.L + c.b * q * c.b * q * c.b * q);
   }
-  return t[1] < t[0] && (N + 31) / 32 <= 65535;
+  if (kernel == STE_DIFF_SEQ && !cut && load == LD_GEMM_ROWS) t[1] *= kUnalignedDiff;
+  return kBase[1] + t[1] < kBase[0] + t[0] && grid_fits(M, N, 32, 32);
 }
 
 int fill_scales(Problem* p, const float* sa, int sa_len, const float* sb, int sb_len, const float* bias) {
@@ -732,7 +744,9 @@ int lba_gemm_last_overflow(const uint8_t* A, const uint8_t* B, int64_t M, int64_
   p.out = reinterpret_cast<float*>(last);
   apply_plan(&p, pl);
   const bool vec = K % BK == 0 && aligned16(A) && aligned16(B);
-  const cudaError_t e = launch_last_overflow(small_ste_tile(M, N, K, STE_TRACK_OF), pl.qm, vec ? LD_GEMM_VEC : LD_GEMM_ROWS, p, (cudaStream_t)stream);
+  const int load = vec ? LD_GEMM_VEC : LD_GEMM_ROWS;
+  const bool small = small_ste_tile(M, N, K, STE_LAST, pl.qm == QM_FLOOR_FULL, load);
+  const cudaError_t e = launch_last_overflow(small, pl.qm, load, p, (cudaStream_t)stream);
   return e == cudaSuccess ? LBA_OK : cuda_fail(e);
 }
 
@@ -802,8 +816,13 @@ int lba_gemm_ste_mask(const uint8_t* A, const uint8_t* B, int64_t M, int64_t N, 
   // the overflow masks in sequential and chunk-16 order come from the packed kernel (tile override 3 keeps the
   // scalar tracking kernel, for tests and comparisons); everything else from the scalar one
   const bool packed = ste == LBA_STE_OF && (!chunked || chunk == BK) && g_tile_override.load(std::memory_order_relaxed) != 3;
-  const cudaError_t e = packed ? launch_ste_packed(small_ste_tile(M, N, K, chunked ? STE_OF_CHUNK : STE_OF_SEQ), pl.qm == QM_FLOOR_FAST ? PQ_NONE : pl.pq, chunked ? 1 : 0, load, p, (cudaStream_t)stream)
-                               : launch_ste_mask(small_ste_tile(M, N, K, ste != LBA_STE_DIFF ? STE_TRACK_OF : chunked ? STE_DIFF_CHUNK : STE_DIFF_SEQ), pl.qm, ord, ste == LBA_STE_DIFF, load, p, (cudaStream_t)stream);
+  const bool diff = ste == LBA_STE_DIFF;
+  const SteKernel kernel = packed ? (chunked ? STE_OF_CHUNK16 : STE_OF_SEQ)
+                           : ord == ORD_SEQ ? (diff ? STE_DIFF_SEQ : STE_LAST)
+                           : ord == ORD_CHUNK_SLAB ? (diff ? STE_DIFF_LONG : STE_OF_LONG) : (diff ? STE_DIFF_ANY : STE_OF_ANY);
+  const bool small = small_ste_tile(M, N, K, kernel, pl.qm == QM_FLOOR_FULL, load);
+  const cudaError_t e = packed ? launch_ste_packed(small, pl.qm == QM_FLOOR_FAST ? PQ_NONE : pl.pq, chunked ? 1 : 0, load, p, (cudaStream_t)stream)
+                               : launch_ste_mask(small, pl.qm, ord, diff, load, p, (cudaStream_t)stream);
   return e == cudaSuccess ? LBA_OK : cuda_fail(e);
 }
 

@@ -130,3 +130,25 @@ def test_mask_passes_on_both_tiles(tile, name):
             assert (last == orc.gemm_last_overflow(A.numpy(), B.numpy(), t, a)).all(), (M, N, K)
     finally:
         lba.set_tile_override(-1)
+
+
+@pytest.mark.parametrize("tile", [2, 7])
+@pytest.mark.parametrize("name", ["m7e4", "m4e4"])
+@pytest.mark.parametrize("chunk", [7, 24, 32, 40])
+def test_mask_passes_of_other_chunk_lengths_on_both_tiles(tile, name, chunk):
+    # the scalar kernels: chunks that end inside a slab, a slab that holds several, short last chunks and words
+    prod, acc = SMALL_FORMATS[name]
+    t, a = prod.as_tuple(), acc.as_tuple()
+    lba.set_tile_override(tile)
+    try:
+        for (M, N, K) in ((1, 1, 1), (33, 31, 48), (65, 70, 301), (30, 100, 272)):
+            A, B = synth.random_codes((M, K), 3 * M + K), synth.random_codes((N, K), 5 * N + K)
+            if K == 301:
+                A, B = A & 0x7F, B & 0x7F
+            for kind, e1, e2 in ((lba.STE_OF, 0.0, 0.0), (lba.STE_DIFF, 4.0, 2.0 ** -7)):
+                got = lba.lba_gemm_ste_mask(A.to(DEV), B.to(DEV), prod, acc, CHK, chunk, kind, e1, e2)
+                want = orc.gemm_ste_mask(A.numpy(), B.numpy(), t, a, CHK, chunk, kind, e1, e2)
+                for g, w in zip(got, want):
+                    assert (g.cpu().numpy().view(np.uint32) == w).all(), (M, N, K, kind)
+    finally:
+        lba.set_tile_override(-1)
