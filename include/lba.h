@@ -259,8 +259,8 @@ int lba_describe_plan_batched(int64_t batch, int64_t M, int64_t N, int64_t K, co
  * rounding and 16-byte loads, ignored otherwise; 6, 7 = the small-problem kernels of chunk-16 order on 16x16 and 32x32
  * tiles, 10 = that of sequential order, ignored where they do not apply; -1 = automatic choice, the default).  For lba_gemm_ste_mask, 3
  * selects the scalar tracking kernel where the packed one would run, and 2 and 7 force the 64x64 and the 32x32 tile of
- * the mask and last-overflow passes.  Results never depend on the tile, only speed
- * does.  The setting is one process-wide word (an atomic store): it is meant for tests and tuning runs, it applies
+ * the mask and last-overflow passes (difference masks in chunks that are a multiple of 16 have the 64x64 tile only).
+ * Results never depend on the tile, only speed does.  The setting is one process-wide word (an atomic store): it is meant for tests and tuning runs, it applies
  * to every thread's later calls, and a caller that changes it while other threads are inside the library gets an
  * unspecified mix of old and new tiles, never a wrong result.  Returns LBA_OK, or LBA_ERR_SHAPE for an unknown tile. */
 int lba_set_tile_override(int tile);

@@ -489,8 +489,8 @@ TileChoice choose_tile(int64_t M, int64_t N, int64_t K, int64_t batch, const Pla
 enum SteKernel { STE_OF_SEQ = 0, STE_OF_CHUNK16 = 1, STE_LAST = 2, STE_OF_LONG = 3, STE_OF_ANY = 4, STE_DIFF_SEQ = 5, STE_DIFF_ANY = 6, STE_DIFF_LONG = 7 };
 bool small_ste_tile(int64_t M, int64_t N, int64_t K, SteKernel kernel, bool cut, int load) {
   const int forced = g_tile_override.load(std::memory_order_relaxed);
-  if (forced == 2 || forced == 7) return forced == 7;
   if (kernel == STE_DIFF_LONG) return false;
+  if (forced == 2 || forced == 7) return forced == 7;
   struct SteCost { double L, b; };
   static const SteCost kSte[7][2][2] = {
       {{{1.13, 1.05}, {0.874, 0.313}}, {{2.16, 1.35}, {1.04, 0.39}}},   // overflow masks, sequential (packed kernel)

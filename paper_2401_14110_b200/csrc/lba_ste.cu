@@ -17,7 +17,8 @@ cudaError_t launch_tile(const Problem& p, cudaStream_t stream) {
 
 template <int QM, int ORD, int LD, int TRACK>
 cudaError_t launch(bool small, const Problem& p, cudaStream_t stream) {
-  return small ? launch_tile<32, 32, QM, ORD, LD, TRACK>(p, stream) : launch_tile<64, 64, QM, ORD, LD, TRACK>(p, stream);
+  if constexpr (TRACK == TRACK_MASK_DIFF && ORD == ORD_CHUNK_SLAB) return launch_tile<64, 64, QM, ORD, LD, TRACK>(p, stream);  // the host's only choice
+  else return small ? launch_tile<32, 32, QM, ORD, LD, TRACK>(p, stream) : launch_tile<64, 64, QM, ORD, LD, TRACK>(p, stream);
 }
 
 template <int QM, int ORD, int TRACK>
