@@ -987,14 +987,21 @@ int lba_describe_plan_batched(int64_t batch, int64_t M, int64_t N, int64_t K, co
   }
   const TileChoice choice = choose_tile(M > 0 ? M : 1, N > 0 ? N : 1, K, batch < 65535 ? batch : 65535, pl, load);  // a launch takes 65535 problems
   const int tile = choice.packed;
-  const char* const by = choice.run == choice.packed ? "" : choice.run == TILE_SPLIT ? " by=split16x16" : choice.run == TILE_CHAIN ? " by=chain16x16" : " by=split32x32";
+  const bool small = choice.run != choice.packed;  // then the text ends in the kernel that runs
   // which kernel runs and what Q_prod costs there beyond the flush
   const bool packed = pl.ord != ORD_CHUNK_ANY &&
                       (pl.qm == QM_FLOOR_FAST || pl.qm == QM_FLOOR_FULL || (pl.qm == QM_RNE_FULL && pl.rne_packed));
   const char* const kern = packed ? "packed" : "generic";
-  const char* const pq = (pl.fused && packed && tile < TILE_PAIR) ? "fused"
-                         : (pl.qm == QM_FLOOR_FAST || pl.qm == QM_RNE_WIDE ? "none"
-                            : (pl.pq == PQ_MASK_SAT ? "cut_sat" : (pl.pq == PQ_MASK ? "cut" : "none")));
+  const char* const plain_pq = pl.qm == QM_FLOOR_FAST || pl.qm == QM_RNE_WIDE ? "none"
+                               : pl.pq == PQ_MASK_SAT ? "cut_sat" : pl.pq == PQ_MASK ? "cut" : "none";
+  const char* const pq = pl.fused && packed && tile < TILE_PAIR ? "fused" : plain_pq;
+  char by[112] = "";
+  if (small) {  // these have no fused variant
+    const int e = choice.run == TILE_SPLIT + 1 ? 32 : 16;
+    std::snprintf(by, sizeof(by), " by=%s%dx%d(micro=%s,grid=%lldx%lld,pq=%s)", choice.run == TILE_CHAIN ? "chain" : "split", e, e,
+                  choice.run == TILE_CHAIN ? "1x2" : e == 16 ? "2x4" : "4x8", (long long)((M + e - 1) / e), (long long)((N + e - 1) / e),
+                  plain_pq);
+  }
   if (tile == TILE_PAIR) {
     if (buf && buf_len)
       std::snprintf(buf, buf_len, "tile=64x64x%d pair micro=4x8 q=%s pq=%s kernel=%s order=%s load=%s grid=%lldx%lld%s", BK,
@@ -1003,7 +1010,7 @@ int lba_describe_plan_batched(int64_t batch, int64_t M, int64_t N, int64_t K, co
     return LBA_OK;
   }
   const TileInfo ti = tile_info(tile);
-  if (choice.run == tile && !grid_fits(M, N, ti.bm, ti.bn)) return LBA_ERR_SHAPE;
+  if (!small && !grid_fits(M, N, ti.bm, ti.bn)) return LBA_ERR_SHAPE;
   if (buf && buf_len)
     std::snprintf(buf, buf_len, "tile=%dx%dx%d micro=%dx%d q=%s pq=%s kernel=%s order=%s load=%s grid=%lldx%lld%s", ti.bm, ti.bn,
                   BK, ti.tm, ti.tn, kQmName[pl.qm], pq, kern, kOrdName[pl.ord], kLdName[load],

@@ -136,7 +136,7 @@ def test_wide_outputs_get_a_tile_that_can_be_launched(fmts, order, chunk):
         for M in (1, 17, 80, 96, 280):
             for K in (64, 17):
                 plan = lba.describe_plan(M, N, K, *fmts, order, chunk, vec_ok=K % 16 == 0)
-                assert int(plan.split("grid=")[1].split()[0].split("x")[1]) <= 65535 or "by=" in plan, (M, N, K, plan)
+                assert int(re.findall(r"grid=\d+x(\d+)", plan)[-1]) <= 65535, (M, N, K, plan)
     with pytest.raises(lba.LbaError) as e:
         lba.describe_plan(4, 128 * 65535 + 1, 64, *fmts, order, chunk)
     assert e.value.status == -2
@@ -194,3 +194,18 @@ def test_tile_choice_of_a_convolution_with_few_channels(fmts, order, chunk):
     assert lba.describe_plan(16384, 64, 216, *fmts, order, chunk, is_conv=True, vec_ok=False).startswith("tile=128x64x16")
     # the ResNet stem, batch 1: 64x64 or 32x32 tiles fill the SMs
     assert lba.describe_plan(12544, 64, 147, *fmts, order, chunk, is_conv=True, vec_ok=False).startswith(("tile=64x64x16", "tile=32x32x16"))
+
+
+def test_plan_names_the_small_kernel_that_runs():
+    by = lambda shape, fm, order, chunk=16, **kw: lba.describe_plan(*shape, *fm, order, chunk, **kw).partition(" by=")[2]
+    formats = {"none": [code_domain_formats(7, 4), code_domain_formats(10, 5, 1), code_domain_formats(10, 6), code_domain_formats(10, 7, 1)],
+               "cut": [code_domain_formats(4, 4), code_domain_formats(4, 4, 1)], "cut_sat": [(LbaFormat(5, 4, 4), LbaFormat(7, 4, 6))]}
+    for pq, several in formats.items():   # M10E6 and M10E7 are fused in the packed kernel, which has that variant
+        for f in several:
+            # a small problem gets the small kernels by itself, whatever the mode; one that fills the SMs does not
+            assert by((64, 64, 576), f, CHK) == f"split16x16(micro=2x4,grid=4x4,pq={pq})"
+            assert by((32, 1000, 512), f, CHK) == f"split16x16(micro=2x4,grid=2x63,pq={pq})"      # the classifier
+            assert by((64, 64, 576), f, SEQ) == f"chain16x16(micro=1x2,grid=4x4,pq={pq})"
+            assert by((49, 512, 4608), f, SEQ, is_conv=True) == f"chain16x16(micro=1x2,grid=4x32,pq={pq})"
+            assert by((4096, 4096, 4096), f, CHK) == by((4096, 4096, 4096), f, SEQ) == by((64, 64, 576), f, CHK, 32) == ""
+    assert by((512, 768, 768), code_domain_formats(7, 4), CHK) == "split32x32(micro=4x8,grid=16x24,pq=none)"
