@@ -96,7 +96,7 @@ def _one_case(rng, trial):
         M, N = (int(rng.integers(1, 700)), int(rng.integers(1, 130))) if rng.random() < 0.5 else (M, N)
     order = SEQ if (rng.random() < 0.35 or kind == "last") else CHK
     chunk = int(rng.choice([16, 16, 16, 1, 2, 7, 32, 48, 64, int(rng.integers(1, 100))]))
-    tile = int(rng.choice([-1, -1, -1, 0, 1, 2, 3, 5]))
+    tile = int(rng.choice([-1, -1, -1, 0, 1, 2, 3, 5, 6, 7, 10]))
     ka, kb = rng.choice(["uniform", "gauss", "one_sign", "sparse", "small", "climb"], 2)
     stride = pad = None
     misaligned = bool(rng.random() < 0.15)

@@ -22,14 +22,33 @@ def check_gemm(A, B, prod, acc, order, chunk=16, what=""):
 @pytest.mark.parametrize("rounding", [0, 1])
 @pytest.mark.parametrize("man", [1, 3, 4, 5, 6, 7, 8, 10])
 def test_rounding_cuts_of_every_width(man, rounding):
-    # product and sum cut to `man` bits, in both orders, E4M3 and M4E3 bytes; dense codes and Gaussian data
+    # product and sum cut to `man` bits, in both orders, E4M3 and M4E3 bytes; dense codes and Gaussian data; every tile,
+    # for by itself the shape runs in the small-problem kernels, whose cuts are not those of the packed kernel
     for exp in (4, 5, 6):
         for make, dense in ((code_domain_formats, synth.random_codes((70, 112), 3)),
                             (m4e3_input_formats, torch.arange(70 * 112).mul(37).to(torch.uint8).reshape(70, 112))):
             prod, acc = make(man, exp, rounding)
             B = dense.flip(0).roll(5, 1)[:67].contiguous()
-            for order in (SEQ, CHK):
-                check_gemm(dense, B, prod, acc, order, what=f"{make.__name__} M{man}E{exp} r{rounding} order {order}")
+            a, b, one = dense.to(DEV), B.to(DEV), torch.ones(1)
+            for order, tiles in ((SEQ, (-1, 0, 1, 2, 3, 10)), (CHK, (-1, 0, 1, 2, 3, 5, 6, 7))):
+                want = orc.gemm(dense.numpy(), B.numpy(), one.numpy(), one.numpy(), None, prod.as_tuple(), acc.as_tuple(), order, 16)
+                for tile in tiles:
+                    lba.set_tile_override(tile)
+                    try:
+                        plan = lba.describe_plan(70, 67, 112, prod, acc, order, 16)
+                        got = lba.lba_gemm(a, b, one.to(DEV), one.to(DEV), None, prod, acc, order, 16).cpu().numpy()
+                    finally:
+                        lba.set_tile_override(-1)
+                    what = f"{make.__name__} M{man}E{exp} r{rounding} order {order} tile {tile}: {plan}"
+                    assert (got.view(np.uint32) == want.view(np.uint32)).all(), what
+                    if 0 <= tile < 4:
+                        assert plan.startswith("tile=" + ("128x128", "128x64", "64x64", "32x32")[tile]) and "by=" not in plan, what
+                    elif tile == 5:
+                        assert (" pair " in plan) == (rounding == 0), what
+                    elif tile > 5:
+                        assert ({6: "by=split16x16", 7: "by=split32x32", 10: "by=chain16x16"}[tile] in plan) == ("kernel=packed" in plan), what
+                    if rounding == 0:
+                        assert "kernel=packed" in plan, what
 
 
 @pytest.mark.parametrize("K", [1, 15, 16, 17, 31, 33, 130])
@@ -70,8 +89,8 @@ def test_small_problem_kernels(tile, name):
             if K == 1040:
                 A, B = A & 0x7F, B & 0x7F
                 A[:, 600:] |= 0x80
-            if name == "m7e4":
-                assert "by=" in lba.describe_plan(M, N, K, prod, acc, order, 16, vec_ok=K % 16 == 0)
+            by = lba.describe_plan(M, N, K, prod, acc, order, 16, vec_ok=K % 16 == 0).partition(" by=")[2]
+            assert by.startswith({6: "split16x16(", 7: "split32x32(", 10: "chain16x16("}[tile]), by
             sa, sb, bias = torch.linspace(0.5, 1.5, M), torch.linspace(0.01, 0.02, N), torch.linspace(-1, 1, N)
             got = lba.lba_gemm(A.to(DEV), B.to(DEV), sa.to(DEV), sb.to(DEV), bias.to(DEV), prod, acc, order, 16).cpu().numpy()
             want = orc.gemm(A.numpy(), B.numpy(), sa.numpy(), sb.numpy(), bias.numpy(), prod.as_tuple(), acc.as_tuple(), order, 16)
@@ -93,7 +112,12 @@ def test_small_problem_kernels(tile, name):
     ("plain", code_domain_formats(7, 4)), ("fused", code_domain_formats(10, 6)), ("cut", code_domain_formats(4, 4)),
     ("product_wider", (LbaFormat(7, 4, -2), LbaFormat(5, 4, -4))), ("flush_not_shared", (LbaFormat(7, 4, -2), LbaFormat(7, 4, 0))),
     ("no_acc_flush", (LbaFormat(7, 4, -2), LbaFormat(7, 4, -4, 0, 0))), ("saturating", (LbaFormat(7, 4, 12), LbaFormat(7, 4, 10))),
-    ("rne", code_domain_formats(7, 4, 1)), ("rne_cut", code_domain_formats(4, 4, 1))], ids=lambda v: v if isinstance(v, str) else "")
+    ("rne", code_domain_formats(7, 4, 1)), ("rne_cut", code_domain_formats(4, 4, 1)),
+    # M4E3 bytes, whose products are the widest (10 bits)
+    ("m4e3_cut", m4e3_input_formats(7, 4)), ("m4e3_fused", m4e3_input_formats(9, 4)),
+    ("m4e3_flush", (LbaFormat(9, 4, -3, 0, 5), LbaFormat(9, 4, -5))), ("m4e3_cut_flush", (LbaFormat(6, 4, -3, 0, 5), LbaFormat(7, 4, -5))),
+    ("m4e3_product_wider", (LbaFormat(9, 4, -3, 0, 5), LbaFormat(7, 4, -5))),
+    ("m4e3_rne_flush", (LbaFormat(9, 4, -3, 1, 5), LbaFormat(9, 4, -5, 1))), ("m4e3_rne_cut", m4e3_input_formats(7, 4, 1))], ids=lambda v: v if isinstance(v, str) else "")
 @pytest.mark.parametrize("tile", [0, 2, 5])
 def test_first_step_of_a_chunk(tile, name, fmts):
     # chunks whose first product is tiny, short or large: the step that may leave out the mask and one multiplication
