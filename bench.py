@@ -45,33 +45,55 @@ LANES_PER_SM_CLK = 128
 MIX = {
     # mode: (issue, logic, packed_fp, scalar_fp, text)
     "floor": (2.0, 1.0, 1.0, 0.0, "0.5 FMUL2 + 0.5 FFMA2 + 1 LOP3"),
-    "floor_cut": (3.0, 2.0, 1.0, 0.0, "0.5 FMUL2 + 1 LOP3 (product mask) + 0.5 FFMA2 + 1 LOP3"),
-    "floor_cut_sat": (4.0, 3.0, 1.0, 0.0, "0.5 FMUL2 + 1 LOP3 + 1 FMNMX (product) + 0.5 FFMA2 + 1 LOP3"),
+    "floor_cut": (3.0, 1.5, 1.5, 0.0, "0.5 FMUL2 + 0.5 FFMA2 + 1 LOP3, product cut by 1 LOP3 in one register pair and by "
+                                      "0.5 FMUL2 + 0.5 FFMA2 in the next"),
+    "floor_cut_sat": (4.0, 2.5, 1.5, 0.0, "as floor_cut, plus 1 FMNMX for the product's saturation"),
     "floor_fused": (1.5, 1.0, 0.5, 0.0, "0.5 FFMA2 (product and sum in one instruction) + 1 LOP3"),
-    "rne": (4.0, 2.0, 2.0, 0.0, "0.5 FMUL2 + 0.5 FFMA2 + 1 LOP3 + 1 FFMA2 (rounding on the FP32 pipe) + 1 FMNMX"),
-    "rne_cut": (6.0, 3.0, 3.0, 0.0, "as rne, plus 1 LOP3 + 1 FFMA2 for the product's rounding"),
-    "rne_cut_sat": (7.0, 4.0, 3.0, 0.0, "as rne_cut, plus 1 FMNMX for the product's saturation"),
-    "rne_fused": (3.5, 2.0, 1.5, 0.0, "0.5 FFMA2 (product and sum) + 1 LOP3 + 1 FFMA2 (rounding) + 1 FMNMX"),
+    "rne": (2.0, 0.0, 2.0, 0.0, "0.5 FMUL2 + 0.5 FFMA2 + 0.5 FMUL2 + 0.5 FFMA2 (rounding on the FP32 pipe)"),
+    "rne_bf16": (2.5, 1.0, 1.0, 0.0, "0.5 FMUL2 + 0.5 FFMA2 + 0.5 F2FP (rounding to bfloat16) + 0.5 SHL + 0.5 LOP3"),
+    "rne_cut": (3.0, 0.0, 3.0, 0.0, "as rne, plus 0.5 FMUL2 + 0.5 FFMA2 for the product's rounding"),
+    "rne_bf16_cut": (3.5, 1.0, 2.0, 0.0, "as rne_bf16, plus 0.5 FMUL2 + 0.5 FFMA2 for the product's rounding"),
+    "rne_cut_sat": (4.0, 1.0, 3.0, 0.0, "as rne_cut, plus 1 FMNMX for the product's saturation"),
+    "rne_bf16_cut_sat": (4.5, 2.0, 2.0, 0.0, "as rne_bf16_cut, plus 1 FMNMX for the product's saturation"),
+    "rne_fused": (1.5, 0.0, 1.5, 0.0, "0.5 FFMA2 (product and sum) + 0.5 FMUL2 + 0.5 FFMA2 (rounding)"),
+    "rne_bf16_fused": (2.0, 1.0, 0.5, 0.0, "0.5 FFMA2 (product and sum) + 0.5 F2FP + 0.5 SHL + 0.5 LOP3 (rounding)"),
     "rne_wide": (1.0, 0.0, 0.0, 1.0, "1 FFMA (24-bit accumulator: one IEEE FMA per MAC)"),
     "generic": (6.0, 4.0, 0.0, 2.0, "scalar FMUL + FFMA + mask + clamp (+ product steps): the generic kernel"),
     "fixed": (6.0, 4.0, 0.0, 2.0, "2 SHF + 2 add-min/max on the logic pipe; IMAD + IADD beside them"),
     "ste_diff": (7.0, 3.0, 3.0, 1.0, "0.5 each of FMUL2, FFMA2 (chain), FMUL2, FFMA2 (distance), FFMA2, FMUL2 (threshold) "
                                      "+ LOP3 + FMNMX + FADD (thr - |d|) + SHF (its sign into the mask)"),
 }
-FOLD = {  # per output per chunk: (issue, logic, packed_fp, scalar_fp)
-    "floor": (2.5, 2.0, 0.5, 0.0), "rne": (3.5, 2.0, 1.5, 0.0), "rne_wide": (1.0, 0.0, 0.0, 1.0), "generic": (4.0, 2.0, 0.0, 1.0),
-    "fixed": (4.0, 4.0, 0.0, 0.0),
+# per output per chunk, (issue, logic, packed_fp, scalar_fp): the fold, with its clamp, and what the first step of a chunk of
+# 16 saves, which is the (cut) product alone where the formats allow it, as they do throughout the benchmark
+FOLD = {
+    "floor": (2.5, 2.0, 0.5, 0.0), "rne": (2.5, 1.0, 1.5, 0.0), "rne_bf16": (3.0, 2.0, 0.5, 0.0), "rne_wide": (1.0, 0.0, 0.0, 1.0),
+    "generic": (4.0, 2.0, 0.0, 1.0), "fixed": (4.0, 4.0, 0.0, 0.0),
 }
+FIRST_STEP = {
+    "floor": (1.5, 1.0, 0.5, 0.0), "floor_cut": (1.5, 1.0, 0.5, 0.0), "floor_fused": (1.0, 1.0, 0.0, 0.0),
+    "rne": (1.5, 0.0, 1.5, 0.0), "rne_fused": (1.0, 0.0, 1.0, 0.0), "rne_bf16": (2.0, 1.0, 0.5, 0.0), "rne_bf16_fused": (1.5, 1.0, 0.0, 0.0),
+}
+
+
+def per_chunk(mode: str, chunk: int):
+    """What a chunk adds per output to the mix of its steps: the fold, less what its first step saves."""
+    for base in ("floor", "rne_wide", "rne_bf16", "rne", mode):
+        if mode == base or mode.startswith(base + "_"):
+            break
+    fold = FOLD.get(base, FOLD["generic"])
+    first = FIRST_STEP.get(mode) if chunk == 16 else None
+    return tuple(f - s for f, s in zip(fold, first)) if first else fold
+
+
+def mix_per_mac(mode: str, chunk: int):
+    """(issue, logic, packed_fp, scalar_fp) per emulated MAC of the minimal mix of `mode`; chunk = 0: sequential."""
+    extra = per_chunk(mode, chunk) if chunk else (0.0,) * 4
+    return tuple(x + (e / chunk if chunk else 0.0) for x, e in zip(MIX[mode], extra))
 
 
 def clocks_per_warp_mac(mode: str, chunk: int):
     """(clocks per warp-MAC per scheduler, which limit binds) of the minimal mix of `mode`; chunk = 0: sequential."""
-    issue, logic, packed, scalar, _ = MIX[mode]
-    if chunk:
-        base = "rne" if mode.startswith("rne") and mode != "rne_wide" else ("floor" if mode.startswith("floor") else mode)
-        f = FOLD.get(base, FOLD["generic"])
-        issue, logic, packed, scalar = (issue + f[0] / chunk, logic + f[1] / chunk, packed + f[2] / chunk,
-                                        scalar + f[3] / chunk)
+    issue, logic, packed, scalar = mix_per_mac(mode, chunk)
     limits = {"issue": issue, "logic pipe": 2.0 * logic, "fp32 pipe": 2.0 * packed + scalar}
     which = max(limits, key=limits.get)
     return limits[which], which
@@ -79,18 +101,19 @@ def clocks_per_warp_mac(mode: str, chunk: int):
 
 def min_issue_slots(mode: str, chunk: int) -> float:
     """Issue slots per emulated MAC of the minimal mix (the figure executed instructions per MAC compare with)."""
-    base = "rne" if mode.startswith("rne") and mode != "rne_wide" else ("floor" if mode.startswith("floor") else mode)
-    return MIX[mode][0] + (FOLD.get(base, FOLD["generic"])[0] / chunk if chunk else 0.0)
+    return mix_per_mac(mode, chunk)[0]
 
 
-def mode_of(desc: str, ste=None, fixed=False) -> str:
-    """Mix name of the kernel variant a plan description names."""
+def mode_of(desc: str, ste=None, fixed=False, acc_man_bits=None) -> str:
+    """Mix name of the kernel variant a plan description names (`acc_man_bits`: M of the accumulator's format)."""
     if fixed:
         return "fixed"
     if ste == "diff":
         return "ste_diff"
     f = dict(p.split("=", 1) for p in desc.split() if "=" in p)
     q, pq = f.get("q", ""), f.get("pq", "none")
+    if "by" in f:  # a small-problem kernel runs, with a product mode of its own
+        pq = f["by"].rpartition("pq=")[2].rstrip(")")
     suffix = {"none": "", "cut": "_cut", "cut_sat": "_cut_sat", "fused": "_fused"}.get(pq, "")
     if f.get("kernel") == "generic" and q != "rne_wide":
         return "generic"
@@ -98,7 +121,7 @@ def mode_of(desc: str, ste=None, fixed=False) -> str:
         return "floor" + suffix
     if q == "rne_wide":
         return "rne_wide"
-    return "rne" + suffix
+    return ("rne_bf16" if acc_man_bits == 7 and f.get("order") == "chunk16" else "rne") + suffix
 
 
 def peak_gmacs(mode, chunk, sm_count, mhz):
@@ -414,7 +437,7 @@ def kernel_table(wl, per_call_ms, sm_count, max_mhz):
         e["macs"] += c.macs
         e["launches"] += 1
     for key, e in table.items():
-        mode = mode_of(key, ste=wl.ste if wl.ste == "diff" else None, fixed=wl.fixed is not None)
+        mode = mode_of(key, ste=wl.ste if wl.ste == "diff" else None, fixed=wl.fixed is not None, acc_man_bits=wl.acc.man_bits)
         peak, slots, pipe = peak_gmacs(mode, wl.chunk if wl.order == 1 else 0, sm_count, max_mhz)
         e.update(gmacs=e["macs"] / (e["ms"] * 1e-3) / 1e9, mode=mode, peak=peak, slots=slots, pipe=pipe)
         e["frac"] = e["gmacs"] / peak
@@ -714,8 +737,8 @@ def main(argv=None):
         "kernel_share_of_step": dom["ms"] / sum(per_call_ms),
         "peak_derivation": f"{sm_count} SMs x {LANES_PER_SM_CLK} lanes issued per clock x {max_mhz:.0f} MHz (clocks.max.sm) / "
                            f"{dom['slots']:g} issue slots per emulated MAC of the minimal mix ({MIX[dom['mode']][4]}"
-                           + (f", plus {FOLD.get('rne' if dom['mode'].startswith('rne') else 'floor', FOLD['generic'])[0]:g} per output "
-                              f"per chunk of {wl.chunk}" if wl.order == 1 else "") + ")",
+                           + (f", plus {per_chunk(dom['mode'], wl.chunk)[0]:g} per output "
+                              f"per chunk of {wl.chunk}: the fold less what the first step saves" if wl.order == 1 else "") + ")",
         "pipe_limit": dom["pipe"],
         "frac_at_sampled_clock": dom["gmacs"] / (dom["peak"] * mhz / max_mhz),
         "whole_step_frac_of_peak": ideal_ms / sum(per_call_ms),

@@ -209,3 +209,17 @@ def test_plan_names_the_small_kernel_that_runs():
             assert by((49, 512, 4608), f, SEQ, is_conv=True) == f"chain16x16(micro=1x2,grid=4x32,pq={pq})"
             assert by((4096, 4096, 4096), f, CHK) == by((4096, 4096, 4096), f, SEQ) == by((64, 64, 576), f, CHK, 32) == ""
     assert by((512, 768, 768), code_domain_formats(7, 4), CHK) == "split32x32(micro=4x8,grid=16x24,pq=none)"
+
+
+def test_benchmark_mix_is_that_of_the_kernel_that_runs():
+    import bench
+    mode = lambda shape, f, order: bench.mode_of(lba.describe_plan(*shape, *f, order, 16), acc_man_bits=f[1].man_bits)
+    small, large = (64, 64, 576), (4096, 4096, 4096)
+    assert mode(large, code_domain_formats(10, 6), CHK) == "floor_fused" and mode(small, code_domain_formats(10, 6), CHK) == "floor"
+    assert mode(large, code_domain_formats(7, 4, 1), CHK) == "rne_bf16" and mode(large, code_domain_formats(7, 4, 1), SEQ) == "rne"
+    assert mode(large, code_domain_formats(5, 5, 1), CHK) == "rne_cut" and mode(large, code_domain_formats(12, 5, 1), CHK) == "generic"
+    # two packed instructions cut a pair: half of FMUL2, FFMA2, FMUL2, FFMA2 per MAC; a chunk adds the fold's FADD2, cut and
+    # clamp (2.5) and saves the first step's FFMA2 and cut (1.5)
+    assert bench.min_issue_slots("rne", 0) == 2.0 and bench.min_issue_slots("rne", 16) == 2.0625
+    assert bench.min_issue_slots("floor", 16) == 2.0625 and bench.min_issue_slots("floor", 32) == 2 + 2.5 / 32
+    assert all(bench.clocks_per_warp_mac(m, c)[0] >= bench.min_issue_slots(m, c) for m in bench.MIX for c in (0, 16, 24))
