@@ -243,7 +243,7 @@ int make_plan(const lba_fmt* pf, const lba_fmt* af, int order, int chunk, int64_
   const int u1 = (-ka) / 2, u2 = (-ka) - u1;
   pl->un1 = (float)std::ldexp(1.0, u1);
   pl->un2 = (float)std::ldexp(1.0, u2);
-  // packed floor kernel: operands decoded by the hardware converter, then scaled by 2^sx, 2^sw; row
+  // packed and small-problem kernels: operands decoded by the hardware converter, then scaled by 2^sx, 2^sw; row
   // norms and |S| are measured as fractions of 2^(e_max_acc + 1), the first magnitude the mantissa
   // mask alone would not bring back to R_OF.  A scale that binary32 cannot hold switches the
   // clamp-free path off (infinite norms) rather than risk an underestimate.

@@ -14,14 +14,17 @@
 //     exact sum (truncations compose), so `t & mask` is the floor of Eq. 2 on the exact sum.  `.ftz` flushes
 //     exactly the sums below R_UF_acc, because a toward-zero rounding never moves a value across 2^-126.
 //   * saturation: min.xorsign.abs(t, R_OF') = sign(t) * min(|t|, R_OF'), one instruction.
-// Nearest-even does not compose with a binary32 rounding, so that mode first builds the round-to-odd image of
-// the exact sum (from directed roundings of the FMA) and rounds that.
+// Nearest-even does not compose with a binary32 rounding in general.  Where the host proves that the rounding of the FMA
+// cannot decide a tie (M_acc <= 10 and the conditions in make_plan), the sum is one FMA rounded to nearest and is cut by
+// two FP32 instructions (rne2_fp) or by the conversion to bfloat16 (rne2_bf16); elsewhere the generic kernel builds the
+// round-to-odd image of the exact sum (from directed roundings of the FMA) and rounds that.
 // The host proves per call which branches of Eq. 2 E4M3 inputs can reach and picks the cheapest exact variant.
 //
 // Two kernels share the operand loaders:
 //   lba_contract_packed_kernel  packed f32x2 arithmetic (two outputs per instruction), the magnitude clamp
 //                               skipped per slab under a norm bound; floor and nearest-even; the fast path
-//   lba_contract_kernel         scalar arithmetic, always clamped; any chunk length, 24-bit accumulator
+//   lba_contract_kernel         scalar arithmetic, always clamped; any chunk length, 24-bit accumulator, nearest-even with
+//                               wider mantissas
 // Data path of both: a CTA owns a BM x BN output tile and walks K in slabs of 16 bytes per row; each thread
 // fetches 16-byte row pieces (one 128-bit load), decodes the 16 E4M3 bytes to scaled binary32 once, and stores
 // them k-major into shared memory (double buffered, one barrier per slab).  Each thread keeps a TM x TN
@@ -35,7 +38,7 @@
 namespace lba {
 
 enum QMode { QM_FLOOR_FAST = 0, QM_FLOOR_FULL = 1, QM_RNE_FULL = 2, QM_RNE_WIDE = 3, QM_COUNT = 4 };
-// ORD_CHUNK16: chunk == BK, the paper's chunk size; only the packed floor kernel specialises it
+// ORD_CHUNK16: chunk == BK, the paper's chunk size; the packed kernel and the small-problem kernels specialise it
 enum OrdMode { ORD_SEQ = 0, ORD_CHUNK_SLAB = 1, ORD_CHUNK_ANY = 2, ORD_CHUNK16 = 3, ORD_COUNT = 4 };
 // GEMM rows at 16-byte boundaries; NHWC taps with C_in a multiple of 16; any convolution, byte by byte; GEMM rows at any
 // byte address with any K
@@ -70,7 +73,7 @@ struct Problem {
   QConst qp, qa;
   int chunk_slabs;     // ORD_CHUNK_SLAB: chunk / BK
   int chunk;           // ORD_CHUNK_ANY
-  // packed floor kernel only
+  // packed and small-problem kernels
   float pk_a, pk_b;    // 2^sx, 2^sw: decoded value -> product-carrier operand
   // chunk-16 order: 1 if the first step of a chunk, Q_acc(Q_prod(x w) + 0), is the (cut) product alone: it has no more
   // significant bits than the accumulator and is flushed by Q_acc wherever Q_prod flushes it.  A's first operand of
@@ -882,12 +885,11 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), TRACK == TRACK_MASK_DIF
   }
 }
 
-// ------------------------------------------------------------------ packed floor kernel
-// The fast floor quantiser (Q_prod reduced to its flush, floor rounding) on the packed binary32
-// instructions of sm_100: two neighbouring outputs of a row share one 64-bit register pair, so
-// the product and the sum of two emulated MACs cost one `mul.ftz.f32x2` and one `fma.rz.ftz.f32x2`,
-// followed by one mantissa mask per output.  The magnitude clamp of Eq. 2 is left out of a slab
-// whenever it provably cannot act there:
+// ------------------------------------------------------------------ packed kernel
+// The packed binary32 instructions of sm_100: two neighbouring outputs of a row share one 64-bit register pair, so
+// the product and the sum of two emulated MACs cost one `mul.ftz.f32x2` and one `fma.rz.ftz.f32x2` (`fma.rn.ftz.f32x2`
+// under nearest-even), followed by one mantissa mask per output (nearest-even: rne2_fp or rne2_bf16 per pair).  The
+// magnitude clamp of Eq. 2 is left out of a slab whenever it provably cannot act there; under floor rounding
 //   |S_i| <= |S_start| + sum_k |x_k w_k| <= |S_start| + ||x||_2 ||w||_2        (floor never grows |.|)
 // so if that bound stays below 2^(e_max+1) every masked sum is already <= R_OF.  The loader
 // computes the squared 2-norm of every 16-byte row piece while decoding it; the largest A-row and
