@@ -311,7 +311,7 @@ int make_plan(const lba_fmt* pf, const lba_fmt* af, int order, int chunk, int64_
     const int prod_bits = (p_sat || pf->man_bits + 1 < in.product_bits) ? pf->man_bits + 1 : in.product_bits;
     const bool ok = (top_acc + 25 - af->man_bits <= 127) && (top_prod + 25 - pf->man_bits <= 127) && af->man_bits <= 10 &&
                      prod_bits <= af->man_bits + 1 && ka - kp >= -12 && ka - kp <= 60;
-    // M = 7 in chunks of 16: round through bfloat16 (8.6 against 7.7 TMAC/s on 4096 x 4096 x 2048).  Sequentially the
+    // M = 7 in chunks of 16: round through bfloat16 (9.2 against 7.7 TMAC/s on 8192^3).  Sequentially the
     // conversion sits in every link of the chain and the FP32-pipe cut is faster (7.9 against 7.4).
     pl->rne_packed = !ok ? 0 : (af->man_bits == 7 && order == LBA_ORDER_CHUNKED && chunk == BK && K > BK) ? 2 : 1;
   }
