@@ -944,7 +944,10 @@ __host__ __device__ constexpr int packed_tmem_cols() {
 // sums are not in registers.  So is the 4x8 one in chunk-16 order, where 130 to 144 registers had cost a quarter (64x64) or
 // half (128x64) of the CTAs: nearest-even M7E4 on the 128x64 tile, GEMM 4096 x 4096 x 512 1146 to 983 us, ResNet stem
 // 729 to 598 us.  So are, under floor rounding, the loaders of unaligned rows and of any convolution, whose loads in flight would
-// otherwise cost fifty registers and half the resident CTAs, and the mask passes.
+// otherwise cost fifty registers and half the resident CTAs, and the mask passes.  In longer chunks only the byte-wise loader with
+// a floor cut of the product is (181 registers without; the FP32-pipe cut is a longer chain, which one CTA per SM does not hide):
+// 25088 x 64 x 147 in chunks of 32, M5E5: 6.5 % slower than with masks alone, 77 us against 59 with the bound (401408 rows 807, 682;
+// 16384 x 64 x 216, one CTA per SM in any case, 53.1, 54.1 and 54.7 with masks alone).  The other modes would lose up to 7 % on that last shape.
 // PQ: what Q_prod has to do beyond the flush (the host proves which cases are reachable): nothing, cut the
 // mantissa (M_prod < 7), or cut and saturate (448^2 >= R_OF_prod)
 // PQ_FUSED: Q_prod is the identity on every reachable product (no cut, no saturation, and no product can fall under
@@ -974,6 +977,7 @@ enum PackedProd { PQ_NONE = 0, PQ_MASK = 1, PQ_MASK_SAT = 2, PQ_FUSED = 3 };
 template <int BM, int BN, int TM, int TN, int PQ, int RNE, int ORD, int LD, int STE = 0, int CL = 1, bool H16 = false>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN),
                                   ((TM * TN == 64 && ORD != ORD_CHUNK_SLAB && !RNE) || (TM * TN == 32 && ORD == ORD_CHUNK16) ||
+                                   (TM * TN == 32 && ORD == ORD_CHUNK_SLAB && LD == LD_CONV_ANY && (PQ == PQ_MASK || PQ == PQ_MASK_SAT) && !RNE) ||
                                    ((LD == LD_CONV_ANY || LD == LD_GEMM_ROWS || STE != 0) && !RNE && ORD != ORD_CHUNK_SLAB))
                                       ? 512 / ((BM / TM) * (BN / TN)) : 1)
     lba_contract_packed_kernel(const Problem p) {
