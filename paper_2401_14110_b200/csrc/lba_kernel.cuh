@@ -1000,16 +1000,14 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
   static_assert(TN == 4 || TN == 8, "micro-tile cols");
   static_assert(BM % 32 == 0 && BN % 32 == 0, "a warp loads rows of one operand only");
 
-  // A is stored twice, {a, a}, so that a 64-bit shared load yields the packed multiplier directly
+  // operands of a slab, [buffer][k][row]: the BM rows of A, then the BN rows of B
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  typedef float2 (*AsT)[BK][BM];
-  typedef float (*BsT)[BK][BN];
-  AsT As = reinterpret_cast<AsT>(smem_raw);
-  BsT Bs = reinterpret_cast<BsT>(smem_raw + sizeof(float2) * 2 * BK * BM);
+  typedef float (*SlabT)[BK][ROWS];
+  SlabT ab = reinterpret_cast<SlabT>(smem_raw);
   // largest normalised squared row norm of the slab, as binary32 bits (non-negative, so they order
   // like integers): [slab % 3][0 = A, 1 = B]; three cells so that one can be cleared while the
   // neighbours are read and filled
-  unsigned (*nrm)[2] = reinterpret_cast<unsigned (*)[2]>(smem_raw + sizeof(float2) * 2 * BK * BM + sizeof(float) * 2 * BK * BN);
+  unsigned (*nrm)[2] = reinterpret_cast<unsigned (*)[2]>(smem_raw + sizeof(float) * 2 * BK * ROWS);
   unsigned* tmem_slot = reinterpret_cast<unsigned*>(nrm) + 6;  // base address written by tcgen05.alloc
   // STE: [q][tid] words, q = i * PN + j: bits of the pair's low output in the low half, of its high output above
   uint32_t* const stash1 = reinterpret_cast<uint32_t*>(nrm) + 8;
@@ -1052,8 +1050,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
           for (int j = 0; j < 4; ++j) {
             n2 = fma_rn(v[j], v[j], n2);
             const float s = mul_ieee(v[j], q + j == 0 ? mul_first : mul);
-            if (is_a) As[buf][q * 4 + j][r] = make_float2(s, s);
-            else Bs[buf][q * 4 + j][r - BM] = s;
+            ab[buf][q * 4 + j][r] = s;
           }
         }
         {
@@ -1110,16 +1107,20 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
     }
 #pragma unroll UNR
     for (int kk = 0; kk < BK; ++kk) {
+      // A is stored once and paired with itself in registers.  What the inner loop waits for is the register file: a packed
+      // multiply with one register as both halves of a factor reads one register less, and a 4x8 micro-tile takes three
+      // 128-bit loads per k-step instead of the four that a copy {a, a} in shared memory took.  8192 x 8192 x 1024, M7E4,
+      // clocks per warp-MAC, before and after: chunk 16 3.26 and 3.11 (128x128 tile), 3.34 and 3.14 (64x64); sequential 3.07
+      // and 2.94; product cut 4.92 and 4.55 (64x64); nearest-even through bfloat16 4.08 and 3.85.
       u64 a2[TM], b2[PN];
 #pragma unroll
       for (int h = 0; h < TM / 4; ++h) {
-        const ulonglong2* src = reinterpret_cast<const ulonglong2*>(&As[buf][kk][h * (BM / 2) + ty * 4]);
-        const ulonglong2 v0 = src[0], v1 = src[1];
-        a2[h * 4 + 0] = v0.x; a2[h * 4 + 1] = v0.y; a2[h * 4 + 2] = v1.x; a2[h * 4 + 3] = v1.y;
+        const float4 v = *reinterpret_cast<const float4*>(&ab[buf][kk][h * (BM / 2) + ty * 4]);
+        a2[h * 4 + 0] = pack2(v.x, v.x); a2[h * 4 + 1] = pack2(v.y, v.y); a2[h * 4 + 2] = pack2(v.z, v.z); a2[h * 4 + 3] = pack2(v.w, v.w);
       }
 #pragma unroll
       for (int h = 0; h < TN / 4; ++h) {
-        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(&Bs[buf][kk][h * (BN / 2) + tx * 4]);
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(&ab[buf][kk][BM + h * (BN / 2) + tx * 4]);
         b2[h * 2 + 0] = v.x; b2[h * 2 + 1] = v.y;
       }
       if constexpr (!RNE) {
@@ -1780,7 +1781,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
 
 template <int BM, int BN>
 constexpr size_t packed_smem_bytes() {
-  return sizeof(float2) * 2 * BK * BM + sizeof(float) * 2 * BK * BN + sizeof(unsigned) * 8;
+  return sizeof(float) * 2 * BK * (BM + BN) + sizeof(unsigned) * 8;
 }
 // the cluster variant adds the double-buffered hand-over of chunk sums (one word per output of a column half and buffer)
 template <int BM, int BN, int TM, int TN>
@@ -1795,8 +1796,7 @@ constexpr size_t packed_ste_smem_bytes() {
 
 // Launch entry of one (quantiser mode, order mode) family; defined once per translation unit.
 // tile: 0 = 128x128 (8x8 per thread, 256 threads), 1 = 128x64 (4x8, 256 threads), 2 = 64x64 (4x8, 128 threads),
-// 3 = 32x32 (4x4, 64 threads).  Micro-tiles are wider than tall because only the A operand is stored twice:
-// a 4x8 micro-tile needs 2 + 2 shared loads per k-step, an 8x4 one 4 + 1.  Measured and dropped: 8x8 in CTAs of
+// 3 = 32x32 (4x4, 64 threads).  Measured and dropped (with A stored twice): 8x8 in CTAs of
 // 64 or 128 threads, 4x8 in 32x64, 32x128, 64x128, 128x128, 64x256 tiles, a one-warp 32x32 tile.
 struct TileInfo { int bm, bn, tm, tn; };
 constexpr int TILE_COUNT = 4;
