@@ -902,16 +902,71 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), TRACK == TRACK_MASK_DIF
 constexpr int FP_CUT = 1;
 constexpr int KUNROLL = 16;  // k-steps unrolled in the packed slab body (the whole slab: measured fastest)
 
-// two E4M3 bytes (low 16 bits of `pair`) -> their exact values, by the hardware converter
-__device__ __forceinline__ void e4m3x2_to_f32(uint32_t pair, float& v0, float& v1) {
-  asm("{\n\t.reg .b16 c, lo, hi;\n\t.reg .b32 h;\n\t"
-      "cvt.u16.u32 c, %2;\n\t"
-      "cvt.rn.f16x2.e4m3x2 h, c;\n\t"
-      "mov.b32 {lo, hi}, h;\n\t"
-      "cvt.f32.f16 %0, lo;\n\t"
-      "cvt.f32.f16 %1, hi;\n\t}"
-      : "=f"(v0), "=f"(v1)
-      : "r"(pair));
+// Four operand bytes -> their exact values, two pairs.  E4M3 bytes go through the hardware converter to half precision, and a
+// half is widened by a mixed-precision FMA (h * 1 - 0, signs of zero kept), a plain FP32-pipe instruction where the conversion
+// holds its pipe for two clocks.  M4E3 bytes become halves by moving their seven magnitude bits under half precision's
+// exponent, for two bytes at a time, and adding 15 to it; the FMA's other factor is 0 for the code e = m = 0 and 1 for all others.
+template <bool M4E3>
+__device__ __forceinline__ void decode4(uint32_t w, u64& v01, u64& v23) {
+  uint32_t h[2], g[2] = {0x3C003C00u, 0x3C003C00u};
+  if (M4E3) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const uint32_t t = __byte_perm(w, 0u, q == 0 ? 0x1404 : 0x3424);  // each byte on top of its half: s eee mmmm 0000 0000
+      const uint32_t mag = (t >> 2) & 0x1FC01FC0u;
+      h[q] = (mag + 0x3C003C00u) | (t & 0x80008000u);
+      asm("set.ne.f16x2.f16x2 %0, %1, %2;" : "=r"(g[q]) : "r"(mag), "r"(0u));
+    }
+  } else {
+    asm("{\n\t.reg .b16 lo, hi;\n\t"
+        "mov.b32 {lo, hi}, %2;\n\t"
+        "cvt.rn.f16x2.e4m3x2 %0, lo;\n\t"
+        "cvt.rn.f16x2.e4m3x2 %1, hi;\n\t}"
+        : "=r"(h[0]), "=r"(h[1])
+        : "r"(w));
+  }
+  float v[4];
+#pragma unroll
+  for (int q = 0; q < 2; ++q)
+    asm("{\n\t.reg .b16 lo, hi, one, two;\n\t"
+        "mov.b32 {lo, hi}, %2;\n\t"
+        "mov.b32 {one, two}, %3;\n\t"
+        "fma.rn.f32.f16 %0, lo, one, %4;\n\t"
+        "fma.rn.f32.f16 %1, hi, two, %4;\n\t}"
+        : "=f"(v[2 * q]), "=f"(v[2 * q + 1])
+        : "r"(h[q]), "r"(g[q]), "f"(-0.0f));
+  v01 = pack2(v[0], v[1]);
+  v23 = pack2(v[2], v[3]);
+}
+
+// Sixteen bytes of a row -> scaled values, handed over pair by pair (store(k, pair), k even), and their squared 2-norm.
+// `first` scales the first pair, `mul` the others.  About 50 instructions where byte-wise steps took 91 (E4M3) and 170
+// (M4E3): the slab's decode is 7 to 10 % of the inner loop on the 64x64 and 32x32 tiles, and it costs what it issues.
+template <bool M4E3, typename Store>
+__device__ __forceinline__ float decode_row(const uint4& row, u64 first, u64 mul, Store store) {
+  const uint32_t w4[4] = {row.x, row.y, row.z, row.w};
+  u64 n[2];  // partial sums: one chain of sixteen would be the longest in here
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    u64 v[2];
+    decode4<M4E3>(w4[q], v[0], v[1]);
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      n[e] = q == 0 ? mul2_rn(v[e], v[e]) : fma2_rn(v[e], v[e], n[e]);
+      store(4 * q + 2 * e, mul2_rn(v[e], q + e == 0 ? first : mul));
+    }
+  }
+  float n0, n1, n2, n3;
+  unpack2(n[0], n0, n1);
+  unpack2(n[1], n2, n3);
+  return (n0 + n1) + (n2 + n3);
+}
+
+// square root of a bound; the 1 % that every user adds covers its error
+__device__ __forceinline__ float sqrt_approx(float v) {
+  float d;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(d) : "f"(v));
+  return d;
 }
 
 // ---- tensor memory as a second register file.  In chunk-16 order the second-level sums T are touched
@@ -1004,13 +1059,14 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
   extern __shared__ __align__(16) unsigned char smem_raw[];
   typedef float (*SlabT)[BK][ROWS];
   SlabT ab = reinterpret_cast<SlabT>(smem_raw);
-  // largest normalised squared row norm of the slab, as binary32 bits (non-negative, so they order
-  // like integers): [slab % 3][0 = A, 1 = B]; three cells so that one can be cleared while the
-  // neighbours are read and filled
-  unsigned (*nrm)[2] = reinterpret_cast<unsigned (*)[2]>(smem_raw + sizeof(float) * 2 * BK * ROWS);
-  unsigned* tmem_slot = reinterpret_cast<unsigned*>(nrm) + 6;  // base address written by tcgen05.alloc
+  // largest normalised squared row norms of a slab, as binary32 bits (non-negative, so they order like integers):
+  // [buffer][warp's 32 rows], A's first
+  constexpr int NRM = ROWS / 32, NRM_A = BM / 32;
+  unsigned (*nrm)[8] = reinterpret_cast<unsigned (*)[8]>(smem_raw + sizeof(float) * 2 * BK * ROWS);
+  static_assert(NRM <= 8, "norm cells");
+  unsigned* tmem_slot = reinterpret_cast<unsigned*>(nrm) + 16;  // base address written by tcgen05.alloc
   // STE: [q][tid] words, q = i * PN + j: bits of the pair's low output in the low half, of its high output above
-  uint32_t* const stash1 = reinterpret_cast<uint32_t*>(nrm) + 8;
+  uint32_t* const stash1 = reinterpret_cast<uint32_t*>(nrm) + 20;
   uint32_t* const stash2 = stash1 + (STE ? TM * PN * NT : 0);   // [o][tid], o = i * TN + 2 * j + half
 
   const int tid = threadIdx.x;
@@ -1021,44 +1077,35 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
   const int64_t n0 = (int64_t)blockIdx.y * BN;
   const int nslab = (int)((p.K + BK - 1) / BK);
   // CL = 2: chunk sums in flight between the two CTAs, [buffer][group of 2 pairs][thread] as uint4
-  uint4* const hand = reinterpret_cast<uint4*>(reinterpret_cast<uint32_t*>(nrm) + 8);
+  uint4* const hand = reinterpret_cast<uint4*>(reinterpret_cast<uint32_t*>(nrm) + 20);
 
   RowLoader<BM, BN, NT, LD> loader;
   loader.init(p, tid, m0, n0);
 
-  auto decode_store = [&](const uint4 (&raw)[LPT], int buf, int cell, int slab) {
+  auto decode_store = [&](const uint4 (&raw)[LPT], int buf, int slab) {
 #pragma unroll
     for (int l = 0; l < LPT; ++l) {
       const int r = tid + l * NT;
       if (r < ROWS) {  // uniform per warp: BM, BN and NT are multiples of 32
-        const bool is_a = r < BM;
-        const float mul = is_a ? p.pk_a : p.pk_b, mul_first = CH16 && is_a ? p.pk_a0 : mul;
         const uint4 row = loader.take(p, l, slab, raw[l]);
-        const uint32_t w4[4] = {row.x, row.y, row.z, row.w};
-        float n2 = 0.0f;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          float v[4];
-          if (p.in_m4e3) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) v[j] = decode_m4e3_top(byte_to_top(w4[q], j));
-          } else {
-            e4m3x2_to_f32(w4[q], v[0], v[1]);
-            e4m3x2_to_f32(w4[q] >> 16, v[2], v[3]);
-          }
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            n2 = fma_rn(v[j], v[j], n2);
-            const float s = mul_ieee(v[j], q + j == 0 ? mul_first : mul);
-            ab[buf][q * 4 + j][r] = s;
-          }
-        }
-        {
-          const unsigned m = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(n2 * p.nrm_scale));
-          if ((tid & 31) == 0) atomicMax(&nrm[cell][is_a ? 0 : 1], m);
-        }
+        const float mul = r < BM ? p.pk_a : p.pk_b, first = CH16 && r < BM ? p.pk_a0 : mul;
+        float* const dst = &ab[buf][0][r];
+        const auto store = [&](int k, u64 v) { unpack2(v, dst[k * ROWS], dst[(k + 1) * ROWS]); };
+        const float n2 = p.in_m4e3 ? decode_row<true>(row, pack2(first, mul), pack2(mul, mul), store)
+                                   : decode_row<false>(row, pack2(first, mul), pack2(mul, mul), store);
+        const unsigned m = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(n2 * p.nrm_scale));
+        if ((tid & 31) == 0) nrm[buf][r / 32] = m;
       }
     }
+  };
+  // ||x|| ||w|| / 2^(e_max+1) of the slab in `buf`, rounded up generously (the norms carry rounding errors near 2^-20)
+  auto slab_growth = [&](int buf) -> float {
+    unsigned na = nrm[buf][0], nb = nrm[buf][NRM_A];
+#pragma unroll
+    for (int i = 1; i < NRM_A; ++i) na = max(na, nrm[buf][i]);
+#pragma unroll
+    for (int i = NRM_A + 1; i < NRM; ++i) nb = max(nb, nrm[buf][i]);
+    return sqrt_approx(__uint_as_float(na) * __uint_as_float(nb)) * 1.01f;
   };
 
   u64 acc1[TM][PN];
@@ -1349,7 +1396,6 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
     return mx;
   };
 
-  if (tid < 6) nrm[tid >> 1][tid & 1] = 0u;
   if (T_IN_TMEM) {
     // one warp allocates for the CTA; tcgen05.alloc returns once the SM has the columns free (CTAs
     // that hold columns never wait for anything before they release them at the end of the kernel)
@@ -1378,7 +1424,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
   if (CL > 1 && crank != 0) loader.skip_slab(p);
   if (s_first < nslab) {
     loader.fetch(p, tid, s_first, raw);
-    decode_store(raw, 0, 0, s_first);
+    decode_store(raw, 0, s_first);
   }
   __syncthreads();
 
@@ -1495,7 +1541,6 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
   float u = 0.0f;   // upper bound of max |acc1| of this thread, as a fraction of 2^(e_max + 1)
   float u2 = 0.0f;  // chunk-16 order: the same for the second-level sums
   int slabs_in_chunk = 0;
-  int cell = 0;     // s % 3
   if constexpr (CL > 1) {
     // ---- two CTAs per output tile (see the kernel's header comment).  Both run the same number of rounds and
     // meet at one cluster barrier per round; nothing leaves the loop early.  CTA r forms the chunk sums of the
@@ -1593,17 +1638,13 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
       const bool have = s < nslab;          // only CTA 1 can run out, in the last round of an odd slab count
       const bool more = s + CL < nslab;
       const int buf = q & 1;
-      const int cell_next = cell == 2 ? 0 : cell + 1;
-      const int cell_clear = cell_next == 2 ? 0 : cell_next + 1;
       if (more) {
         loader.skip_slab(p);
         loader.fetch(p, tid, s + CL, raw);
       }
       float grow = 0.0f;
       if (have) {
-        const float na = __uint_as_float(nrm[cell][0]), nb = __uint_as_float(nrm[cell][1]);
-        if (tid < 2) nrm[cell_clear][tid] = 0u;
-        grow = sqrtf(na * nb) * 1.01f;
+        grow = slab_growth(buf);
         if (grow < lim) slab_body(buf, std::false_type());
         else slab_body(buf, std::true_type());
         if (crank == 0) send(std::integral_constant<int, 1>(), q);
@@ -1619,9 +1660,8 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
         fold_received(std::integral_constant<int, 1>(), q);
         if (have) fold_own(std::integral_constant<int, 1>(), grow);
       }
-      if (more) decode_store(raw, buf ^ 1, cell_next, s + CL);
+      if (more) decode_store(raw, buf ^ 1, s + CL);
       __syncthreads();
-      cell = cell_next;
     }
 
     // ---- epilogue of the pair: this CTA's column half
@@ -1659,13 +1699,8 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
   } else
   for (int s = 0; s < nslab; ++s) {
     const int buf = s & 1;
-    const int cell_next = cell == 2 ? 0 : cell + 1;
-    const int cell_clear = cell_next == 2 ? 0 : cell_next + 1;
     if (s + 1 < nslab) loader.fetch(p, tid, s + 1, raw);
-    const float na = __uint_as_float(nrm[cell][0]), nb = __uint_as_float(nrm[cell][1]);
-    if (tid < 2) nrm[cell_clear][tid] = 0u;  // read during the previous slab, filled during the next
-    // ||x|| ||w|| / 2^(e_max+1), rounded up generously (the norms carry rounding errors near 2^-20)
-    const float grow = sqrtf(na * nb) * 1.01f;
+    const float grow = slab_growth(buf);
     if (CH16) {
       // the chunk starts from zero, so the CTA-wide bound alone decides (same value in every thread)
       const float gw = grow * gs;
@@ -1716,9 +1751,8 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
         }
       }
     }
-    if (s + 1 < nslab) decode_store(raw, buf ^ 1, cell_next, s + 1);
+    if (s + 1 < nslab) decode_store(raw, buf ^ 1, s + 1);
     __syncthreads();
-    cell = cell_next;
   }
   if (CHUNKED && !CH16 && slabs_in_chunk > 0) close_chunk(std::true_type());
   if (T_IN_TMEM) {  // every thread is done with its columns (with K = 0 nothing was ever closed and acc1 is 0)
@@ -1781,7 +1815,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
 
 template <int BM, int BN>
 constexpr size_t packed_smem_bytes() {
-  return sizeof(float) * 2 * BK * (BM + BN) + sizeof(unsigned) * 8;
+  return sizeof(float) * 2 * BK * (BM + BN) + sizeof(unsigned) * 20;
 }
 // the cluster variant adds the double-buffered hand-over of chunk sums (one word per output of a column half and buffer)
 template <int BM, int BN, int TM, int TN>

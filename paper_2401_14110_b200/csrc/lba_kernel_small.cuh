@@ -82,46 +82,20 @@ struct PairSteps {
   }
 };
 
-// square root of a bound; the 1 % that every user adds covers its error
-__device__ __forceinline__ float sqrt_approx(float v) {
-  float d;
-  asm("sqrt.approx.f32 %0, %1;" : "=f"(d) : "f"(v));
-  return d;
-}
-
 // sixteen bytes of a row -> scaled binary32, k-major in shared memory, `stride` elements from one k to the next (T = float2:
 // every value twice); returns the squared 2-norm, scaled
 __device__ __forceinline__ void put(float2& dst, float v) { dst = make_float2(v, v); }
 __device__ __forceinline__ void put(float& dst, float v) { dst = v; }
 template <typename T>
-__device__ __forceinline__ float decode_row(const Problem& p, const uint4& row, float mul, T* dst, int stride) {
-  const uint32_t w4[4] = {row.x, row.y, row.z, row.w};
-  u64 n4[2];  // partial sums: one chain of sixteen would be the longest in here
+__device__ __forceinline__ float stage_row(const Problem& p, const uint4& row, float mul, T* dst, int stride) {
+  const auto store = [&](int k, u64 v) {
+    float s0, s1;
+    unpack2(v, s0, s1);
+    put(dst[k * stride], s0);
+    put(dst[(k + 1) * stride], s1);
+  };
   const u64 mul2 = pack2(mul, mul);
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    float v[4];
-    if (p.in_m4e3) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) v[j] = decode_m4e3_top(byte_to_top(w4[q], j));
-    } else {
-      e4m3x2_to_f32(w4[q], v[0], v[1]);
-      e4m3x2_to_f32(w4[q] >> 16, v[2], v[3]);
-    }
-#pragma unroll
-    for (int j = 0; j < 4; j += 2) {
-      const u64 v2 = pack2(v[j], v[j + 1]);
-      n4[j / 2] = q == 0 ? mul2_rn(v2, v2) : fma2_rn(v2, v2, n4[j / 2]);
-      float s0, s1;
-      unpack2(mul2_rn(v2, mul2), s0, s1);
-      put(dst[(q * 4 + j) * stride], s0);
-      put(dst[(q * 4 + j + 1) * stride], s1);
-    }
-  }
-  float x0, x1, x2, x3;
-  unpack2(n4[0], x0, x1);
-  unpack2(n4[1], x2, x3);
-  const float n2 = (x0 + x1) + (x2 + x3);
+  const float n2 = p.in_m4e3 ? decode_row<true>(row, mul2, mul2, store) : decode_row<false>(row, mul2, mul2, store);
   return n2 == 0.0f ? 0.0f : n2 * p.nrm_scale;  // (the scale may be infinite)
 }
 
@@ -209,12 +183,12 @@ __global__ void __launch_bounds__(32 * G) lba_split_kernel(const Problem p) {
       float na = 0.0f, nb = 0.0f;
       if constexpr (S::TWICE) {
         static_assert(!S::TWICE || (BM == 32 && BN == 32), "a row of A and a row of B per lane");
-        na = decode_row(p, loader.take(p, 0, s, raw[0]), p.pk_a, &As[0][lane], BM);
-        nb = decode_row(p, loader.take(p, Loader::LPT - 1, s, raw[Loader::LPT - 1]), p.pk_b, &Bs[0][lane], BN);
+        na = stage_row(p, loader.take(p, 0, s, raw[0]), p.pk_a, &As[0][lane], BM);
+        nb = stage_row(p, loader.take(p, Loader::LPT - 1, s, raw[Loader::LPT - 1]), p.pk_b, &Bs[0][lane], BN);
       } else {
         static_assert(S::TWICE || (BM == 16 && BN == 16), "a row of A or of B per lane");
         const bool is_a = lane < BM;
-        const float n2 = decode_row(p, loader.take(p, 0, s, raw[0]), is_a ? p.pk_a : p.pk_b,
+        const float n2 = stage_row(p, loader.take(p, 0, s, raw[0]), is_a ? p.pk_a : p.pk_b,
                                     reinterpret_cast<float*>(is_a ? (void*)&As[0][lane] : (void*)&Bs[0][lane - BM]), BM);
         na = is_a ? n2 : 0.0f;
         nb = is_a ? 0.0f : n2;
@@ -338,7 +312,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS) lba_chain_kernel(const Problem 
         loader.fetch_apart(p, lane, s + CHAIN_SLABS, raw);
       }
       float* const dst = lane < BM ? &As[slot][0][lane] : &Bs[slot][0][lane - BM];
-      const float n2 = decode_row(p, row, lane < BM ? p.pk_a : p.pk_b, dst, BM);
+      const float n2 = stage_row(p, row, lane < BM ? p.pk_a : p.pk_b, dst, BM);
       const unsigned na = __reduce_max_sync(0xFFFFFFFFu, lane < BM ? __float_as_uint(n2) : 0u);
       const unsigned nb = __reduce_max_sync(0xFFFFFFFFu, lane < BM ? 0u : __float_as_uint(n2));
       if (lane == 0) bound[slot] = sqrt_approx(__uint_as_float(na) * __uint_as_float(nb)) * 1.01f;
