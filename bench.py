@@ -45,9 +45,9 @@ LANES_PER_SM_CLK = 128
 MIX = {
     # mode: (issue, logic, packed_fp, scalar_fp, text)
     "floor": (2.0, 1.0, 1.0, 0.0, "0.5 FMUL2 + 0.5 FFMA2 + 1 LOP3"),
-    "floor_cut": (3.0, 1.5, 1.5, 0.0, "0.5 FMUL2 + 0.5 FFMA2 + 1 LOP3, product cut by 1 LOP3 in one register pair and by "
-                                      "0.5 FMUL2 + 0.5 FFMA2 in the next"),
-    "floor_cut_sat": (4.0, 2.5, 1.5, 0.0, "as floor_cut, plus 1 FMNMX for the product's saturation"),
+    "floor_cut": (2.5, 1.0, 1.5, 0.0, "0.5 FMUL2 + 0.5 FFMA2 (product and its cut, from two scalings of A) + 0.5 FFMA2 + 1 LOP3"),
+    "floor_cut_sat": (4.0, 2.5, 1.5, 0.0, "as floor, the product cut by 1 LOP3 in one register pair and by 0.5 FMUL2 + 0.5 FFMA2 in "
+                                          "the next, plus 1 FMNMX for its saturation"),
     "floor_fused": (1.5, 1.0, 0.5, 0.0, "0.5 FFMA2 (product and sum in one instruction) + 1 LOP3"),
     "rne": (2.0, 0.0, 2.0, 0.0, "0.5 FMUL2 + 0.5 FFMA2 + 0.5 FMUL2 + 0.5 FFMA2 (rounding on the FP32 pipe)"),
     "rne_bf16": (2.5, 1.0, 1.0, 0.0, "0.5 FMUL2 + 0.5 FFMA2 + 0.5 F2FP (rounding to bfloat16) + 0.5 SHL + 0.5 LOP3"),

@@ -77,7 +77,7 @@ struct Plan {
   int first_plain;
   float clamp_lim, slab_factor, fold_factor;
   int pq, rne_packed;
-  float acc_k1, acc_k2, prod_k1, prod_k2;
+  float acc_k1, acc_k2, prod_k1, prod_k2, cut_a, cut_a0, cut_ratio;
   QConst qp, qa;
   int chunk_slabs, chunk;
   int kp, ka, sx;   // product carrier = value * 2^kp, accumulator carrier = value * 2^ka, A operand = x * 2^sx
@@ -326,6 +326,21 @@ int make_plan(const lba_fmt* pf, const lba_fmt* af, int order, int chunk, int64_
     pl->pk_a0 = pl->first_plain ? (float)std::ldexp(1.0, s0) : pl->pk_a;
   }
 
+  // ---- floor cut of the product inside A's scales (see cut_product): x (1 + 2^s) must fit 24 bits beside x's own 4 (E4M3) or 5
+  // (M4E3), s = 23 - M_prod, and x times 2^s must stay a binary32 number.  Where it does not, the kernel with the general
+  // cut runs, whose saturation is then a no-op.
+  pl->cut_a = pl->cut_a0 = pl->cut_ratio = 0.0f;
+  if (pl->pq == PQ_MASK && !nearest) {
+    const int s = 23 - pf->man_bits, top = 9 + s + (sx > sx + ka - kp ? sx : sx + ka - kp);
+    if (s + (pl->in_m4e3 ? 5 : 4) <= 24 && top <= 127) {
+      pl->cut_a = pl->pk_a * pl->prod_k2;
+      pl->cut_a0 = pl->pk_a0 * pl->prod_k2;
+      pl->cut_ratio = pl->prod_k1 / pl->prod_k2;
+    } else {
+      pl->pq = PQ_MASK_SAT;
+    }
+  }
+
   // ---- fused product and sum: Q_prod must be the identity on every reachable product (no cut, no saturation, no
   // product under R_UF_prod), and the rescaled B operand must stay a normal binary32 number
   {
@@ -550,6 +565,7 @@ void apply_plan(Problem* p, const Plan& pl) {
   p->in_m4e3 = pl.in_m4e3;
   p->acc_k1 = pl.acc_k1; p->acc_k2 = pl.acc_k2;
   p->prod_k1 = pl.prod_k1; p->prod_k2 = pl.prod_k2;
+  p->cut_a = pl.cut_a; p->cut_a0 = pl.cut_a0; p->cut_ratio = pl.cut_ratio;
   p->fx_shift0 = pl.fx_shift0;
   p->fx_lo_p = pl.fx_lo_p; p->fx_hi_p = pl.fx_hi_p; p->fx_sh_p = pl.fx_sh_p; p->fx_hold_p = pl.fx_hold_p;
   p->fx_lo_a = pl.fx_lo_a; p->fx_hi_a = pl.fx_hi_a; p->fx_sh_a = pl.fx_sh_a; p->fx_wrap_a = pl.fx_wrap_a;

@@ -87,6 +87,8 @@ struct Problem {
   int in_m4e3;         // operands are bytes of the paper's M4E3 W/A format (Sec. 3.1) instead of OCP E4M3
   float acc_k1, acc_k2;    // nearest-even cut of a sum: v k2 + rn(v k1) (see rne2_fp)
   float prod_k1, prod_k2;  // the same for a product; under floor rounding v k2 + rz(v k1) (see floor2_fp)
+  // floor cut of the product that A's scales can carry (0: they cannot; see cut_product): the scales times k2, and k1 / k2
+  float cut_a, cut_a0, cut_ratio;
   // clamp elision: a slab or fold runs without the magnitude clamp while (bound + growth) * factor < clamp_lim.
   // Floor never raises a magnitude: factors 1, limit just under 1 (of 2^(e_max+1)).  Nearest-even can raise one by
   // half a grid step per rounding: slab_factor bounds sixteen such steps (and the product's own rounding),
@@ -227,6 +229,13 @@ __device__ __forceinline__ u64 pack2(float lo, float hi) {
 __device__ __forceinline__ void unpack2(u64 v, float& lo, float& hi) {
   asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
 }
+// the two values of a pair, each as both halves of a factor (no copy: a packed instruction reads one register for both)
+__device__ __forceinline__ void both2(u64 v, u64& lo2, u64& hi2) {
+  float lo, hi;
+  unpack2(v, lo, hi);
+  lo2 = pack2(lo, lo);
+  hi2 = pack2(hi, hi);
+}
 __device__ __forceinline__ u64 mul2_ftz(u64 a, u64 b) {
   u64 d;
   asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
@@ -289,6 +298,14 @@ __device__ __forceinline__ u64 mul2_rz_ftz(u64 a, u64 b) {
 // Floor cut of a pair of products to M bits on the FP32 pipe: k1 = 1 + 2^s, k2 = -2^s, r = rz(v * k1) = 2^s v + v cut to v's
 // grid, minus 2^s v exactly.  Only for values of at most 10 significant bits (s > 10): v k1 must not reach the next binade.
 __device__ __forceinline__ u64 floor2_fp(u64 v, u64 k1, u64 k2) { return fma2_rn(v, k2, mul2_rz_ftz(v, k1)); }
+// The same without the product itself: ak1 = a k1 and ak2 = a k2 are exact (5 significant bits times 1 + 2^s, s <= 19), so
+// r = rz(b ak1) is the r above and b ak2 + r the cut.  `.ftz` flushes the cut exactly where it would have flushed the product: R_UF
+// lies on the cut's grid, so a value is below it if and only if its cut is.  An r that is flushed itself belongs to a product below
+// 2^-s R_UF, whose b ak2 is flushed as well.
+// Two FP32 instructions per pair where mul and floor2_fp take three and mul and two masks as many plus two logic ones; the
+// 64x64 tile runs 8192 x 8192 x 1024 at 4.29 clocks per warp-MAC (M4E3 operands, M7E4, chunk 16; 4.44 with every second pair on
+// the logic pipe), 4.13 (M5E5, sequential; 4.21).
+__device__ __forceinline__ u64 cut_product(u64 b, u64 ak1, u64 ak2) { return fma2_rn_ftz(b, ak2, mul2_rz_ftz(b, ak1)); }
 __device__ __forceinline__ u64 add2_rz_ftz(u64 a, u64 b) {
   u64 d;
   asm("add.rz.ftz.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
@@ -896,9 +913,8 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), TRACK == TRACK_MASK_DIF
 // B-row norms of the slab give one bound per CTA, and each thread carries an upper bound `u` of
 // its own |S| (as a fraction of 2^(e_max+1)), refreshed from the registers when it gets too loose.
 // A warp whose bound fails runs the same slab with the clamp.  Results are identical either way.
-// Under floor rounding with a product cut the logic pipe binds (four masks per pair and step).  Every second register pair of
-// a micro-tile row (j % 2 == FP_CUT) therefore cuts its product on the FP32 pipe: 7.8 against 7.1 TMAC/s on 4096^3 in chunk-16
-// order (every fourth pair 7.3), 8.1 against 7.8 sequentially.
+// Under floor rounding with a product cut in which the product can saturate too the logic pipe binds (four masks per pair and
+// step).  Every second register pair of a micro-tile row (j % 2 == FP_CUT) therefore cuts its product on the FP32 pipe.
 constexpr int FP_CUT = 1;
 constexpr int KUNROLL = 16;  // k-steps unrolled in the packed slab body (the whole slab: measured fastest)
 
@@ -1003,8 +1019,9 @@ __host__ __device__ constexpr int packed_tmem_cols() {
 // a floor cut of the product is (181 registers without; the FP32-pipe cut is a longer chain, which one CTA per SM does not hide):
 // 25088 x 64 x 147 in chunks of 32, M5E5: 6.5 % slower than with masks alone, 77 us against 59 with the bound (401408 rows 807, 682;
 // 16384 x 64 x 216, one CTA per SM in any case, 53.1, 54.1 and 54.7 with masks alone).  The other modes would lose up to 7 % on that last shape.
-// PQ: what Q_prod has to do beyond the flush (the host proves which cases are reachable): nothing, cut the
-// mantissa (M_prod < 7), or cut and saturate (448^2 >= R_OF_prod)
+// PQ: what Q_prod has to do beyond the flush (the host proves which cases are reachable): nothing, cut the mantissa (M_prod < 7;
+// under floor rounding where A's scales can carry the cut, M_prod >= 3 or 4), or cut and saturate (448^2 >= R_OF_prod, and the
+// floor cuts to fewer bits, whose saturation is a no-op)
 // PQ_FUSED: Q_prod is the identity on every reachable product (no cut, no saturation, and no product can fall under
 // R_UF_prod), so FMAq(x, w, S) = Q_acc(x w + S) and the product needs no instruction of its own: one packed FMA forms the
 // exact product and the sum; the B operand then carries the accumulator's scaling.
@@ -1049,6 +1066,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
   constexpr int TMEM_COLS = packed_tmem_cols<BM, BN, TM, TN, RNE, ORD>();
   constexpr bool T_IN_TMEM = TMEM_COLS > 0;   // second-level sums in tensor memory
   constexpr bool T_IN_REGS = CHUNKED && !T_IN_TMEM;
+  constexpr bool CUT = PQ == PQ_MASK && !RNE;  // A's scales carry the cut of the product
   static_assert(!T_IN_TMEM || (TM * TN) % 16 == 0, "tensor-memory groups of 16 columns");
   static_assert(ORD == ORD_SEQ || ORD == ORD_CHUNK_SLAB || ORD == ORD_CHUNK16, "order");
   static_assert(TM == 4 || TM == 8, "micro-tile rows");
@@ -1088,7 +1106,8 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
       const int r = tid + l * NT;
       if (r < ROWS) {  // uniform per warp: BM, BN and NT are multiples of 32
         const uint4 row = loader.take(p, l, slab, raw[l]);
-        const float mul = r < BM ? p.pk_a : p.pk_b, first = CH16 && r < BM ? p.pk_a0 : mul;
+        const float mul = r < BM ? (CUT ? p.cut_a : p.pk_a) : p.pk_b;
+        const float first = CH16 && r < BM ? (CUT ? p.cut_a0 : p.pk_a0) : mul;
         float* const dst = &ab[buf][0][r];
         const auto store = [&](int k, u64 v) { unpack2(v, dst[k * ROWS], dst[(k + 1) * ROWS]); };
         const float n2 = p.in_m4e3 ? decode_row<true>(row, pack2(first, mul), pack2(mul, mul), store)
@@ -1129,6 +1148,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
   const bool first_plain = p.first_plain;
   const u64 acc_k1 = pack2(p.acc_k1, p.acc_k1), acc_k2 = pack2(p.acc_k2, p.acc_k2);
   const u64 prod_k1 = pack2(p.prod_k1, p.prod_k1), prod_k2 = pack2(p.prod_k2, p.prod_k2);
+  const u64 cut_ratio = pack2(p.cut_ratio, p.cut_ratio);
   auto rne_acc = [&](u64 v) -> u64 {
     if (RNE == 2) {
       float lo, hi;
@@ -1159,11 +1179,20 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
       // 128-bit loads per k-step instead of the four that a copy {a, a} in shared memory took.  8192 x 8192 x 1024, M7E4,
       // clocks per warp-MAC, before and after: chunk 16 3.26 and 3.11 (128x128 tile), 3.34 and 3.14 (64x64); sequential 3.07
       // and 2.94; product cut 4.92 and 4.55 (64x64); nearest-even through bfloat16 4.08 and 3.85.
-      u64 a2[TM], b2[PN];
+      u64 a2[TM], b2[PN], a1[CUT ? TM : 1];
 #pragma unroll
       for (int h = 0; h < TM / 4; ++h) {
-        const float4 v = *reinterpret_cast<const float4*>(&ab[buf][kk][h * (BM / 2) + ty * 4]);
-        a2[h * 4 + 0] = pack2(v.x, v.x); a2[h * 4 + 1] = pack2(v.y, v.y); a2[h * 4 + 2] = pack2(v.z, v.z); a2[h * 4 + 3] = pack2(v.w, v.w);
+        const float* const src = &ab[buf][kk][h * (BM / 2) + ty * 4];
+        if constexpr (CUT) {
+          const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(src);
+          both2(v.x, a2[h * 4 + 0], a2[h * 4 + 1]);
+          both2(v.y, a2[h * 4 + 2], a2[h * 4 + 3]);
+          both2(mul2_rn(v.x, cut_ratio), a1[h * 4 + 0], a1[h * 4 + 1]);
+          both2(mul2_rn(v.y, cut_ratio), a1[h * 4 + 2], a1[h * 4 + 3]);
+        } else {
+          const float4 v = *reinterpret_cast<const float4*>(src);
+          a2[h * 4 + 0] = pack2(v.x, v.x); a2[h * 4 + 1] = pack2(v.y, v.y); a2[h * 4 + 2] = pack2(v.z, v.z); a2[h * 4 + 3] = pack2(v.w, v.w);
+        }
       }
 #pragma unroll
       for (int h = 0; h < TN / 4; ++h) {
@@ -1172,8 +1201,9 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
       }
       if constexpr (!RNE) {
         auto product = [&](int i, int j) -> u64 {
+          if constexpr (CUT) return cut_product(b2[j], a1[i], a2[i]);
           u64 pr = mul2_ftz(b2[j], a2[i]);
-          if (PQ == PQ_MASK || PQ == PQ_MASK_SAT) {  // floor of Eq. 2 on the exact product, then its saturation
+          if (PQ == PQ_MASK_SAT) {  // floor of Eq. 2 on the exact product, then its saturation
             float plo, phi;
             if (j % 2 == FP_CUT) pr = floor2_fp(pr, prod_k1, prod_k2);
             unpack2(pr, plo, phi);
@@ -1181,11 +1211,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
               plo = and_bits(plo, pmask);
               phi = and_bits(phi, pmask);
             }
-            if (PQ == PQ_MASK_SAT) {
-              plo = clamp_mag(plo, psat);
-              phi = clamp_mag(phi, psat);
-            }
-            pr = pack2(plo, phi);
+            pr = pack2(clamp_mag(plo, psat), clamp_mag(phi, psat));
           }
           return pr;
         };
@@ -1249,9 +1275,10 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
         // The order of the pairs, as measured (8192 x 8192 x 1024, M7E4, clocks per warp-MAC).  Chunks of 16: pair after pair, along
         // a row and back along the next one (so that neighbours share a factor): 3.05 on the 64x64 tile and 3.14 on 128x64,
         // 3.12 and 3.22 with the products one row ahead of the sums; down the columns of the 8x8 micro-tile: 3.03, 3.08.
-        // Sequentially, and beside the logic instructions of a product cut, one row ahead: 2.95 against 2.97 to 3.00.
-        if constexpr (CH16 && PQ == PQ_NONE) {
-          if constexpr (TM == 8) {
+        // Sequentially, and beside the logic instructions of a saturating product, one row ahead: 2.95 against 2.97 to 3.00.
+        // A cut product along the rows in every order (4.29 on 64x64, 4.39 one row ahead; sequentially 4.13, 4.14).
+        if constexpr ((CH16 && PQ == PQ_NONE) || CUT) {
+          if constexpr (TM == 8 && !CUT) {
 #pragma unroll
             for (int j = 0; j < PN; ++j)
 #pragma unroll

@@ -6,7 +6,8 @@ import torch
 from oracle import lba_oracle as orc
 from paper_2401_14110_b200 import binding as lba
 from paper_2401_14110_b200 import synth
-from paper_2401_14110_b200 import LbaFormat, code_domain_formats, m4e3_input_formats, ORDER_SEQUENTIAL as SEQ, ORDER_CHUNKED as CHK
+from paper_2401_14110_b200 import (FLAG_INPUT_M4E3, LbaFormat, code_domain_formats, m4e3_input_formats, ORDER_SEQUENTIAL as SEQ,
+                                   ORDER_CHUNKED as CHK)
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -176,3 +177,26 @@ def test_mask_passes_of_other_chunk_lengths_on_both_tiles(tile, name, chunk):
                     assert (g.cpu().numpy().view(np.uint32) == w).all(), (M, N, K, kind)
     finally:
         lba.set_tile_override(-1)
+
+
+@pytest.mark.parametrize("man", [1, 2, 3, 4, 6, 8])
+@pytest.mark.parametrize("wa", ["e4m3", "m4e3"])
+def test_floor_cut_inside_the_operand_scales(wa, man):
+    # every pair of codes as the only product of a chain, at the first step of a chunk, inside one and in the second slab: the cut
+    # that A's scales carry, down to the shortest mantissa they can (E4M3: 3 bits, M4E3: 4) and below, with the product
+    # flush in reach and not.  (E4M3 products have 8 bits: M = 8 is no cut.)
+    for bias in (-6, 0):
+        prod = LbaFormat(man, 5, bias, 0, 1 | (FLAG_INPUT_M4E3 if wa == "m4e3" else 0))
+        acc = LbaFormat(man, 5, bias - 2)
+        for pos in (0, 5, 18):
+            A = torch.zeros(256, 20, dtype=torch.uint8)
+            A[:, pos] = torch.arange(256, dtype=torch.uint8)
+            if wa == "e4m3":
+                A[127, pos] = A[255, pos] = 0  # NaN codes
+            for tile in (0, 2, 3) if pos == 0 else (2,):
+                lba.set_tile_override(tile)
+                try:
+                    for order in (SEQ, CHK):
+                        check_gemm(A, A, prod, acc, order, what=f"{wa} M{man} bias {bias} step {pos} tile {tile}")
+                finally:
+                    lba.set_tile_override(-1)
