@@ -1,4 +1,4 @@
-"""Build ``liblba.so`` (the CUDA library behind the C ABI) in-tree for sm_100a.
+"""Build ``liblba.so`` (the CUDA library behind the C ABI) in-tree for sm_100a, and ``lba_torch.so`` (its calls from PyTorch tensors).
 
 Objects go to ``_build/`` at the repository root (ignored by git); the shared library is written
 next to this file so that it travels with the source tree.  nvcc cross-compiles without a GPU.
@@ -7,6 +7,7 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -14,6 +15,8 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OBJ_DIR = os.path.join(ROOT, "_build", "liblba")
 LIB = os.path.join(HERE, "liblba.so")
+TORCH_SRC = os.path.join(CSRC, "lba_torch.cpp")
+TORCH_LIB = os.path.join(HERE, "lba_torch.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC",
          "-I", os.path.join(ROOT, "include")]
@@ -47,6 +50,26 @@ def _compile(src, verbose):
     return obj
 
 
+def build_torch(force: bool = False) -> str:
+    """The Python module over the library, linked to the liblba.so beside it."""
+    if force or _stale(TORCH_LIB, [TORCH_SRC] + glob.glob(os.path.join(ROOT, "include", "*.h"))):
+        import torch
+        top = os.path.dirname(torch.__file__)
+        cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", TORCH_SRC, "-o", TORCH_LIB + ".tmp",
+               f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+        for inc in (os.path.join(ROOT, "include"), os.path.join(top, "include"),
+                    os.path.join(top, "include", "torch", "csrc", "api", "include"), sysconfig.get_paths()["include"],
+                    os.path.join(os.path.dirname(os.path.dirname(NVCC)), "include")):
+            cmd += ["-I", inc]
+        cmd += ["-L", os.path.join(top, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda",
+                "-L", HERE, "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN"]
+        r = subprocess.run(cmd, capture_output=True, text=True)
+        if r.returncode != 0:
+            raise RuntimeError(f"g++ failed on {TORCH_SRC}:\n{r.stdout}\n{r.stderr}")
+        os.replace(TORCH_LIB + ".tmp", TORCH_LIB)
+    return TORCH_LIB
+
+
 def build(force: bool = False, verbose: bool = False, jobs: int = 0) -> str:
     os.makedirs(OBJ_DIR, exist_ok=True)
     srcs = _sources()
@@ -62,6 +85,7 @@ def build(force: bool = False, verbose: bool = False, jobs: int = 0) -> str:
         if r.returncode != 0:
             raise RuntimeError(f"link failed:\n{r.stdout}\n{r.stderr}")
         os.replace(LIB + ".tmp", LIB)
+    build_torch(force)
     return LIB
 
 

@@ -1,0 +1,70 @@
+"""The native path of the forward entry points against their ctypes path: same results, same refusals."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2401_14110_b200 import binding as lba
+from paper_2401_14110_b200 import synth, code_domain_formats, ORDER_SEQUENTIAL as SEQ, ORDER_CHUNKED as CHK
+
+P, A12 = code_domain_formats(7, 4)
+
+
+def test_irregular_calls_are_left_to_ctypes():
+    lba.load_library()
+    a, one = torch.zeros(4, 16, dtype=torch.uint8), torch.ones(1)
+    assert lba._native.gemm(a, a, one, one, None, P, A12, CHK, 16, None, None) is None          # not on the GPU
+    assert lba._native.gemm(None, a, one, one, None, P, A12, CHK, 16, None, None) is None       # not a tensor
+    assert lba._native.gemm(a, a, one, one, None, P, A12, CHK, 16) is None                      # too few arguments
+    assert lba._native.conv2d(a, a, one, one, None, [1, 1], (0, 0), P, A12, CHK, 16, None, None) is None
+
+
+@pytest.mark.gpu
+def test_native_and_ctypes_paths_agree():
+    dev = "cuda:0"
+    one, sb, bias = torch.ones(1, device=dev), torch.rand(37, device=dev), torch.rand(37, device=dev)
+    a, b = synth.random_codes((3, 21, 48), 1).to(dev), synth.random_codes((3, 37, 48), 2).to(dev)
+    x, w = synth.random_codes((2, 9, 11, 16), 3).to(dev), synth.random_codes((37, 3, 2, 16), 4).to(dev)
+    here = torch.cuda.current_stream()
+    for order in (SEQ, CHK):
+        for pf, af in ((P, A12), (P.as_tuple(), A12.as_tuple())):
+            calls = [(lba.lba_gemm, (a[0], b[0], one, sb, bias, pf, af, order, 16)),
+                     (lba.lba_gemm_batched, (a, b, one, sb, None, pf, af, order, 16)),
+                     (lba.lba_gemm_batched, (a, b[1], one, one, bias, pf, af, order, 16)),
+                     (lba.lba_conv2d, (x, w, one, sb, bias, (2, 1), (1, 0), pf, af, order, 16))]
+            for f, args in calls:
+                want = f(*args, stream=here)            # an explicit stream is the ctypes path's
+                assert lba._native is not None and torch.equal(f(*args).view(torch.int32), want.view(torch.int32))
+                out = torch.empty_like(want)
+                assert f(*args, out=out) is out and torch.equal(out.view(torch.int32), want.view(torch.int32))
+    side = torch.cuda.Stream()
+    side.wait_stream(here)
+    with torch.cuda.stream(side):                       # the current stream is the one that is used
+        got = lba.lba_gemm(a[0], b[0], one, sb, bias, P, A12, CHK, 16)
+    side.synchronize()
+    assert torch.equal(got.view(torch.int32), lba.lba_gemm(a[0], b[0], one, sb, bias, P, A12, CHK, 16, stream=here).view(torch.int32))
+
+
+@pytest.mark.gpu
+def test_what_was_refused_stays_refused():
+    dev = "cuda:0"
+    one = torch.ones(1, device=dev)
+    a, b = synth.random_codes((8, 32), 1).to(dev), synth.random_codes((8, 48), 2).to(dev)
+    with pytest.raises(ValueError):
+        lba.lba_gemm(a, b, one, one, None, P, A12)
+    with pytest.raises(TypeError):
+        lba.lba_gemm(a, b[:, ::2][:, :32], one, one, None, P, A12)             # not contiguous
+    with pytest.raises(TypeError):
+        lba.lba_gemm(a.float(), a, one, one, None, P, A12)
+    with pytest.raises(TypeError):
+        lba.lba_gemm(a, a, one.cpu(), one, None, P, A12)
+    with pytest.raises(lba.LbaError):
+        lba.lba_gemm(a, a, torch.ones(3, device=dev), one, None, P, A12)        # scale length
+    with pytest.raises(lba.LbaError):
+        lba.lba_gemm(a, a, one, one, None, P, A12, 7, 16)                       # order
+    # arguments of other types go on being accepted
+    want = lba.lba_gemm(a, a, one, one, None, P, A12).view(torch.int32)
+    for args in ((torch.nn.Parameter(a, requires_grad=False), a, one, one, None, P, A12, True),
+                 (a, a, one, one, None, list(P.as_tuple()), A12, CHK, np.int64(16))):
+        assert torch.equal(lba.lba_gemm(*args).view(torch.int32), want)
+    x, w = a.view(1, 1, 8, 32), a.view(8, 1, 1, 32)
+    assert torch.equal(lba.lba_conv2d(x, w, one, one, None, [1, 1], [0, 0], P, A12).view(8, 8).view(torch.int32), want)
