@@ -12,19 +12,8 @@ cudaError_t launch(const Problem& p, cudaStream_t stream) {
   auto kernel = lba_contract_packed_kernel<BM, BN, TM, TN, PQ, 0, ORD_CHUNK16, LD, 0, CL, H16>;
   constexpr size_t smem = packed_cluster_smem_bytes<BM, BN, TM, TN>();
   static_assert(smem <= 48 * 1024, "no opt-in needed");
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((p.M + BM - 1) / BM) * CL, (unsigned)((p.N + BN - 1) / BN), (unsigned)p.batch);
-  cfg.blockDim = dim3((BM / TM) * (BN / TN), 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = CL;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, p);
+  const dim3 grid((unsigned)((p.M + BM - 1) / BM) * CL, (unsigned)((p.N + BN - 1) / BN), (unsigned)p.batch);
+  return launch_after(kernel, grid, (BM / TM) * (BN / TN), smem, stream, p, CL);
 }
 
 template <int PQ>

@@ -27,13 +27,8 @@ struct PairSteps {
         prod_k1(pack2(p.prod_k1, p.prod_k1)), prod_k2(pack2(p.prod_k2, p.prod_k2)), mask(p.qa.mask), pmask(p.qp.mask),
         sat(p.qa.sat), psat(p.qp.sat) {}
 
-  __device__ __forceinline__ u64 product(u64 a, u64 b) const { return cut_product(mul2_ftz(b, a)); }
-  __device__ __forceinline__ u64 product(float a, u64 b) const {
-    float b0, b1;
-    unpack2(b, b0, b1);
-    return cut_product(pack2(mul_ftz(a, b0), mul_ftz(a, b1)));
-  }
-  __device__ __forceinline__ u64 cut_product(u64 pr) const {
+  __device__ __forceinline__ u64 product(u64 a, u64 b) const { return cut(mul2_ftz(b, a)); }
+  __device__ __forceinline__ u64 cut(u64 pr) const {
     if (SAT) {
       if (RNE) pr = rne2_fp(pr, prod_k1, prod_k2);
       float lo, hi;
@@ -69,8 +64,8 @@ struct PairSteps {
     }
     return pack2(lo, hi);
   }
-  template <bool CLAMP, typename A>
-  __device__ __forceinline__ u64 step(A a, u64 b, u64 s) const {
+  template <bool CLAMP>
+  __device__ __forceinline__ u64 step(u64 a, u64 b, u64 s) const {
     return add<CLAMP>(product(a, b), s);
   }
   template <bool CLAMP>
@@ -82,48 +77,28 @@ struct PairSteps {
   }
 };
 
-// sixteen bytes of a row -> scaled binary32, k-major in shared memory, `stride` elements from one k to the next (T = float2:
-// every value twice); returns the squared 2-norm, scaled
-__device__ __forceinline__ void put(float2& dst, float v) { dst = make_float2(v, v); }
-__device__ __forceinline__ void put(float& dst, float v) { dst = v; }
-template <typename T>
-__device__ __forceinline__ float stage_row(const Problem& p, const uint4& row, float mul, T* dst, int stride) {
-  const auto store = [&](int k, u64 v) {
-    float s0, s1;
-    unpack2(v, s0, s1);
-    put(dst[k * stride], s0);
-    put(dst[(k + 1) * stride], s1);
-  };
+// sixteen bytes of a row -> scaled binary32, k-major in shared memory, `stride` elements from one k to the next; returns the
+// squared 2-norm, scaled
+__device__ __forceinline__ float stage_row(const Problem& p, const uint4& row, float mul, float* dst, int stride) {
+  const auto store = [&](int k, u64 v) { unpack2(v, dst[k * stride], dst[(k + 1) * stride]); };
   const u64 mul2 = pack2(mul, mul);
   const float n2 = p.in_m4e3 ? decode_row<true>(row, mul2, mul2, store) : decode_row<false>(row, mul2, mul2, store);
   return n2 == 0.0f ? 0.0f : n2 * p.nrm_scale;  // (the scale may be infinite)
 }
 
-// micro-tile operands of one k-step: TM rows from a0, TN columns from b0
+// micro-tile operands of one k-step: TM rows from a0, each as both halves of a factor (see both2), TN columns from b0
 template <int TM, int TN>
-__device__ __forceinline__ void load_step(const float2* a0, const float* b0, u64 (&a)[TM], u64 (&b2)[TN / 2]) {
-#pragma unroll
-  for (int i = 0; i < TM; i += 2) {
-    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(a0 + i);
-    a[i] = v.x;
-    a[i + 1] = v.y;
-  }
+__device__ __forceinline__ void load_step(const float* a0, const float* b0, u64 (&a)[TM], u64 (&b2)[TN / 2]) {
+  static_assert(TM == 2 || TM == 4, "one load");
+  const typename std::conditional<TM == 4, ulonglong2, ulonglong1>::type v = *reinterpret_cast<decltype(&v)>(a0);
+  both2(v.x, a[0], a[1]);
+  if constexpr (TM == 4) both2(v.y, a[2], a[3]);
 #pragma unroll
   for (int j = 0; j < TN; j += 4) {
     const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(b0 + j);
     b2[j / 2] = v.x;
     b2[j / 2 + 1] = v.y;
   }
-}
-template <int TM, int TN>
-__device__ __forceinline__ void load_step(const float* a0, const float* b0, float (&a)[TM], u64 (&b2)[TN / 2]) {
-  static_assert(TM == 2 && TN == 4, "the 16x16 tile");
-  const float2 v = *reinterpret_cast<const float2*>(a0);
-  a[0] = v.x;
-  a[1] = v.y;
-  const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(b0);
-  b2[0] = w.x;
-  b2[1] = w.y;
 }
 
 // back to a real value, +0 for every zero, scales and bias in binary32
@@ -141,12 +116,8 @@ struct SplitShape {
   static constexpr int OUTS = BM * BN / (32 * G) < 2 ? 2 : BM * BN / (32 * G);  // outputs a thread folds
   static constexpr int FOLDERS = BM * BN / OUTS;                                 // threads that fold
   static_assert(OUTS == 2 || OUTS == 4, "consecutive columns of one row");
-  // A is stored twice for the packed multiplier only where a lane's rows are all of one operand; the 16x16 tile decodes
-  // both operands with the same instructions and multiplies with scalar ones (which cost as many issue slots)
-  static constexpr bool TWICE = BM == 32;
-  typedef std::conditional_t<TWICE, float2, float> AT;
-  typedef std::conditional_t<TWICE, u64, float> AReg;
-  static constexpr size_t A_BYTES = sizeof(AT) * BK * BM, B_BYTES = sizeof(float) * BK * BN;
+  static constexpr bool TWO_ROWS = BM == 32;  // a lane decodes a row of A and a row of B, or one of either
+  static constexpr size_t A_BYTES = sizeof(float) * BK * BM, B_BYTES = sizeof(float) * BK * BN;
   static constexpr size_t SMEM = G * (A_BYTES + B_BYTES) + sizeof(float) * 2 * G * BM * BN;
 };
 
@@ -157,7 +128,7 @@ __global__ void __launch_bounds__(32 * G) lba_split_kernel(const Problem p) {
   typedef RowLoader<BM, BN, 32, LD> Loader;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  typename S::AT (*const As)[BM] = reinterpret_cast<typename S::AT (*)[BM]>(smem_raw + w * (S::A_BYTES + S::B_BYTES));
+  float (*const As)[BM] = reinterpret_cast<float (*)[BM]>(smem_raw + w * (S::A_BYTES + S::B_BYTES));
   float (*const Bs)[BN] = reinterpret_cast<float (*)[BN]>(smem_raw + w * (S::A_BYTES + S::B_BYTES) + S::A_BYTES);
   float* const sums = reinterpret_cast<float*>(smem_raw + G * (S::A_BYTES + S::B_BYTES));  // [2][G][BM * BN]
   const int tx = lane % TX, ty = lane / TX;
@@ -167,6 +138,8 @@ __global__ void __launch_bounds__(32 * G) lba_split_kernel(const Problem p) {
   const PairSteps<SAT, RNE> steps(p);
 
   Loader loader;
+  after_previous();
+  next_may_start();
   loader.init(p, lane, m0, n0);
   uint4 raw[Loader::LPT];
   for (int i = 0; i < w; ++i) loader.skip_slab(p);
@@ -181,15 +154,15 @@ __global__ void __launch_bounds__(32 * G) lba_split_kernel(const Problem p) {
     float* const mine = sums + ((q & 1) * G + w) * (BM * BN);
     if (s < nslab) {
       float na = 0.0f, nb = 0.0f;
-      if constexpr (S::TWICE) {
-        static_assert(!S::TWICE || (BM == 32 && BN == 32), "a row of A and a row of B per lane");
+      if constexpr (S::TWO_ROWS) {
+        static_assert(!S::TWO_ROWS || (BM == 32 && BN == 32), "a row of A and a row of B per lane");
         na = stage_row(p, loader.take(p, 0, s, raw[0]), p.pk_a, &As[0][lane], BM);
         nb = stage_row(p, loader.take(p, Loader::LPT - 1, s, raw[Loader::LPT - 1]), p.pk_b, &Bs[0][lane], BN);
       } else {
-        static_assert(S::TWICE || (BM == 16 && BN == 16), "a row of A or of B per lane");
+        static_assert(S::TWO_ROWS || (BM == 16 && BN == 16), "a row of A or of B per lane");
         const bool is_a = lane < BM;
         const float n2 = stage_row(p, loader.take(p, 0, s, raw[0]), is_a ? p.pk_a : p.pk_b,
-                                    reinterpret_cast<float*>(is_a ? (void*)&As[0][lane] : (void*)&Bs[0][lane - BM]), BM);
+                                    is_a ? &As[0][lane] : &Bs[0][lane - BM], BM);
         na = is_a ? n2 : 0.0f;
         nb = is_a ? 0.0f : n2;
       }
@@ -210,8 +183,7 @@ __global__ void __launch_bounds__(32 * G) lba_split_kernel(const Problem p) {
         for (int i = 0; i < TM; ++i)
 #pragma unroll
           for (int j = 0; j < PN; ++j) acc[i][j] = 0ull;
-        typename S::AReg a2[2][TM];
-        u64 b2[2][PN];  // the operands of the next step are on their way while a step is computed
+        u64 a2[2][TM], b2[2][PN];  // the operands of the next step are on their way while a step is computed
         load_step<TM, TN>(&As[0][ty * TM], &Bs[0][tx * TN], a2[0], b2[0]);
 #pragma unroll (CLAMP ? 1 : 4)
         for (int kk = 0; kk < BK; kk += 2) {
@@ -297,6 +269,8 @@ __global__ void __launch_bounds__(CHAIN_THREADS) lba_chain_kernel(const Problem 
   const int nslab = (int)((p.K + BK - 1) / BK);
   const int supers = (nslab + CHAIN_SLABS - 1) / CHAIN_SLABS;
 
+  after_previous();
+  next_may_start();
   if (tid >= 128) {
     const int lane = tid & 31, w = (tid - 128) >> 5;
     Loader loader;
@@ -347,7 +321,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS) lba_chain_kernel(const Problem 
   __syncthreads();
   load(0, 0);
 #pragma unroll
-  for (int i = 0; i < H; ++i) pr[i] = steps.product(a[i], b[i]);
+  for (int i = 0; i < H; ++i) pr[i] = steps.product(pack2(a[i], a[i]), b[i]);
   int slot = 0;
   // whether the clamp can act in a slab (see the packed kernel) is decided while the slab before it runs
   float grow = bound[0];
@@ -369,8 +343,8 @@ __global__ void __launch_bounds__(CHAIN_THREADS) lba_chain_kernel(const Problem 
 #pragma unroll
           for (int i = H / 2; i < H; ++i) {
             acc = steps.template add<CLAMP>(pr[i], acc);
-            nx[2 * i - H] = steps.product(a[2 * i - H], b[2 * i - H]);
-            nx[2 * i - H + 1] = steps.product(a[2 * i - H + 1], b[2 * i - H + 1]);
+#pragma unroll
+            for (int e = 2 * i - H; e < 2 * i - H + 2; ++e) nx[e] = steps.product(pack2(a[e], a[e]), b[e]);
           }
 #pragma unroll
           for (int i = 0; i < H; ++i) pr[i] = nx[i];

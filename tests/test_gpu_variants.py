@@ -1,4 +1,6 @@
 """Kernel variants at the sizes where they can go wrong, against the CPU oracle, bit for bit.  Needs a B200."""
+import gc
+
 import numpy as np
 import pytest
 import torch
@@ -200,3 +202,41 @@ def test_floor_cut_inside_the_operand_scales(wa, man):
                         check_gemm(A, A, prod, acc, order, what=f"{wa} M{man} bias {bias} step {pos} tile {tile}")
                 finally:
                     lba.set_tile_override(-1)
+
+
+@pytest.mark.parametrize("order", [SEQ, CHK])
+@pytest.mark.parametrize("shape", [(33, 64, 64), (700, 640, 64)])
+def test_launches_keep_stream_order(shape, order):
+    # launches that may be set up while the one before them drains: each call reads what the call before it wrote (its sums
+    # as the bias, its buffer as the output of the call after next), in a stream and replayed from a graph
+    M, N, K = shape
+    prod, acc = code_domain_formats(7, 4)
+    a, b, one = synth.random_codes((M, K), 1).to(DEV), synth.random_codes((N, K), 2).to(DEV), torch.ones(1, device=DEV)
+    bufs = [torch.zeros(M, N, device=DEV) for _ in range(2)]
+
+    def chain(steps, sync):
+        for t in range(steps):
+            lba.lba_gemm(a, b, one, one, bufs[t % 2].view(-1)[-N:], prod, acc, order, 16, out=bufs[(t + 1) % 2])
+            if sync:
+                torch.cuda.synchronize()
+        return bufs[steps % 2].clone()
+
+    def reset():
+        for t in bufs:
+            t.zero_()
+
+    want = chain(40, True)
+    for _ in range(5):
+        reset()
+        assert torch.equal(chain(40, False), want)
+    reset()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        got = chain(40, False)
+    for _ in range(3):
+        reset()
+        graph.replay()
+        assert torch.equal(got, want)
+    torch.cuda.synchronize()
+    del graph, got
+    gc.collect()
