@@ -393,14 +393,14 @@ enum CostRow { ROW_SEQ = 0, ROW_CHUNK16 = 1, ROW_CUT_SEQ = 2, ROW_CUT_CHUNK16 = 
                ROW_WIDE_SEQ = 14, ROW_WIDE_LONG = 15, ROW_WIDE_ANY = 16, ROW_COUNT = 17 };
 const TileCost kCost[ROW_COUNT][COST_TILES] = {
     // 128x128, 128x64, 64x64, 32x32, pair, 16x16 chain (sequential) or split, 32x32 split
-    {{0.02, 3.314, 5.3, 0.87}, {0.98, 1.785, 3.8, 0.92}, {0.88, 0.867, 4.3, 1}, {0.71, 0.261, 3.9, 1}, {0, 0, 0, 0}, {0.02, 0.138, 3.4, 1}, {0, 0, 0, 0}},  // floor, sequential
+    {{3.14, 3.23, 3.87, 0.705}, {0.598, 3.77, 3.51, 0.68}, {0.865, 0.856, 1.45, 0.777}, {0.595, 0.228, 5.92, 0.816}, {0, 0, 0, 0}, {0.252, 0.196, 3.02, 0.821}, {0, 0, 0, 0}},  // floor, sequential
     {{2.4, 3.66, 5.8, 0.84}, {1.14, 1.878, 3.5, 0.96}, {0.94, 0.931, 4, 1}, {0.73, 0.28, 3.1, 1}, {1.8, 1.079, 3.4, 1}, {0, 1.863, 2.4, 0.57}, {1.49, 2.437, 2.4, 0.85}},  // floor, chunks of 16
-    {{3.81, 6.691, 3, 1}, {3.08, 3.613, 1.9, 1}, {1.67, 1.822, 3.7, 0.779}, {0.882, 0.506, 2.2, 0.585}, {0, 0, 0, 0}, {0, 0.206, 3.9, 0.85}, {0, 0, 0, 0}},  // floor with product cut, sequential
-    {{2.87, 5.191, 6, 1}, {1.78, 2.756, 3.7, 0.97}, {1.76, 1.37, 4.4, 0.97}, {0.934, 0.392, 3.4, 0.97}, {2.86, 1.551, 3.2, 0.62}, {0, 2.736, 2.6, 0.82}, {2.42, 4.412, 2.9, 0.96}},  // floor with product cut, chunks of 16
+    {{3, 5.536, 6.06, 0.854}, {1.58, 3.147, 4.8, 0.881}, {1.07, 1.121, 4.73, 0.976}, {0.649, 0.32, 3.4, 0.814}, {0, 0, 0, 0}, {0.264, 0.176, 2.25, 0.954}, {0, 0, 0, 0}},  // floor with product cut, sequential
+    {{2.74, 5.811, 7.86, 0.941}, {1.28, 2.804, 4.99, 0.69}, {0.955, 1.147, 5.83, 0.985}, {0.446, 0.3284, 4.22, 0.69}, {1.82, 1.495, 6.12, 0.916}, {0.000185, 2.325, 1.77, 0.883}, {2.28, 3.672, 2.38, 0.982}},  // floor with product cut, chunks of 16
     {{1.9, 4.724, 4.7, 0.98}, {1.49, 2.478, 3.2, 1}, {1.2, 1.277, 2.9, 1}, {0.95, 0.354, 2.1, 1}, {0, 0, 0, 0}, {0.24, 0.145, 2.5, 0.99}, {0, 0, 0, 0}},  // nearest-even, sequential
     {{0.08, 5.151, 4.6, 1}, {0.01, 2.783, 3.2, 1}, {1.25, 1.317, 3.5, 1}, {0.97, 0.365, 3.5, 1}, {0, 0, 0, 0}, {0.01, 1.993, 2.6, 0.68}, {1.8, 2.967, 2.7, 0.9}},  // nearest-even, chunks of 16
     {{0, 4.75, 4.2, 1}, {0.05, 2.575, 3.3, 1}, {1.29, 1.14, 3.9, 1}, {0.95, 0.323, 3, 1}, {0, 0, 0, 0}, {0, 1.972, 2.6, 0.5}, {1.98, 2.766, 2.5, 0.92}},  // nearest-even through bfloat16, chunks of 16
-    {{0, 3.39, 4.56, 1}, {0, 2.08, 4.18, 1}, {1.05, 0.843, 4.45, 1}, {0.703, 0.28, 3.64, 0.973}},  // floor, longer chunks
+    {{0, 3.712, 7.36, 0.948}, {0.969, 2.205, 3.74, 0.761}, {0.871, 0.8876, 3.47, 0.915}, {0.599, 0.2523, 2.61, 0.427}},  // floor, longer chunks
     {{0, 5.16, 4.99, 0.967}, {1.71, 2.6, 4.34, 1}, {1.65, 1.28, 4.82, 1}, {0.89, 0.361, 4.97, 0.834}},  // floor with product cut, longer chunks
     {{0, 5.15, 4.7, 1}, {0, 2.77, 4.11, 1}, {1.17, 1.27, 4.27, 1}, {0.877, 0.36, 3.9, 0.906}},  // nearest-even, longer chunks
     {{0, 7.52, 4.36, 1}, {2.57, 3.76, 3.39, 1}, {2.22, 1.93, 2.73, 0.838}, {1.65, 0.514, 3.3, 1}},  // generic kernel, floor, any chunk length
