@@ -140,23 +140,7 @@ def peak_gmacs(mode, chunk, sm_count, mhz):
 # DRAM bytes (read + write) of ONE launch of the dominant kernel, from an ncu capture summarised under profiles/:
 # (workload, kernel description) -> (bytes, what was captured, executed instructions per emulated MAC).  An entry is taken out
 # when the kernel that it names changes.
-_K_FLOOR = "tile=128x128x16 micro=8x8 q=floor_fast pq=none kernel=packed order=chunk16 load=gemm_vec"
-_CAP = "profiles/packed_floor_kernel_gemm_8192x8192x1024_chunk.txt"
-NCU = {
-    # the headline launch is too long for a capture of many passes (48 ms): the K = 1024 case of the same kernel was
-    # captured; its reads grow in proportion to K (x 8), its writes (the output) do not grow with K
-    ("single_lba_gemm_8192x8192x8192_m7e4_chunk16", _K_FLOOR):
-        (8 * 17448192 + 211388928, "scaled from the 8192x8192x1024 capture (" + _CAP + "): 8 x 17.4 MB read + 211.4 MB written; "
-         "algorithmic 128 MB + 256 MB (part of the output is still in L2 when the kernel ends)", 2.367),
-    ("single_lba_gemm_8192x8192x1024_m7e4_chunk16", _K_FLOOR):
-        (17448192 + 211388928, "17.4 MB read + 211.4 MB written (" + _CAP + "); algorithmic 272 MB", 2.367),
-    ("single_lba_gemm_8192x8192x1024_m7e4_sequential", "tile=128x128x16 micro=8x8 q=floor_fast pq=none kernel=packed order=seq load=gemm_vec"):
-        (18188800 + 211328000, "18.2 MB read + 211.3 MB written (profiles/packed_floor_kernel_gemm_8192x8192x1024_seq.txt)", 2.323),
-    ("single_lba_gemm_8192x8192x1024_m7e4_rne_chunk16", "tile=64x64x16 micro=4x8 q=rne_full pq=none kernel=packed order=chunk16 load=gemm_vec"):
-        (16999424 + 212712960, "17.0 MB read + 212.7 MB written (profiles/packed_nearest_even_kernel_gemm_8192x8192x1024_chunk.txt)", 3.116),
-    ("single_lba_gemm_8192x8192x1024_m8e6_chunk16", "tile=128x128x16 micro=8x8 q=floor_fast pq=fused kernel=packed order=chunk16 load=gemm_vec"):
-        (17105408 + 210696960, "17.1 MB read + 210.7 MB written (profiles/packed_floor_kernel_fused_gemm_8192x8192x1024_chunk.txt)", 1.898),
-}
+NCU = {}
 
 
 def parse_args(argv=None):
