@@ -397,8 +397,8 @@ const TileCost kCost[ROW_COUNT][COST_TILES] = {
     {{2.4, 3.66, 5.8, 0.84}, {1.14, 1.878, 3.5, 0.96}, {0.94, 0.931, 4, 1}, {0.73, 0.28, 3.1, 1}, {1.8, 1.079, 3.4, 1}, {0, 1.863, 2.4, 0.57}, {1.49, 2.437, 2.4, 0.85}},  // floor, chunks of 16
     {{3, 5.536, 6.06, 0.854}, {1.58, 3.147, 4.8, 0.881}, {1.07, 1.121, 4.73, 0.976}, {0.649, 0.32, 3.4, 0.814}, {0, 0, 0, 0}, {0.264, 0.176, 2.25, 0.954}, {0, 0, 0, 0}},  // floor with product cut, sequential
     {{2.74, 5.811, 7.86, 0.941}, {1.28, 2.804, 4.99, 0.69}, {0.955, 1.147, 5.83, 0.985}, {0.446, 0.3284, 4.22, 0.69}, {1.82, 1.495, 6.12, 0.916}, {0.000185, 2.325, 1.77, 0.883}, {2.28, 3.672, 2.38, 0.982}},  // floor with product cut, chunks of 16
-    {{1.9, 4.724, 4.7, 0.98}, {1.49, 2.478, 3.2, 1}, {1.2, 1.277, 2.9, 1}, {0.95, 0.354, 2.1, 1}, {0, 0, 0, 0}, {0.24, 0.145, 2.5, 0.99}, {0, 0, 0, 0}},  // nearest-even, sequential
-    {{0.08, 5.151, 4.6, 1}, {0.01, 2.783, 3.2, 1}, {1.25, 1.317, 3.5, 1}, {0.97, 0.365, 3.5, 1}, {0, 0, 0, 0}, {0.01, 1.993, 2.6, 0.68}, {1.8, 2.967, 2.7, 0.9}},  // nearest-even, chunks of 16
+    {{1.9, 4.724, 4.7, 0.98}, {1.49, 2.478, 3.2, 1}, {1.2, 1.277, 2.9, 1}, {0.95, 0.354, 2.1, 1}, {0, 0, 0, 0}, {0.279, 0.165, 2.18, 0.94}, {0, 0, 0, 0}},  // nearest-even, sequential
+    {{0.08, 5.151, 4.6, 1}, {0.01, 2.783, 3.2, 1}, {1.25, 1.285, 3.5, 1}, {0.97, 0.365, 3.5, 1}, {0, 0, 0, 0}, {0.01, 1.993, 2.6, 0.68}, {1.8, 2.967, 2.7, 0.9}},  // nearest-even, chunks of 16
     {{0, 4.75, 4.2, 1}, {0.05, 2.575, 3.3, 1}, {1.29, 1.14, 3.9, 1}, {0.95, 0.323, 3, 1}, {0, 0, 0, 0}, {0, 1.972, 2.6, 0.5}, {1.98, 2.766, 2.5, 0.92}},  // nearest-even through bfloat16, chunks of 16
     {{0, 3.712, 7.36, 0.948}, {0.969, 2.205, 3.74, 0.761}, {0.871, 0.8876, 3.47, 0.915}, {0.599, 0.2523, 2.61, 0.427}},  // floor, longer chunks
     {{0, 5.16, 4.99, 0.967}, {1.71, 2.6, 4.34, 1}, {1.65, 1.28, 4.82, 1}, {0.89, 0.361, 4.97, 0.834}},  // floor with product cut, longer chunks
