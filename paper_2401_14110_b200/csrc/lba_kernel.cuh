@@ -316,15 +316,16 @@ __device__ __forceinline__ u64 add2_rz_ftz(u64 a, u64 b) {
 // Kernels that begin with after_previous() are launched by launch_after: the grid may be set up while the kernel before it in
 // the stream drains, and every CTA waits there, before its first access to global memory, until that kernel has completed and
 // its writes are visible.  Stream order is what it was; what is saved is the gap between two launches (empty kernels follow
-// each other every 0.6 us instead of 2.1, at the same host time).  A kernel of small problems, one or two CTAs per SM, lets its
-// successor's CTAs in from its start (next_may_start): 64 x 64 x 576 sequential, launch after launch, 12.3 to 11.1 us.  The
-// packed kernel does not: its successor's CTAs would settle where SMs have room at that moment and stay unevenly spread
-// (1111 x 777 x 1203 took 193 us instead of 125, ResNet-18 6.97 ms instead of 6.23; from the epilogue on 129 us and 6.38 ms).
-// Let in when it ends, as now: 125 us, 6.20 ms; attention of 384 heads 94.4 to 90.7 us; ResNet-50 on M4E3 bytes 10.47 to 10.37 ms.
+// each other every 0.6 us instead of 2.1, at the same host time): attention of 384 heads 94.4 to 90.7 us, ResNet-50 on M4E3 bytes
+// 10.47 to 10.37 ms.  A kernel's CTAs are let in as its predecessor's end, never earlier (griddepcontrol.launch_dependents): waiting
+// CTAs would settle where SMs have room at that moment and stay unevenly spread.  Let in from the predecessor's start, 32 x 1000 x
+// 512 in chunks of 16 and sequentially in turn took 34.9 us instead of 15.0, 128 x 1000 x 512 sequentially behind itself 29.3
+// instead of 20.3, a 64x64 tile on 148 SMs behind the classifier of 64 rows 117 us instead of 47.7, 1111 x 777 x 1203 behind
+// itself 193 instead of 125 (from the epilogue on: 129).  With at most one CTA per SM the chain and split kernels still lost up
+// to 57 % that way before another kernel and gained less than 3 % anywhere.
 __device__ __forceinline__ void after_previous() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
-__device__ __forceinline__ void next_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 inline cudaError_t launch_after(void (*kernel)(const Problem), dim3 grid, int threads, size_t smem, cudaStream_t stream, const Problem& p,
                                 int cluster = 1) {
   cudaLaunchConfig_t cfg = {};

@@ -139,7 +139,6 @@ __global__ void __launch_bounds__(32 * G) lba_split_kernel(const Problem p) {
 
   Loader loader;
   after_previous();
-  next_may_start();
   loader.init(p, lane, m0, n0);
   uint4 raw[Loader::LPT];
   for (int i = 0; i < w; ++i) loader.skip_slab(p);
@@ -270,7 +269,6 @@ __global__ void __launch_bounds__(CHAIN_THREADS) lba_chain_kernel(const Problem 
   const int supers = (nslab + CHAIN_SLABS - 1) / CHAIN_SLABS;
 
   after_previous();
-  next_may_start();
   if (tid >= 128) {
     const int lane = tid & 31, w = (tid - 128) >> 5;
     Loader loader;
