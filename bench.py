@@ -46,8 +46,9 @@ MIX = {
     # mode: (issue, logic, packed_fp, scalar_fp, text)
     "floor": (2.0, 1.0, 1.0, 0.0, "0.5 FMUL2 + 0.5 FFMA2 + 1 LOP3"),
     "floor_cut": (2.5, 1.0, 1.5, 0.0, "0.5 FMUL2 + 0.5 FFMA2 (product and its cut, from two scalings of A) + 0.5 FFMA2 + 1 LOP3"),
-    "floor_cut_sat": (4.0, 2.5, 1.5, 0.0, "as floor, the product cut by 1 LOP3 in one register pair and by 0.5 FMUL2 + 0.5 FFMA2 in "
-                                          "the next, plus 1 FMNMX for its saturation"),
+    "floor_cut_any": (3.0, 1.5, 1.5, 0.0, "as floor, the product cut by 1 LOP3 in one register pair and by 0.5 FMUL2 + 0.5 FFMA2 in "
+                                          "the next"),
+    "floor_cut_sat": (4.0, 2.5, 1.5, 0.0, "as floor_cut_any, plus 1 FMNMX for the product's saturation"),
     "floor_fused": (1.5, 1.0, 0.5, 0.0, "0.5 FFMA2 (product and sum in one instruction) + 1 LOP3"),
     "rne": (2.0, 0.0, 2.0, 0.0, "0.5 FMUL2 + 0.5 FFMA2 + 0.5 FMUL2 + 0.5 FFMA2 (rounding on the FP32 pipe)"),
     "rne_bf16": (2.5, 1.0, 1.0, 0.0, "0.5 FMUL2 + 0.5 FFMA2 + 0.5 F2FP (rounding to bfloat16) + 0.5 SHL + 0.5 LOP3"),
@@ -114,7 +115,7 @@ def mode_of(desc: str, ste=None, fixed=False, acc_man_bits=None) -> str:
     q, pq = f.get("q", ""), f.get("pq", "none")
     if "by" in f:  # a small-problem kernel runs, with a product mode of its own
         pq = f["by"].rpartition("pq=")[2].rstrip(")")
-    suffix = {"none": "", "cut": "_cut", "cut_sat": "_cut_sat", "fused": "_fused"}.get(pq, "")
+    suffix = {"none": "", "cut": "_cut", "cut_any": "_cut_any", "cut_sat": "_cut_sat", "fused": "_fused"}.get(pq, "")
     if f.get("kernel") == "generic" and q != "rne_wide":
         return "generic"
     if q.startswith("floor"):

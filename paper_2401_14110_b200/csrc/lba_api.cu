@@ -328,7 +328,7 @@ int make_plan(const lba_fmt* pf, const lba_fmt* af, int order, int chunk, int64_
 
   // ---- floor cut of the product inside A's scales (see cut_product): x (1 + 2^s) must fit 24 bits beside x's own 4 (E4M3) or 5
   // (M4E3), s = 23 - M_prod, and x times 2^s must stay a binary32 number.  Where it does not, the kernel with the general
-  // cut runs, whose saturation is then a no-op.
+  // cut runs (PQ_CUT_ANY).
   pl->cut_a = pl->cut_a0 = pl->cut_ratio = 0.0f;
   if (pl->pq == PQ_MASK && !nearest) {
     const int s = 23 - pf->man_bits, top = 9 + s + (sx > sx + ka - kp ? sx : sx + ka - kp);
@@ -337,7 +337,7 @@ int make_plan(const lba_fmt* pf, const lba_fmt* af, int order, int chunk, int64_
       pl->cut_a0 = pl->pk_a0 * pl->prod_k2;
       pl->cut_ratio = pl->prod_k1 / pl->prod_k2;
     } else {
-      pl->pq = PQ_MASK_SAT;
+      pl->pq = PQ_CUT_ANY;
     }
   }
 
@@ -1009,7 +1009,7 @@ int lba_describe_plan_batched(int64_t batch, int64_t M, int64_t N, int64_t K, co
                       (pl.qm == QM_FLOOR_FAST || pl.qm == QM_FLOOR_FULL || (pl.qm == QM_RNE_FULL && pl.rne_packed));
   const char* const kern = packed ? "packed" : "generic";
   const char* const plain_pq = pl.qm == QM_FLOOR_FAST || pl.qm == QM_RNE_WIDE ? "none"
-                               : pl.pq == PQ_MASK_SAT ? "cut_sat" : pl.pq == PQ_MASK ? "cut" : "none";
+                               : pl.pq == PQ_MASK_SAT ? "cut_sat" : pl.pq == PQ_CUT_ANY ? "cut_any" : pl.pq == PQ_MASK ? "cut" : "none";
   const char* const pq = pl.fused && packed && tile < TILE_PAIR ? "fused" : plain_pq;
   char by[112] = "";
   if (small) {  // these have no fused variant

@@ -34,6 +34,7 @@ cudaError_t launch_cluster_pair(int pq, int load, const Problem& p, cudaStream_t
   switch (pq) {
     case PQ_NONE: return by_loader<PQ_NONE>(load, p, stream);
     case PQ_MASK: return by_loader<PQ_MASK>(load, p, stream);
+    case PQ_CUT_ANY: return by_loader<PQ_CUT_ANY>(load, p, stream);
     default: return by_loader<PQ_MASK_SAT>(load, p, stream);
   }
 }

@@ -39,6 +39,7 @@ cudaError_t by_product(bool small, int pq, int load, const Problem& p, cudaStrea
   switch (pq) {
     case PQ_NONE: return by_loader<PQ_NONE, ORD>(small, load, p, stream);
     case PQ_MASK: return by_loader<PQ_MASK, ORD>(small, load, p, stream);
+    case PQ_CUT_ANY: return by_loader<PQ_CUT_ANY, ORD>(small, load, p, stream);
     default: return by_loader<PQ_MASK_SAT, ORD>(small, load, p, stream);
   }
 }

@@ -949,7 +949,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), TRACK == TRACK_MASK_DIF
 // B-row norms of the slab give one bound per CTA, and each thread carries an upper bound `u` of
 // its own |S| (as a fraction of 2^(e_max+1)), refreshed from the registers when it gets too loose.
 // A warp whose bound fails runs the same slab with the clamp.  Results are identical either way.
-// Under floor rounding with a product cut in which the product can saturate too the logic pipe binds (four masks per pair and
+// Under floor rounding with a product cut that A's scales do not carry the logic pipe binds (four masks and clamps per pair and
 // step).  Every second register pair of a micro-tile row (j % 2 == FP_CUT) therefore cuts its product on the FP32 pipe.
 constexpr int FP_CUT = 1;
 constexpr int KUNROLL = 16;  // k-steps unrolled in the packed slab body (the whole slab: measured fastest)
@@ -1056,12 +1056,13 @@ __host__ __device__ constexpr int packed_tmem_cols() {
 // 25088 x 64 x 147 in chunks of 32, M5E5: 6.5 % slower than with masks alone, 77 us against 59 with the bound (401408 rows 807, 682;
 // 16384 x 64 x 216, one CTA per SM in any case, 53.1, 54.1 and 54.7 with masks alone).  The other modes would lose up to 7 % on that last shape.
 // PQ: what Q_prod has to do beyond the flush (the host proves which cases are reachable): nothing, cut the mantissa (M_prod < 7;
-// under floor rounding where A's scales can carry the cut, M_prod >= 3 or 4), or cut and saturate (448^2 >= R_OF_prod, and the
-// floor cuts to fewer bits, whose saturation is a no-op)
+// under floor rounding where A's scales can carry the cut, M_prod >= 3 or 4), or cut and saturate (448^2 >= R_OF_prod).
+// PQ_CUT_ANY (floor only): cut to fewer bits than A's scales can carry, as in PQ_MASK_SAT but without the clamp.  4096^3, M2E5 on
+// E4M3 bytes: sequential 7.84 ms, chunks of 16 8.04, of 32 8.17; with the clamp as a no-op 11.2, 11.4, 11.4.
 // PQ_FUSED: Q_prod is the identity on every reachable product (no cut, no saturation, and no product can fall under
 // R_UF_prod), so FMAq(x, w, S) = Q_acc(x w + S) and the product needs no instruction of its own: one packed FMA forms the
 // exact product and the sum; the B operand then carries the accumulator's scaling.
-enum PackedProd { PQ_NONE = 0, PQ_MASK = 1, PQ_MASK_SAT = 2, PQ_FUSED = 3 };
+enum PackedProd { PQ_NONE = 0, PQ_MASK = 1, PQ_MASK_SAT = 2, PQ_FUSED = 3, PQ_CUT_ANY = 4 };
 
 // RNE: nearest-even instead of floor, 1 = any M <= 10, 2 = M_acc = 7 (then PQ_MASK means "round the product to M_prod bits").  Nearest-even
 // can raise a magnitude by half a grid step per rounding, so the slab-level proof that the clamp is idle carries a
@@ -1085,11 +1086,12 @@ enum PackedProd { PQ_NONE = 0, PQ_MASK = 1, PQ_MASK_SAT = 2, PQ_FUSED = 3 };
 template <int BM, int BN, int TM, int TN, int PQ, int RNE, int ORD, int LD, int STE = 0, int CL = 1, bool H16 = false>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN),
                                   ((TM * TN == 64 && ORD != ORD_CHUNK_SLAB && !RNE) || (TM * TN == 32 && ORD == ORD_CHUNK16) ||
-                                   (TM * TN == 32 && ORD == ORD_CHUNK_SLAB && LD == LD_CONV_ANY && (PQ == PQ_MASK || PQ == PQ_MASK_SAT) && !RNE) ||
+                                   (TM * TN == 32 && ORD == ORD_CHUNK_SLAB && LD == LD_CONV_ANY && (PQ == PQ_MASK || PQ == PQ_MASK_SAT || PQ == PQ_CUT_ANY) && !RNE) ||
                                    ((LD == LD_CONV_ANY || LD == LD_GEMM_ROWS || STE != 0) && !RNE && ORD != ORD_CHUNK_SLAB))
                                       ? 512 / ((BM / TM) * (BN / TN)) : 1)
     lba_contract_packed_kernel(const Problem p) {
   static_assert(STE == 0 || (!RNE && TM == 4 && (ORD == ORD_SEQ || ORD == ORD_CHUNK16)), "mask variant");
+  static_assert(!RNE || PQ != PQ_CUT_ANY, "nearest-even has one cut");
   static_assert(CL == 1 || LD == LD_GEMM_VEC || LD == LD_CONV_VEC, "a CTA of the pair skips slabs");
   static_assert(CL == 1 || (CL == 2 && !RNE && STE == 0 && ORD == ORD_CHUNK16 && TM == 4), "cluster variant");
   constexpr int NT = (BM / TM) * (BN / TN);
@@ -1240,7 +1242,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
         auto product = [&](int i, int j) -> u64 {
           if constexpr (CUT) return cut_product(b2[j], a1[i], a2[i]);
           u64 pr = mul2_ftz(b2[j], a2[i]);
-          if (PQ == PQ_MASK_SAT) {  // floor of Eq. 2 on the exact product, then its saturation
+          if (PQ == PQ_MASK_SAT || PQ == PQ_CUT_ANY) {  // floor of Eq. 2 on the exact product, then its saturation
             float plo, phi;
             if (j % 2 == FP_CUT) pr = floor2_fp(pr, prod_k1, prod_k2);
             unpack2(pr, plo, phi);
@@ -1248,7 +1250,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
               plo = and_bits(plo, pmask);
               phi = and_bits(phi, pmask);
             }
-            pr = pack2(clamp_mag(plo, psat), clamp_mag(phi, psat));
+            pr = PQ == PQ_MASK_SAT ? pack2(clamp_mag(plo, psat), clamp_mag(phi, psat)) : pack2(plo, phi);
           }
           return pr;
         };
@@ -1312,7 +1314,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN),
         // The order of the pairs, as measured (8192 x 8192 x 1024, M7E4, clocks per warp-MAC).  Chunks of 16: pair after pair, along
         // a row and back along the next one (so that neighbours share a factor): 3.05 on the 64x64 tile and 3.14 on 128x64,
         // 3.12 and 3.22 with the products one row ahead of the sums; down the columns of the 8x8 micro-tile: 3.03, 3.08.
-        // Sequentially, and beside the logic instructions of a saturating product, one row ahead: 2.95 against 2.97 to 3.00.
+        // Sequentially, and beside the logic instructions of a cut of its own, one row ahead: 2.95 against 2.97 to 3.00.
         // A cut product along the rows in every order (4.29 on 64x64, 4.39 one row ahead; sequentially 4.13, 4.14).
         if constexpr ((CH16 && PQ == PQ_NONE) || CUT) {
           if constexpr (TM == 8 && !CUT) {

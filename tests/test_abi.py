@@ -9,7 +9,7 @@ import pytest
 import torch
 
 from paper_2401_14110_b200 import binding as lba
-from paper_2401_14110_b200 import LbaFormat, code_domain_formats, ORDER_CHUNKED as CHK, ORDER_SEQUENTIAL as SEQ
+from paper_2401_14110_b200 import FLAG_INPUT_M4E3, LbaFormat, code_domain_formats, ORDER_CHUNKED as CHK, ORDER_SEQUENTIAL as SEQ
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
@@ -209,6 +209,19 @@ def test_plan_names_the_small_kernel_that_runs():
             assert by((49, 512, 4608), f, SEQ, is_conv=True) == f"chain16x16(micro=1x2,grid=4x32,pq={pq})"
             assert by((4096, 4096, 4096), f, CHK) == by((4096, 4096, 4096), f, SEQ) == by((64, 64, 576), f, CHK, 32) == ""
     assert by((512, 768, 768), code_domain_formats(7, 4), CHK) == "split32x32(micro=4x8,grid=16x24,pq=none)"
+
+
+def test_cuts_too_short_for_the_operand_scales_run_without_a_clamp():
+    # x (1 + 2^(23 - M)) must fit 24 bits beside x's own: M >= 3 on E4M3 bytes, M >= 4 on M4E3.  Below that the product is cut by
+    # itself; only one that can saturate (R_OF_prod <= 448^2, 248^2) is clamped too
+    import bench
+    a = code_domain_formats(7, 4)[1]
+    for order, chunk in ((SEQ, 16), (CHK, 16), (CHK, 32)):
+        for flags, fits, bias in ((1, 3, 14), (1 | FLAG_INPUT_M4E3, 4, 15)):   # biases at which nothing of 2 bits and more saturates
+            for man, more, want in ((fits, 0, "cut"), (fits - 1, 0, "cut_any"), (2, 0, "cut_any"), (2, 4, "cut_sat")):
+                plan = lba.describe_plan(4096, 4096, 4096, LbaFormat(man, 5, bias + more, 0, flags), a, order, chunk)
+                assert re.search(r"pq=(\w+)", plan)[1] == want and bench.mode_of(plan) == "floor_" + want, (man, more, plan)
+    assert bench.min_issue_slots("floor_cut_any", 0) == 3.0
 
 
 def test_benchmark_mix_is_that_of_the_kernel_that_runs():

@@ -204,6 +204,41 @@ def test_floor_cut_inside_the_operand_scales(wa, man):
                     lba.set_tile_override(-1)
 
 
+@pytest.mark.parametrize("order,chunk", [(SEQ, 16), (CHK, 16), (CHK, 32)])
+@pytest.mark.parametrize("prod,acc", [(LbaFormat(2, 5, 14), LbaFormat(2, 5, 12)),
+                                      (LbaFormat(3, 6, 47, 0, 1 | FLAG_INPUT_M4E3), LbaFormat(3, 6, 45))], ids=["e4m3", "m4e3"])
+def test_short_cuts_without_saturation(prod, acc, order, chunk):
+    # mantissas that A's scales cannot carry, of products that cannot saturate: every tile and loader, and the overflow masks
+    assert "pq=cut_any" in lba.describe_plan(4096, 4096, 4096, prod, acc, order, chunk)
+    fmts = prod.as_tuple(), acc.as_tuple()
+    one, any_code = torch.ones(1), lambda *shape: synth.random_codes(shape, sum(shape))
+    gemms = [(any_code(70, K), any_code(67, K)) for K in (33, 112)]
+    convs = [(any_code(2, 9, 7, C), any_code(67, 3, 3, C)) for C in (3, 16)]
+    want = [orc.gemm(a.numpy(), b.numpy(), one.numpy(), one.numpy(), None, *fmts, order, chunk) for a, b in gemms]
+    want += [orc.conv2d(x.numpy(), w.numpy(), one.numpy(), one.numpy(), None, (1, 1), (1, 1), *fmts, order, chunk) for x, w in convs]
+    d = one.to(DEV)
+    for tile in (-1, 0, 1, 2, 3) + ((5,) if order == CHK and chunk == 16 else ()):
+        lba.set_tile_override(tile)
+        try:
+            got = [lba.lba_gemm(a.to(DEV), b.to(DEV), d, d, None, prod, acc, order, chunk) for a, b in gemms]
+            got += [lba.lba_conv2d(x.to(DEV), w.to(DEV), d, d, None, (1, 1), (1, 1), prod, acc, order, chunk) for x, w in convs]
+        finally:
+            lba.set_tile_override(-1)
+        for g, w in zip(got, want):
+            assert (g.cpu().numpy().view(np.uint32) == w.view(np.uint32)).all(), (tile, w.shape)
+    if prod.flags == 1 and chunk == 16:
+        for a, b in gemms:
+            w1, w2 = orc.gemm_ste_mask(a.numpy(), b.numpy(), *fmts, order, chunk, orc.STE_OF, 0.0, 0.0)
+            for tile in (2, 7):
+                lba.set_tile_override(tile)
+                try:
+                    masks = lba.lba_gemm_ste_mask(a.to(DEV), b.to(DEV), prod, acc, order, chunk, lba.STE_OF)
+                finally:
+                    lba.set_tile_override(-1)
+                for g, w in zip(masks, (w1, w2)):
+                    assert (g is None) == (w is None) and (g is None or (g.cpu().numpy().view(np.uint32) == w).all())
+
+
 @pytest.mark.parametrize("order", [SEQ, CHK])
 @pytest.mark.parametrize("shape", [(33, 64, 64), (700, 640, 64)])
 def test_launches_keep_stream_order(shape, order):
