@@ -1,8 +1,9 @@
-"""Thin ctypes binding of ``liblba.so`` (C ABI declared in ``include/lba.h``).
+"""Thin binding of ``liblba.so`` (C ABI declared in ``include/lba.h``), through ctypes.
 
 The forward entry points hand a regular call (plain contiguous tensors of the current device, its current stream) to
 ``lba_torch.so``, which makes the same checks and the same C call in 4 us of host time instead of 10 to 12; everything else, and
-every error, takes the ctypes path.
+every error, takes the ctypes path.  So do all calls, after one warning, where that module is missing or was built for another
+torch or interpreter.
 
 Argument marshalling only: PyTorch supplies device memory and the current stream; every step of
 the computation runs in the CUDA kernels behind the C entry points.  There is no fallback: if the
@@ -11,9 +12,11 @@ library is missing, or a call returns an error, an exception is raised.
 import ctypes as C
 import importlib.util
 import os
+import warnings
 
 import torch
 
+from .build import torch_tag
 from .formats import LbaFormat, ORDER_CHUNKED, PAPER_CHUNK
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
@@ -38,7 +41,23 @@ class _Fmt(C.Structure):
 
 
 _lib = None
-_native = None  # lba_torch.so
+_native = None  # lba_torch.so, or None where it cannot be used
+
+
+def _load_native():
+    """lba_torch.so, or None with a warning: every call then takes the ctypes path, which needs nothing but the library."""
+    try:
+        spec = importlib.util.spec_from_file_location("lba_torch", TORCH_LIB_PATH)
+        native = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(native)
+        if native.built_for != torch_tag():
+            raise ImportError(f"built for {native.built_for!r}, this is {torch_tag()!r}")
+        native.init(LbaFormat)
+        return native
+    except (ImportError, OSError, AttributeError, TypeError) as e:
+        warnings.warn(f"{TORCH_LIB_PATH} cannot be used, calls go through ctypes (6 to 8 us more of host time each); build it with "
+                      f"`python -m paper_2401_14110_b200.build`: {e}", RuntimeWarning, stacklevel=3)
+        return None
 
 
 def load_library():
@@ -46,10 +65,9 @@ def load_library():
     global _lib, _native
     if _lib is not None:
         return _lib
-    for path in (LIB_PATH, TORCH_LIB_PATH):
-        if not os.path.exists(path):
-            raise RuntimeError(f"{path} is missing: build it with `python -m paper_2401_14110_b200.build` "
-                               "(there is no CPU or PyTorch fallback)")
+    if not os.path.exists(LIB_PATH):
+        raise RuntimeError(f"{LIB_PATH} is missing: build it with `python -m paper_2401_14110_b200.build` "
+                           "(there is no CPU or PyTorch fallback)")
     lib = C.CDLL(LIB_PATH)
     lib.lba_status_string.restype = C.c_char_p
     lib.lba_status_string.argtypes = [C.c_int]
@@ -78,11 +96,7 @@ def load_library():
     lib.lba_describe_plan_batched.argtypes = [C.c_int64] + lib.lba_describe_plan.argtypes
     for name in EXPORTS:
         getattr(lib, name)
-    spec = importlib.util.spec_from_file_location("lba_torch", TORCH_LIB_PATH)
-    native = importlib.util.module_from_spec(spec)
-    spec.loader.exec_module(native)
-    native.init(LbaFormat)
-    _native = native
+    _native = _load_native()
     _lib = lib
     return lib
 
@@ -156,7 +170,7 @@ def lba_gemm(A, B, scale_a, scale_b, bias, prod_fmt, acc_fmt, order=ORDER_CHUNKE
              stream=None):
     """out[M][N] (float32, CUDA) for A [M][K], B [N][K] E4M3 bytes on the GPU.  See ``lba_gemm`` in lba.h."""
     lib = load_library()
-    done = _native.gemm(A, B, scale_a, scale_b, bias, prod_fmt, acc_fmt, order, chunk, out, stream)
+    done = _native and _native.gemm(A, B, scale_a, scale_b, bias, prod_fmt, acc_fmt, order, chunk, out, stream)
     if done is not None:
         return _done(done)
     M, K = A.shape
@@ -177,7 +191,7 @@ def lba_gemm_batched(A, B, scale_a, scale_b, bias, prod_fmt, acc_fmt, order=ORDE
                      stream=None):
     """out[Z][M][N] for A [Z][M][K] and B [Z][N][K] (or [N][K], shared by all Z problems).  See lba.h."""
     lib = load_library()
-    done = _native.gemm_batched(A, B, scale_a, scale_b, bias, prod_fmt, acc_fmt, order, chunk, out, stream)
+    done = _native and _native.gemm_batched(A, B, scale_a, scale_b, bias, prod_fmt, acc_fmt, order, chunk, out, stream)
     if done is not None:
         return _done(done)
     Z, M, K = A.shape
@@ -246,7 +260,7 @@ def lba_conv2d(x, w, scale_x, scale_w, bias, stride, pad, prod_fmt, acc_fmt, ord
                out=None, stream=None):
     """out [B][Hout][Wout][Cout] for x [B][H][W][Cin], w [Cout][KH][KW][Cin] E4M3 bytes.  See lba.h."""
     lib = load_library()
-    done = _native.conv2d(x, w, scale_x, scale_w, bias, stride, pad, prod_fmt, acc_fmt, order, chunk, out, stream)
+    done = _native and _native.conv2d(x, w, scale_x, scale_w, bias, stride, pad, prod_fmt, acc_fmt, order, chunk, out, stream)
     if done is not None:
         return _done(done)
     B, H, W, Cin = x.shape

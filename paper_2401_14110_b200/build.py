@@ -8,6 +8,7 @@ import os
 import subprocess
 import sys
 import sysconfig
+import warnings
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -50,13 +51,25 @@ def _compile(src, verbose):
     return obj
 
 
+def torch_tag() -> str:
+    """What lba_torch.so is built for; it carries this text (``built_for``) and runs with no other torch or interpreter."""
+    import torch
+    return f"lba_torch for torch {torch.__version__} {sys.implementation.cache_tag}"
+
+
+def _carries(path, text) -> bool:
+    with open(path, "rb") as f:
+        return text.encode() in f.read()
+
+
 def build_torch(force: bool = False) -> str:
     """The Python module over the library, linked to the liblba.so beside it."""
-    if force or _stale(TORCH_LIB, [TORCH_SRC] + glob.glob(os.path.join(ROOT, "include", "*.h"))):
+    tag = torch_tag()
+    if force or _stale(TORCH_LIB, [TORCH_SRC] + glob.glob(os.path.join(ROOT, "include", "*.h"))) or not _carries(TORCH_LIB, tag):
         import torch
         top = os.path.dirname(torch.__file__)
         cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", TORCH_SRC, "-o", TORCH_LIB + ".tmp",
-               f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+               f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", f'-DLBA_TORCH_TAG="{tag}"']
         for inc in (os.path.join(ROOT, "include"), os.path.join(top, "include"),
                     os.path.join(top, "include", "torch", "csrc", "api", "include"), sysconfig.get_paths()["include"],
                     os.path.join(os.path.dirname(os.path.dirname(NVCC)), "include")):
@@ -85,7 +98,10 @@ def build(force: bool = False, verbose: bool = False, jobs: int = 0) -> str:
         if r.returncode != 0:
             raise RuntimeError(f"link failed:\n{r.stdout}\n{r.stderr}")
         os.replace(LIB + ".tmp", LIB)
-    build_torch(force)
+    try:
+        build_torch(force)
+    except (OSError, RuntimeError) as e:  # no g++, or a torch without CUDA: the library is complete without the module
+        warnings.warn(f"lba_torch.so was not built, calls will go through ctypes: {e}")
     return LIB
 
 

@@ -231,4 +231,11 @@ PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "lba_torch", nullptr, -1, kMethods
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit_lba_torch() { return PyModule_Create(&kModule); }
+PyMODINIT_FUNC PyInit_lba_torch() {
+  PyObject* const m = PyModule_Create(&kModule);
+  if (m && PyModule_AddStringConstant(m, "built_for", LBA_TORCH_TAG) != 0) {
+    Py_DECREF(m);
+    return nullptr;
+  }
+  return m;
+}

@@ -6,6 +6,7 @@ import pytest
 import torch
 
 from paper_2401_14110_b200 import binding as lba
+from paper_2401_14110_b200 import build as lba_build
 from paper_2401_14110_b200 import synth, code_domain_formats, ORDER_SEQUENTIAL as SEQ, ORDER_CHUNKED as CHK
 
 P, A12 = code_domain_formats(7, 4)
@@ -25,6 +26,64 @@ def test_irregular_calls_are_left_to_ctypes():
     assert lba._native.gemm(None, a, one, one, None, P, A12, CHK, 16, None, None) is None       # not a tensor
     assert lba._native.gemm(a, a, one, one, None, P, A12, CHK, 16) is None                      # too few arguments
     assert lba._native.conv2d(a, a, one, one, None, [1, 1], (0, 0), P, A12, CHK, 16, None, None) is None
+
+
+@pytest.fixture
+def reloaded():
+    """The binding as a fresh process finds it; the library as it was loaded afterwards."""
+    lib, native, path = lba.load_library(), lba._native, lba.TORCH_LIB_PATH
+    lba._lib = lba._native = None
+    yield
+    lba._lib, lba._native, lba.TORCH_LIB_PATH = lib, native, path
+
+
+def _without_native():
+    with pytest.warns(RuntimeWarning, match="ctypes"):
+        lba.load_library()
+    assert lba._native is None
+    assert "q=floor_fast" in lba.describe_plan(64, 64, 576, P, A12, CHK, 16)
+    a, one = torch.zeros(4, 16, dtype=torch.uint8), torch.ones(1)
+    with pytest.raises(TypeError):                      # reached the checks of the ctypes path
+        lba.lba_gemm(a, a, one, one, None, P, A12, CHK, 16)
+
+
+def test_without_the_native_module_calls_go_through_ctypes(reloaded, tmp_path):
+    lba.TORCH_LIB_PATH = str(tmp_path / "lba_torch.so")
+    _without_native()
+
+
+def test_a_native_module_that_cannot_be_imported_is_left_out(reloaded, tmp_path):
+    (tmp_path / "lba_torch.so").write_bytes(b"not a shared library")
+    lba.TORCH_LIB_PATH = str(tmp_path / "lba_torch.so")
+    _without_native()
+
+
+def test_a_native_module_of_another_torch_is_left_out_and_rebuilt(reloaded, monkeypatch):
+    assert lba_build._carries(lba_build.TORCH_LIB, lba_build.torch_tag())
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    _without_native()
+    assert not lba_build._carries(lba_build.TORCH_LIB, lba_build.torch_tag())    # a build now compiles it anew
+
+
+def test_a_failed_build_of_the_native_module_leaves_the_library(monkeypatch):
+    def fail(force):
+        raise RuntimeError("no compiler")
+    monkeypatch.setattr(lba_build, "build_torch", fail)
+    monkeypatch.setattr(lba_build, "_sources", lambda: [])
+    monkeypatch.setattr(lba_build, "_stale", lambda target, sources: False)
+    with pytest.warns(UserWarning, match="no compiler"):
+        assert lba_build.build() == lba_build.LIB
+
+
+@pytest.mark.gpu
+def test_forward_calls_without_the_native_module(reloaded, tmp_path):
+    a, one = synth.random_codes((20, 48), 1).to("cuda:0"), torch.ones(1, device="cuda:0")
+    want = lba.lba_gemm(a, a, one, one, None, P, A12)
+    lba._lib = lba._native = None
+    lba.TORCH_LIB_PATH = str(tmp_path / "lba_torch.so")
+    with pytest.warns(RuntimeWarning):
+        got = lba.lba_gemm(a, a, one, one, None, P, A12)
+    assert lba._native is None and torch.equal(got.view(torch.int32), want.view(torch.int32))
 
 
 @pytest.mark.gpu
