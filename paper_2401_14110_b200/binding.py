@@ -52,7 +52,7 @@ def _load_native():
         spec.loader.exec_module(native)
         if native.built_for != torch_tag():
             raise ImportError(f"built for {native.built_for!r}, this is {torch_tag()!r}")
-        native.init(LbaFormat)
+        native.init(LbaFormat, torch.nn.Parameter)
         return native
     except (ImportError, OSError, AttributeError, TypeError) as e:
         warnings.warn(f"{TORCH_LIB_PATH} cannot be used, calls go through ctypes (6 to 8 us more of host time each); build it with "

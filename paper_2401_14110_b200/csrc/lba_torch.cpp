@@ -22,7 +22,8 @@
 
 namespace {
 
-PyObject* g_format_type = nullptr;  // formats.LbaFormat
+PyObject* g_format_type = nullptr;     // formats.LbaFormat
+PyObject* g_parameter_type = nullptr;  // torch.nn.Parameter: a tensor like any other here, as weights, scales and biases often are
 PyObject* g_field[5];               // its attribute names, interned
 
 struct NotRegular {};
@@ -69,7 +70,7 @@ lba_fmt as_format(PyObject* o) {
 
 // a contiguous tensor of `dtype` on the current device
 const at::Tensor& as_tensor(PyObject* o, c10::ScalarType dtype, int dim, int device) {
-  if (Py_TYPE(o) != (PyTypeObject*)THPVariableClass) not_regular();  // no subclass
+  if (Py_TYPE(o) != (PyTypeObject*)THPVariableClass && Py_TYPE(o) != (PyTypeObject*)g_parameter_type) not_regular();  // no other subclass
   const at::Tensor& t = THPVariable_Unpack(o);
   if (!t.defined() || !t.is_cuda() || t.get_device() != device || t.scalar_type() != dtype || !t.is_contiguous() ||
       (dim >= 0 && t.dim() != dim))
@@ -213,16 +214,21 @@ PyObject* conv2d(PyObject*, PyObject* const* a, Py_ssize_t n) {
   });
 }
 
-PyObject* init_module(PyObject*, PyObject* format_type) {
+PyObject* init_module(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  if (n != 2) {
+    PyErr_SetString(PyExc_TypeError, "init takes the format class and the parameter class");
+    return nullptr;
+  }
   static const char* const names[5] = {"man_bits", "exp_bits", "bias", "rounding", "flags"};
   for (int i = 0; i < 5; ++i)
     if (!g_field[i] && !(g_field[i] = PyUnicode_InternFromString(names[i]))) return nullptr;
-  Py_XSETREF(g_format_type, Py_NewRef(format_type));
+  Py_XSETREF(g_format_type, Py_NewRef(a[0]));
+  Py_XSETREF(g_parameter_type, Py_NewRef(a[1]));
   Py_RETURN_NONE;
 }
 
 PyMethodDef kMethods[] = {
-    {"init", init_module, METH_O, "the format class whose instances are read by attribute"},
+    {"init", (PyCFunction)(void (*)(void))init_module, METH_FASTCALL, "the format class whose instances are read by attribute, and the parameter class"},
     {"gemm", (PyCFunction)(void (*)(void))gemm, METH_FASTCALL, nullptr},
     {"gemm_batched", (PyCFunction)(void (*)(void))gemm_batched, METH_FASTCALL, nullptr},
     {"conv2d", (PyCFunction)(void (*)(void))conv2d, METH_FASTCALL, nullptr},

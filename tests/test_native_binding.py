@@ -113,6 +113,22 @@ def test_native_and_ctypes_paths_agree():
 
 
 @pytest.mark.gpu
+def test_parameters_are_regular_operands():
+    dev = "cuda:0"
+    a, b = synth.random_codes((21, 48), 1).to(dev), synth.random_codes((37, 48), 2).to(dev)
+    x, w = synth.random_codes((2, 9, 11, 16), 3).to(dev), synth.random_codes((37, 3, 2, 16), 4).to(dev)
+    one, sb, bias = torch.ones(1, device=dev), torch.rand(37, device=dev), torch.rand(37, device=dev)
+    par = lambda t: torch.nn.Parameter(t, requires_grad=t.is_floating_point())
+    for f, native, args in ((lba.lba_gemm, "gemm", (a, b, one, sb, bias, P, A12, CHK, 16)),
+                            (lba.lba_gemm_batched, "gemm_batched", (a[None], b, one, sb, bias, P, A12, SEQ, 16)),
+                            (lba.lba_conv2d, "conv2d", (x, w, one, sb, bias, (1, 1), (0, 0), P, A12, CHK, 16))):
+        want = f(*args)
+        got = getattr(lba._native, native)(*(par(t) if isinstance(t, torch.Tensor) else t for t in args), None, None)
+        assert type(got) is torch.Tensor and not got.requires_grad
+        assert torch.equal(got.view(torch.int32), want.view(torch.int32))
+
+
+@pytest.mark.gpu
 def test_what_was_refused_stays_refused():
     dev = "cuda:0"
     one = torch.ones(1, device=dev)
