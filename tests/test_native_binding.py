@@ -152,3 +152,30 @@ def test_what_was_refused_stays_refused():
         assert torch.equal(lba.lba_gemm(*args).view(torch.int32), want)
     x, w = a.view(1, 1, 8, 32), a.view(8, 1, 1, 32)
     assert torch.equal(lba.lba_conv2d(x, w, one, one, None, [1, 1], [0, 0], P, A12).view(8, 8).view(torch.int32), want)
+
+
+@pytest.mark.gpu
+def test_regular_calls_are_made_by_the_native_functions():
+    # called directly, for an entry point goes on through ctypes where they return None
+    dev = "cuda:0"
+    one, sb, bias = torch.ones(1, device=dev), torch.rand(37, device=dev), torch.rand(37, device=dev)
+    a, b = synth.random_codes((3, 21, 48), 1).to(dev), synth.random_codes((3, 37, 48), 2).to(dev)
+    x, w = synth.random_codes((2, 9, 11, 16), 3).to(dev), synth.random_codes((37, 3, 2, 16), 4).to(dev)
+    here, side = torch.cuda.current_stream(), torch.cuda.Stream()
+    lba.load_library()
+    native = lba._native
+    for order in (SEQ, CHK):
+        for pf, af in ((P, A12), (P.as_tuple(), A12.as_tuple())):
+            for f, direct, args in ((lba.lba_gemm, native.gemm, (a[0], b[0], one, sb, bias, pf, af, order, 16)),
+                                    (lba.lba_gemm_batched, native.gemm_batched, (a, b, one, sb, None, pf, af, order, 16)),
+                                    (lba.lba_gemm_batched, native.gemm_batched, (a, b[1], one, one, bias, pf, af, order, 16)),
+                                    (lba.lba_conv2d, native.conv2d, (x, w, one, sb, bias, (2, 1), (1, 0), pf, af, order, 16))):
+                want = f(*args, stream=here).view(torch.int32)
+                out = torch.empty_like(want).view(torch.float32)
+                assert direct(*args, out, None) is out
+                side.wait_stream(here)
+                with torch.cuda.stream(side):
+                    on_side = direct(*args, None, None)
+                side.synchronize()
+                for got in (out, direct(*args, None, None), on_side):
+                    assert type(got) is torch.Tensor and torch.equal(got.view(torch.int32), want)
