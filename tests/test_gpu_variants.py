@@ -321,3 +321,98 @@ def test_launches_of_small_problems_leave_their_successors_evenly_spread():
     finally:
         lba.set_tile_override(-1)
         gc.collect()
+
+
+@pytest.mark.parametrize("how", ["stream", "two streams", "graph"])
+def test_kernels_of_every_kind_keep_their_order(how):
+    # every ordered pair of kernels one behind the other: a call adds the tail of what the call before it or the one before that
+    # wrote (its bias) and writes over what the mask pass behind it still reads; the masks become operands through a PyTorch kernel
+    one = torch.ones(1, device=DEV)
+    codes = torch.empty(700 * 64, dtype=torch.uint8, device=DEV)
+    first = synth.random_codes((700 * 64,), 1).to(DEV)
+    w640, w64 = synth.random_codes((640, 64), 2).to(DEV), synth.random_codes((64, 64), 3).to(DEV)
+    wconv = synth.random_codes((64, 3, 3, 16), 4).to(DEV)
+    bufs = [torch.empty(700 * 640, device=DEV) for _ in range(3)]
+    mask1, mask2 = torch.empty(80, 2, 64, dtype=torch.int32, device=DEV), torch.empty(80, 1, 64, dtype=torch.int32, device=DEV)
+    floor, cut, near, generic = (code_domain_formats(7, 4), code_domain_formats(4, 4), code_domain_formats(7, 4, 1),
+                                 code_domain_formats(12, 5, 1))
+
+    def gemm(M, w, fmts, order, tile, chunk=16):
+        def run(bias, out):
+            lba.set_tile_override(tile)
+            lba.lba_gemm(codes[:M * 64].view(M, 64), w, one, one, bias(len(w)), *fmts, order, chunk, out=out(M, len(w)))
+        return run
+
+    def conv(bias, out):
+        lba.set_tile_override(-1)
+        lba.lba_conv2d(codes[:2 * 9 * 11 * 16].view(2, 9, 11, 16), wconv, one, one, bias(64), (1, 1), (1, 1), *floor, CHK, 16,
+                       out=out(2, 9, 11, 64))
+
+    def masks(ste, order):
+        def run(last, oldest):
+            lba.set_tile_override(-1)
+            lba.lba_gemm_ste_mask(last[:80 * 16].view(torch.uint8).view(80, 64), oldest[:64 * 16].view(torch.uint8).view(64, 64), *floor, order,
+                                  16, ste, 4.0, 2.0 ** -7, mask1, mask2 if order == CHK else None)
+        return run
+
+    def glue(last, oldest):
+        torch.bitwise_and(mask1.view(torch.uint8).view(-1)[:codes.numel()], 0x77, out=codes[:80 * 2 * 64 * 4])
+
+    forward = [gemm(33, w64, floor, SEQ, 10), gemm(33, w64, near, CHK, 6), gemm(65, w64, cut, CHK, 7), gemm(700, w640, floor, CHK, 2),
+               gemm(700, w640, cut, SEQ, 0), gemm(300, w640, floor, CHK, 5), gemm(130, w64, near, SEQ, 3), gemm(130, w64, generic, CHK, -1, 24),
+               conv]
+    others = [masks(lba.STE_OF, CHK), masks(lba.STE_OF, SEQ), masks(lba.STE_DIFF, CHK), masks(lba.STE_DIFF, SEQ), glue]
+    kinds = forward + others
+    steps = [k for f in kinds for g in kinds for k in (f, g)]
+    sides = [torch.cuda.Stream(), torch.cuda.Stream()] if how == "two streams" else None
+
+    def chain(sync):
+        lens, t = [64 * 64] * 3, 0
+        codes.copy_(first)
+        mask1.zero_()
+        mask2.zero_()
+        for b in bufs:
+            b.zero_()
+        for i, step in enumerate(steps):
+            if step in others:
+                step(bufs[t % 3], bufs[(t + 1) % 3])
+            else:
+                source = (t - i % 2) % 3
+
+                def out(*shape):
+                    lens[(t + 1) % 3] = int(np.prod(shape))
+                    return bufs[(t + 1) % 3][:lens[(t + 1) % 3]].view(shape)
+                step(lambda n: bufs[source][lens[source] - n:lens[source]], out)
+                t += 1
+            if sync:
+                torch.cuda.synchronize()
+            elif sides:
+                sides[1 - i % 2].wait_stream(torch.cuda.current_stream())
+                torch.cuda.set_stream(sides[1 - i % 2])
+        return [x.clone() for x in (*bufs, mask1, mask2, codes)]
+
+    def same(got):
+        return all(torch.equal(g.view(torch.uint8), w.view(torch.uint8)) for g, w in zip(got, want))
+
+    home = torch.cuda.current_stream()
+    try:
+        want = chain(True)
+        if how == "graph":
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                got = chain(False)
+            for _ in range(3):
+                graph.replay()
+                torch.cuda.synchronize()
+                assert same(got)
+            del graph
+        else:
+            for _ in range(3):
+                got = chain(False)
+                torch.cuda.set_stream(home)
+                torch.cuda.synchronize()
+                assert same(got)
+    finally:
+        torch.cuda.set_stream(home)
+        lba.set_tile_override(-1)
+        gc.collect()
