@@ -10,17 +10,7 @@ cudaError_t launch_tile(const Problem& p, cudaStream_t stream) {
   const dim3 grid((unsigned)((p.M + BM - 1) / BM), (unsigned)((p.N + BN - 1) / BN), 1);
   auto kernel = lba_contract_packed_kernel<BM, BN, TM, TN, PQ, 0, ORD, LD, 1>;
   constexpr size_t smem = packed_ste_smem_bytes<BM, BN, TM, TN>();
-  if (smem <= 48 * 1024) return launch_after(kernel, grid, (BM / TM) * (BN / TN), smem, stream, p);
-  static bool done[64] = {};  // opt in to large dynamic shared memory, once per device and kernel
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  if (!done[dev]) {
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    done[dev] = true;
-  }
+  static_assert(smem <= 48 * 1024, "no opt-in needed");
   return launch_after(kernel, grid, (BM / TM) * (BN / TN), smem, stream, p);
 }
 

@@ -298,10 +298,10 @@ __device__ __forceinline__ u64 mul2_rz_ftz(u64 a, u64 b) {
 // Floor cut of a pair of products to M bits on the FP32 pipe: k1 = 1 + 2^s, k2 = -2^s, r = rz(v * k1) = 2^s v + v cut to v's
 // grid, minus 2^s v exactly.  Only for values of at most 10 significant bits (s > 10): v k1 must not reach the next binade.
 __device__ __forceinline__ u64 floor2_fp(u64 v, u64 k1, u64 k2) { return fma2_rn(v, k2, mul2_rz_ftz(v, k1)); }
-// The same without the product itself: ak1 = a k1 and ak2 = a k2 are exact (5 significant bits times 1 + 2^s, s <= 19), so
-// r = rz(b ak1) is the r above and b ak2 + r the cut.  `.ftz` flushes the cut exactly where it would have flushed the product: R_UF
-// lies on the cut's grid, so a value is below it if and only if its cut is.  An r that is flushed itself belongs to a product below
-// 2^-s R_UF, whose b ak2 is flushed as well.
+// The same without the product itself: ak1 = a k1 and ak2 = a k2 are exact (4 significant bits times 1 + 2^s, s <= 20, for E4M3, 5
+// and s <= 19 for M4E3), so r = rz(b ak1) is the r above and b ak2 + r the cut.  `.ftz` flushes the cut exactly where it would have
+// flushed the product: R_UF lies on the cut's grid, so a value is below it if and only if its cut is.  An r that is flushed itself
+// belongs to a product below 2^-s R_UF, whose b ak2 is flushed as well.
 // Two FP32 instructions per pair where mul and floor2_fp take three and mul and two masks as many plus two logic ones; the
 // 64x64 tile runs 8192 x 8192 x 1024 at 4.29 clocks per warp-MAC (M4E3 operands, M7E4, chunk 16; 4.44 with every second pair on
 // the logic pipe), 4.13 (M5E5, sequential; 4.21).
