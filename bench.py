@@ -141,7 +141,23 @@ def peak_gmacs(mode, chunk, sm_count, mhz):
 # DRAM bytes (read + write) of ONE launch of the dominant kernel, from an ncu capture summarised under profiles/:
 # (workload, kernel description) -> (bytes, what was captured, executed instructions per emulated MAC).  An entry is taken out
 # when the kernel that it names changes.
-NCU = {}
+_K_FLOOR = "tile=128x128x16 micro=8x8 q=floor_fast pq=none kernel=packed order=chunk16 load=gemm_vec"
+_CAP = "profiles/packed_floor_kernel_gemm_8192x8192x1024_chunk.txt"
+NCU = {
+    # the headline launch is too long for a capture of many passes (45 ms): the K = 1024 case of the same kernel was
+    # captured; its reads grow in proportion to K (x 8), its writes (the output) do not grow with K
+    ("single_lba_gemm_8192x8192x8192_m7e4_chunk16", _K_FLOOR):
+        (8 * 17770752 + 211876608, "scaled from the 8192x8192x1024 capture (" + _CAP + "): 8 x 17.8 MB read + 211.9 MB written; "
+         "algorithmic 128 MB + 256 MB (part of the output is still in L2 when the kernel ends)", 2.277),
+    ("single_lba_gemm_8192x8192x1024_m7e4_chunk16", _K_FLOOR):
+        (17770752 + 211876608, "17.8 MB read + 211.9 MB written (" + _CAP + "); algorithmic 272 MB", 2.277),
+    ("single_lba_gemm_8192x8192x1024_m7e4_sequential", "tile=128x128x16 micro=8x8 q=floor_fast pq=none kernel=packed order=seq load=gemm_vec"):
+        (17844480 + 211308288, "17.8 MB read + 211.3 MB written (profiles/packed_floor_kernel_gemm_8192x8192x1024_seq.txt)", 2.228),
+    ("single_lba_gemm_8192x8192x1024_m7e4_rne_chunk16", "tile=64x64x16 micro=4x8 q=rne_full pq=none kernel=packed order=chunk16 load=gemm_vec"):
+        (18670336 + 213114880, "18.7 MB read + 213.1 MB written (profiles/packed_nearest_even_kernel_gemm_8192x8192x1024_chunk.txt)", 2.947),
+    ("single_lba_gemm_8192x8192x1024_m8e6_chunk16", "tile=128x128x16 micro=8x8 q=floor_fast pq=fused kernel=packed order=chunk16 load=gemm_vec"):
+        (17737984 + 212646912, "17.7 MB read + 212.6 MB written (profiles/packed_floor_kernel_fused_gemm_8192x8192x1024_chunk.txt)", 1.804),
+}
 
 
 def parse_args(argv=None):
