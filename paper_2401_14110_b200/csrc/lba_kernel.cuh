@@ -1052,9 +1052,9 @@ __host__ __device__ constexpr int packed_tmem_cols() {
 // half (128x64) of the CTAs: nearest-even M7E4 on the 128x64 tile, GEMM 4096 x 4096 x 512 1146 to 983 us, ResNet stem
 // 729 to 598 us.  So are, under floor rounding, the loaders of unaligned rows and of any convolution, whose loads in flight would
 // otherwise cost fifty registers and half the resident CTAs, and the mask passes.  In longer chunks only the byte-wise loader with
-// a floor cut of the product is (181 registers without; the FP32-pipe cut is a longer chain, which one CTA per SM does not hide):
-// 25088 x 64 x 147 in chunks of 32, M5E5: 6.5 % slower than with masks alone, 77 us against 59 with the bound (401408 rows 807, 682;
-// 16384 x 64 x 216, one CTA per SM in any case, 53.1, 54.1 and 54.7 with masks alone).  The other modes would lose up to 7 % on that last shape.
+// a floor cut of the product is.  Chunks of 32, with and without the bound, us: 25088 x 64 x 147 cut_product 53.9 and 60.4, a cut of
+// its own (M2) 56.7 and 71.7, with saturation 79.9 and 95.2; 401408 rows 635 and 698, 643 and 758, 853 and 941; 16384 x 64 x 216, one CTA per SM
+// in any case, 50.7 and 47.7, 50.9 and 49.4, 62.7 and 61.6.  The other modes would lose up to 7 % on that last shape.
 // PQ: what Q_prod has to do beyond the flush (the host proves which cases are reachable): nothing, cut the mantissa (M_prod < 7;
 // under floor rounding where A's scales can carry the cut, M_prod >= 3 or 4), or cut and saturate (448^2 >= R_OF_prod).
 // PQ_CUT_ANY (floor only): cut to fewer bits than A's scales can carry, as in PQ_MASK_SAT but without the clamp.  4096^3, M2E5 on
