@@ -385,7 +385,9 @@ int sm_count() {
 // their SM run faster).  One row per kernel: rows shared between kernels had put the generic nearest-even kernel (M12E5) on the
 // 128x128 tile, 3.72 ms where 32x32 takes 2.08 (2048 x 1024 x 1024, sequential) and 13.5 ms where 128x64 takes 7.4
 // (4096 x 4096 x 512, chunks).  profiles/tile_times.txt holds the times that the constants are fitted to and what the choice
-// loses on them.
+// loses on them.  The constants make the fastest tile come out first; kernels that share a row (a fused product, M4E3 bytes without a cut,
+// the rounding of a nearest-even product) differ by up to a half, and a slab that is clamped, which no row can know of, takes up
+// to 1.7 times as long (weights scaled per channel), so the rows are fitted to operands scaled either way at once.
 struct TileCost { double L, b, base, w; };
 enum { COST_PAIR = 4, COST_SMALL = 5, COST_TILES = 7 };
 enum CostRow { ROW_SEQ = 0, ROW_CHUNK16 = 1, ROW_CUT_SEQ = 2, ROW_CUT_CHUNK16 = 3, ROW_RNE_SEQ = 4, ROW_RNE_CHUNK16 = 5, ROW_BF16_CHUNK16 = 6,
@@ -393,12 +395,12 @@ enum CostRow { ROW_SEQ = 0, ROW_CHUNK16 = 1, ROW_CUT_SEQ = 2, ROW_CUT_CHUNK16 = 
                ROW_WIDE_SEQ = 14, ROW_WIDE_LONG = 15, ROW_WIDE_ANY = 16, ROW_COUNT = 17 };
 const TileCost kCost[ROW_COUNT][COST_TILES] = {
     // 128x128, 128x64, 64x64, 32x32, pair, 16x16 chain (sequential) or split, 32x32 split
-    {{3.14, 3.23, 3.87, 0.705}, {0.598, 3.77, 3.51, 0.68}, {0.865, 0.856, 1.45, 0.777}, {0.595, 0.228, 5.92, 0.816}, {0, 0, 0, 0}, {0.252, 0.196, 3.02, 0.821}, {0, 0, 0, 0}},  // floor, sequential
+    {{2.19, 3.23, 7.99, 1}, {0.706, 1.95, 2.61, 0.69}, {1.18, 0.842, 2.25, 1}, {0.777, 0.236, 2.43, 1}, {0, 0, 0, 0}, {0.235, 0.146, 1.87, 1}, {0, 0, 0, 0}},  // floor, sequential
     {{2.4, 3.66, 5.8, 0.84}, {1.14, 1.878, 3.5, 0.96}, {0.94, 0.931, 4, 1}, {0.73, 0.28, 3.1, 1}, {1.8, 1.079, 3.4, 1}, {0, 1.863, 2.4, 0.57}, {1.49, 2.437, 2.4, 0.85}},  // floor, chunks of 16
-    {{3, 5.536, 6.06, 0.854}, {1.58, 3.147, 4.8, 0.881}, {1.07, 1.121, 4.73, 0.976}, {0.649, 0.32, 3.4, 0.814}, {0, 0, 0, 0}, {0.264, 0.176, 2.25, 0.954}, {0, 0, 0, 0}},  // floor with product cut, sequential
-    {{2.74, 5.811, 7.86, 0.941}, {1.28, 2.804, 4.99, 0.69}, {0.955, 1.147, 5.83, 0.985}, {0.446, 0.3284, 4.22, 0.69}, {1.82, 1.495, 6.12, 0.916}, {0.000185, 2.325, 1.77, 0.883}, {2.28, 3.672, 2.38, 0.982}},  // floor with product cut, chunks of 16
-    {{1.9, 4.724, 4.7, 0.98}, {1.49, 2.478, 3.2, 1}, {1.2, 1.277, 2.9, 1}, {0.95, 0.354, 2.1, 1}, {0, 0, 0, 0}, {0.279, 0.165, 2.18, 0.94}, {0, 0, 0, 0}},  // nearest-even, sequential
-    {{0.08, 5.151, 4.6, 1}, {0.01, 2.783, 3.2, 1}, {1.25, 1.285, 3.5, 1}, {0.97, 0.365, 3.5, 1}, {0, 0, 0, 0}, {0.01, 1.993, 2.6, 0.68}, {1.8, 2.967, 2.7, 0.9}},  // nearest-even, chunks of 16
+    {{0, 5.15, 4.63, 0.698}, {0, 2.51, 1.5, 1}, {1.14, 1.16, 4.03, 1}, {0.788, 0.333, 1.74, 1}, {0, 0, 0, 0}, {0.245, 0.162, 2.16, 0.975}, {0, 0, 0, 0}},  // floor with product cut, sequential
+    {{0, 5.35, 5.06, 0.689}, {1.09, 2.53, 1.81, 0.987}, {1.26, 1.19, 3.76, 0.917}, {0.682, 0.338, 2.35, 1}, {2.21, 1.5, 3.27, 0.691}, {0, 2.53, 2.76, 0.575}, {1.86, 4.29, 1.99, 1}},  // floor with product cut, chunks of 16
+    {{0, 7.12, 3.33, 0.441}, {0, 3.44, 1.5, 0.579}, {1.86, 1.49, 3.14, 1}, {1.11, 0.395, 1.5, 1}, {0, 0, 0, 0}, {0.281, 0.151, 2.54, 1}, {0, 0, 0, 0}},  // nearest-even, sequential
+    {{0, 6.19, 3.68, 0.506}, {0, 2.85, 8, 0.969}, {1.85, 1.31, 1.65, 0.842}, {2.03, 0.348, 1.52, 0.999}, {0, 0, 0, 0}, {0, 1.98, 2.77, 0.53}, {1.87, 3.11, 1.82, 1}},  // nearest-even, chunks of 16
     {{0, 4.75, 4.2, 1}, {0.05, 2.575, 3.3, 1}, {1.29, 1.14, 3.9, 1}, {0.95, 0.323, 3, 1}, {0, 0, 0, 0}, {0, 1.972, 2.6, 0.5}, {1.98, 2.766, 2.5, 0.92}},  // nearest-even through bfloat16, chunks of 16
     {{0, 3.712, 7.36, 0.948}, {0.969, 2.205, 3.74, 0.761}, {0.871, 0.8876, 3.47, 0.915}, {0.599, 0.2523, 2.61, 0.427}},  // floor, longer chunks
     {{0, 5.16, 4.99, 0.967}, {1.71, 2.6, 4.34, 1}, {1.65, 1.28, 4.82, 1}, {0.89, 0.361, 4.97, 0.834}},  // floor with product cut, longer chunks

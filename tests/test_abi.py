@@ -9,7 +9,7 @@ import pytest
 import torch
 
 from paper_2401_14110_b200 import binding as lba
-from paper_2401_14110_b200 import FLAG_INPUT_M4E3, LbaFormat, code_domain_formats, ORDER_CHUNKED as CHK, ORDER_SEQUENTIAL as SEQ
+from paper_2401_14110_b200 import FLAG_INPUT_M4E3, LbaFormat, code_domain_formats, m4e3_input_formats, ORDER_CHUNKED as CHK, ORDER_SEQUENTIAL as SEQ
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
@@ -184,6 +184,30 @@ FASTEST = [   # formats, order, chunk, shape, the tile that measured fastest (us
 def test_tile_choice_knows_each_kernel(fmts, order, chunk, shape, tile):
     plan = lba.describe_plan(*shape, *fmts, order, chunk)
     assert plan.startswith(f"tile={tile}x16 micro") and "by=" not in plan
+
+
+M4E3 = m4e3_input_formats(7, 4)
+RUNS = [   # formats, order, shape, convolution, what runs (us; with weights scaled per channel where two figures stand; the next one)
+    (code_domain_formats(7, 4), SEQ, (128, 1000, 512), False, "chain16x16"),          # 20.5, 20.8; 32x32 22.6, 39.4
+    (code_domain_formats(7, 4), SEQ, (256, 512, 4608), True, "chain16x16"),           # 171; 32x32 189
+    (code_domain_formats(7, 4), SEQ, (49, 2048, 512), True, "chain16x16"),            # 21.6; 32x32 26.0
+    (code_domain_formats(7, 4), SEQ, (16, 8192, 4096), False, "chain16x16"),          # 152, 153; 32x32 173, 249
+    (code_domain_formats(7, 4), SEQ, (379, 3296, 144), False, "tile=32x32"),          # 22.7, 27.2; 64x64 25.7, 34.1
+    (code_domain_formats(7, 4), SEQ, (3136, 128, 64), True, "tile=32x32"),            # 6.5; 64x64 8.1
+    (code_domain_formats(4, 4), SEQ, (256, 512, 2304), True, "chain16x16"),           # 100; 32x32 118
+    (M4E3, SEQ, (128, 1000, 512), False, "chain16x16"),                               # 24.1; 32x32 28.8
+    (code_domain_formats(4, 4), CHK, (1931, 96, 2016), False, "split16x16"),          # 90; 32x32 112
+    (M4E3, CHK, (1931, 96, 2016), False, "split16x16"),                               # 94; 32x32 115
+    (code_domain_formats(10, 5, 1), SEQ, (64, 4096, 2048), False, "chain16x16"),      # 141, 143; 32x32 156, 165
+    (code_domain_formats(10, 5, 1), SEQ, (2048, 1024, 1024), False, "tile=32x32"),    # 310, 322; 128x64 343, 357; 128x128 358, 377
+    (code_domain_formats(10, 5, 1), SEQ, (4096, 4096, 4096), False, "tile=64x64"),    # 8950, 9130; 128x128 10200, 10540
+]
+
+
+@pytest.mark.parametrize("fmts,order,shape,conv,what", RUNS, ids=lambda v: str(v) if isinstance(v, (str, int)) else "")
+def test_tile_choice_by_the_times_of_the_present_kernels(fmts, order, shape, conv, what):
+    plan = lba.describe_plan(*shape, *fmts, order, 16, is_conv=conv, vec_ok=shape[2] % 16 == 0)
+    assert (plan.partition(" by=")[2] or plan).startswith(what)
 
 
 @pytest.mark.parametrize("fmts", [code_domain_formats(7, 4), code_domain_formats(10, 6), code_domain_formats(4, 4), code_domain_formats(10, 5, 1)],
