@@ -1916,8 +1916,7 @@ constexpr size_t packed_ste_smem_bytes() {
 
 // Launch entry of one (quantiser mode, order mode) family; defined once per translation unit.
 // tile: 0 = 128x128 (8x8 per thread, 256 threads), 1 = 128x64 (4x8, 256 threads), 2 = 64x64 (4x8, 128 threads),
-// 3 = 32x32 (4x4, 64 threads).  Measured and dropped (with A stored twice): 8x8 in CTAs of
-// 64 or 128 threads, 4x8 in 32x64, 32x128, 64x128, 128x128, 64x256 tiles, a one-warp 32x32 tile.
+// 3 = 32x32 (4x4, 64 threads).
 struct TileInfo { int bm, bn, tm, tn; };
 constexpr int TILE_COUNT = 4;
 constexpr int TILE_PAIR = 5;  // 64x64 tile shared by a cluster of two CTAs (chunk-16 order, floor rounding)
