@@ -87,8 +87,6 @@ struct Problem {
   int in_m4e3;         // operands are bytes of the paper's M4E3 W/A format (Sec. 3.1) instead of OCP E4M3
   float acc_k1, acc_k2;    // nearest-even cut of a sum: v k2 + rn(v k1) (see rne2_fp)
   float prod_k1, prod_k2;  // the same for a product; under floor rounding v k2 + rz(v k1) (see floor2_fp)
-  // floor cut of the product that A's scales can carry (0: they cannot; see cut_product): the scales times k2, and k1 / k2
-  float cut_a, cut_a0, cut_ratio;
   // clamp elision: a slab or fold runs without the magnitude clamp while (bound + growth) * factor < clamp_lim.
   // Floor never raises a magnitude: factors 1, limit just under 1 (of 2^(e_max+1)).  Nearest-even can raise one by
   // half a grid step per rounding: slab_factor bounds sixteen such steps (and the product's own rounding),
@@ -110,6 +108,10 @@ struct Problem {
   int fx_lo_a, fx_hi_a, fx_sh_a, fx_wrap_a;  // accumulator
   int fx_dl, fx_dr;            // product units -> accumulator units: << dl then >> dr
   float fx_unit;               // 2^-b_acc
+  // floor cut of the product that A's scales can carry (0: they cannot; see cut_product): the scales times k2, and k1 / k2.  Behind
+  // all other fields: further up they move the offsets that the scalar kernels read, whose register allocation then changes
+  // (difference masks of 84 x 1440 x 224 sequential 48.4 us, 47.2 like this; nearest-even M12E5 of 3000 x 1500 x 1008 4237 and 4184)
+  float cut_a, cut_a0, cut_ratio;
 };
 
 // ------------------------------------------------------------------ scalar building blocks
